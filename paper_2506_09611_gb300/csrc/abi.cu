@@ -88,7 +88,6 @@ struct Walker {
     // decisions of window w + 1), and the corrected snapshots of the next window's block
     int* wm[2] = {nullptr, nullptr};
     int* widx[2] = {nullptr, nullptr};
-    double* wdtot[2] = {nullptr, nullptr};
     void* Wm[2] = {nullptr, nullptr};
     void* Wx[2] = {nullptr, nullptr};
     void* X[2] = {nullptr, nullptr};
@@ -875,7 +874,6 @@ int afqmc_init_walkers(afqmc_ctx* ctx, int n_walkers, const int* L, const int* n
         for (int q = 0; q < 2; ++q) {
             CK(dalloc(A, &w->wm[q], (size_t)nwk * sizeof(int)));
             CK(dalloc(A, &w->widx[q], (size_t)nwk * NW * sizeof(int)));
-            CK(dalloc(A, &w->wdtot[q], (size_t)nwk * 2 * NW * 8));
             CK(dalloc(A, (char**)&w->Wm[q], (size_t)nwk * 2 * NW * NW * es));
             CK(dalloc(A, (char**)&w->Wx[q], (size_t)nwk * 2 * NW * NW * es));
             CK(dalloc(A, (char**)&w->X[q], (size_t)nwk * 2 * N * NW * es));
@@ -1235,7 +1233,6 @@ static int sweep_impl(afqmc_ctx* ctx, int gi, int ell, int dir, int mode, int k,
         for (int q = 0; q < 2; ++q) {
             wb[q].m = w->wm[q];
             wb[q].idx = w->widx[q];
-            wb[q].dtot = w->wdtot[q];
             wb[q].Wm = w->Wm[q];
             wb[q].Wx = w->Wx[q];
             wb[q].X = w->X[q];
@@ -1366,7 +1363,6 @@ static int tform_windows(afqmc_ctx* ctx, Walker* w, cudaStream_t st, int8_t* xl,
     WindowBufs wb;
     wb.m = w->wm[0];
     wb.idx = w->widx[0];
-    wb.dtot = w->wdtot[0];
     wb.Wm = w->Wm[0];
     wb.Wx = w->Wx[0];
     wb.X = w->X[0];

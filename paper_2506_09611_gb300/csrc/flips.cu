@@ -37,7 +37,6 @@ static WindowBufs flips_layout(unsigned char* scratch, int N) {
     wb.X = scratch + off;
     off += al(2 * (size_t)N * NW * sizeof(T));
     wb.Y = scratch + off;
-    wb.dtot = nullptr;
     return wb;
 }
 

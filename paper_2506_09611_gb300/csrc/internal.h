@@ -245,7 +245,6 @@ cudaError_t launch_local(cudaStream_t st, T* Gu, T* Gd, int8_t* xl, const double
 struct WindowBufs {    // device scratch of the window chain + flush
     int* m;            // accepted count of the window
     int* idx;          // accepted site indices (global), capacity NW
-    double* dtot;      // per spin, 2 x NW: sweep: recursion factor -Delta/r; apply_flips: unused
     void* Wm;          // per spin NW x NW (T): sweep: frozen block coefficients; apply_flips: W
     void* Wx;          // per spin NW x NW (T): sweep: the window's update matrix W
     void* X;           // per spin N x NW column panel (T)

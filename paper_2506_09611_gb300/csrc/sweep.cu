@@ -342,7 +342,6 @@ __device__ __forceinline__ WindowBufs wb_walker(WindowBufs wb, int j, int N) {
     constexpr int NW = WinCap<T>::NW;
     wb.m += j;
     wb.idx += (size_t)j * NW;
-    wb.dtot += (size_t)j * 2 * NW;
     wb.Wm = (T*)wb.Wm + (size_t)j * 2 * NW * NW;
     if (wb.Wx) wb.Wx = (T*)wb.Wx + (size_t)j * 2 * NW * NW;
     wb.X = (T*)wb.X + (size_t)j * 2 * N * NW;
@@ -350,14 +349,20 @@ __device__ __forceinline__ WindowBufs wb_walker(WindowBufs wb, int j, int N) {
     return wb;
 }
 
+// Sites per sub-block of the window (window_sub_sites): what one warp keeps in registers for both
+// spins, 16 FP32 or 4 FP64 elements a lane.
+template <typename T> struct WinSub { static constexpr int B = sizeof(T) == 4 ? 16 : 8; };
+
 template <typename T>
 static size_t window_smem(int n) {
+    constexpr size_t B = WinSub<T>::B;
     size_t P = (size_t)n + 1;
-    size_t g = 2 * (size_t)n * P * sizeof(T);  // Gs[2][n][n+1]
+    size_t g = 2 * (size_t)n * P * sizeof(T);            // Gs[2][n][n+1]
+    size_t pan = 4 * B * (B + (size_t)n) * sizeof(T);    // sub-block coefficients and panels
     size_t s1 = 2 * (size_t)NBMAX * (NBMAX + 1) * sizeof(T);
     size_t vec = 4 * (size_t)n * sizeof(T) + 2 * (size_t)NBMAX * sizeof(T);  // staging vectors
-    size_t misc = (size_t)n * (sizeof(int) + 2 * sizeof(double) + 1) + 8 * (size_t)NBMAX * sizeof(double) + 256;
-    return g + s1 + vec + misc;
+    size_t misc = (size_t)n * (sizeof(int) + 1) + 8 * (size_t)NBMAX * sizeof(double) + 256;
+    return g + pan + s1 + vec + misc;
 }
 
 // G_s[r][c] += f_s * G_s[r][a] * G_s[a][c] for r, c in (a, n), both spins; 32 x 32 thread tiles.
@@ -374,56 +379,54 @@ __device__ __forceinline__ void trailing_update(T* Gs, int n, int P, int a, T f0
     }
 }
 
-// W = -F U1^{-1} L1^{-1} of the window from the frozen coefficients in the block (see the window
-// kernel's tail); written to Wx[s][k][j] (pitch NW).  32 warps: spin = warp / 16, columns
-// (warp % 16) * WCPW + c; lane l holds rows l + 32 r, r < RPL (RPL >= ceil(m / 32)).  The
-// coefficient of the next step is fetched while the current one is applied, and the forward
-// pass of a warp starts at its first column (identity columns are zero above the diagonal).
-template <typename T, int RPL>
-__device__ __forceinline__ void window_w_rpl(const T* Gs, int n, int P, const int* idx, const T (*fk)[WinCap<T>::NW],
-                                             int m, T* Wx, int lane, int w) {
-    constexpr int NW = WinCap<T>::NW, WCPW = NW / 16;
-    const int s = w >> 4, j0 = (w & 15) * WCPW;
+// W = -F U1^{-1} L1^{-1} of the window (see the window kernel's tail); written to Wx[s][k][j] (pitch
+// NW).  Cc[s][k][k'] (pitch P, spin stride n P) holds C[k][k'] f_k'.  32 warps: spin = warp / 16,
+// columns (warp % 16) WC + c; lane l holds rows l + 32 r, r < RPL (RPL >= ceil(m / 32)).  WC is the
+// least count that covers m columns with 16 warps, so all of them work; the next step's coefficient
+// is fetched while the current one is applied, and the forward pass of a warp starts at its first
+// column (identity columns are zero above the diagonal).
+template <typename T, int RPL, int WC>
+__device__ __forceinline__ void window_w_rpl(const T* Cc, int n, int P, const T (*fk)[WinCap<T>::NW], int m, T* Wx,
+                                             int lane, int w) {
+    constexpr int NW = WinCap<T>::NW;
+    const int s = w >> 4, j0 = (w & 15) * WC;
     if (j0 >= m) return;
-    const T* Gb = Gs + (size_t)s * n * P;
-    const T* fks = fk[s];
-    int ik[RPL];
-    T y[RPL][WCPW];
+    const T* Cb = Cc + (size_t)s * n * P;
+    T y[RPL][WC];
 #pragma unroll
-    for (int r = 0; r < RPL; ++r) {
-        const int k = lane + 32 * r;
-        ik[r] = (k < m) ? idx[k] : 0;
+    for (int r = 0; r < RPL; ++r)
 #pragma unroll
-        for (int c = 0; c < WCPW; ++c) y[r][c] = (k == j0 + c) ? T(1) : T(0);
-    }
-    // coefficient cf[r] = C[k][kp] f_kp of this lane's rows for step kp
-    auto coef = [&](int kp, T* cf) {
-        const int ikp = idx[kp];
-        const T f = fks[kp];
+        for (int c = 0; c < WC; ++c) y[r][c] = (lane + 32 * r == j0 + c) ? T(1) : T(0);
+    auto coef = [&](int kp, T* cf) {  // C[k][kp] f_kp of this lane's rows
 #pragma unroll
-        for (int r = 0; r < RPL; ++r) cf[r] = Gb[ik[r] * P + ikp] * f;
+        for (int r = 0; r < RPL; ++r) {
+            const int k = lane + 32 * r;
+            cf[r] = k < m ? Cb[k * P + kp] : T(0);
+        }
     };
-    T cf[RPL], cfn[RPL];
-    // forward: rows k > kp
-    if (j0 + 1 < m) coef(j0, cf);
-    for (int kp = j0; kp + 1 < m; ++kp) {
-        if (kp + 2 < m) coef(kp + 1, cfn);
+    auto bcast = [&](int kp, T* v) {  // row kp of y from the lane that holds it
         const int ro = kp >> 5, lo = kp & 31;
-        T v[WCPW];
 #pragma unroll
-        for (int c = 0; c < WCPW; ++c) {
+        for (int c = 0; c < WC; ++c) {
             T src = y[0][c];
 #pragma unroll
             for (int r = 1; r < RPL; ++r)
                 if (ro == r) src = y[r][c];
             v[c] = __shfl_sync(0xffffffffu, src, lo);
         }
+    };
+    T cf[RPL], cfn[RPL], v[WC];
+    // forward: rows k > kp
+    if (j0 + 1 < m) coef(j0, cf);
+    for (int kp = j0; kp + 1 < m; ++kp) {
+        if (kp + 2 < m) coef(kp + 1, cfn);
+        bcast(kp, v);
 #pragma unroll
         for (int r = 0; r < RPL; ++r) {
             const int k = lane + 32 * r;
             if (k > kp && k < m) {
 #pragma unroll
-                for (int c = 0; c < WCPW; ++c) y[r][c] -= cf[r] * v[c];
+                for (int c = 0; c < WC; ++c) y[r][c] -= cf[r] * v[c];
             }
         }
 #pragma unroll
@@ -433,22 +436,13 @@ __device__ __forceinline__ void window_w_rpl(const T* Gs, int n, int P, const in
     if (m >= 2) coef(m - 1, cf);
     for (int kp = m - 1; kp >= 1; --kp) {
         if (kp >= 2) coef(kp - 1, cfn);
-        const int ro = kp >> 5, lo = kp & 31;
-        T v[WCPW];
-#pragma unroll
-        for (int c = 0; c < WCPW; ++c) {
-            T src = y[0][c];
-#pragma unroll
-            for (int r = 1; r < RPL; ++r)
-                if (ro == r) src = y[r][c];
-            v[c] = __shfl_sync(0xffffffffu, src, lo);
-        }
+        bcast(kp, v);
 #pragma unroll
         for (int r = 0; r < RPL; ++r) {
             const int k = lane + 32 * r;
             if (k < kp) {
 #pragma unroll
-                for (int c = 0; c < WCPW; ++c) y[r][c] -= cf[r] * v[c];
+                for (int c = 0; c < WC; ++c) y[r][c] -= cf[r] * v[c];
             }
         }
 #pragma unroll
@@ -459,24 +453,260 @@ __device__ __forceinline__ void window_w_rpl(const T* Gs, int n, int P, const in
     for (int r = 0; r < RPL; ++r) {
         const int k = lane + 32 * r;
         if (k < m) {
-            const T fkk = -fks[k];
+            const T fkk = -fk[s][k];
 #pragma unroll
-            for (int c = 0; c < WCPW; ++c)
+            for (int c = 0; c < WC; ++c)
                 if (j0 + c < m) Wd[k * NW + j0 + c] = fkk * y[r][c];
         }
     }
 }
 
-template <typename T>
-__device__ __forceinline__ void window_w(const T* Gs, int n, int P, const int* idx, const T (*fk)[WinCap<T>::NW],
-                                         int m, T* Wx, int tid) {
-    constexpr int NW = WinCap<T>::NW;
+// Cc[s][k][k'] = C[k][k'] f_k' in place over the block: every element of the accepted rows and columns
+// is read (RU x CU registers a thread; warps over rows, lanes over columns) before any is written.  The
+// block itself is not needed any more.
+template <typename T, int RU, int CU>
+__device__ __forceinline__ void window_compact(T* Gs, int n, int P, const int* idx, const T (*fk)[WinCap<T>::NW],
+                                               int m, int tid) {
     const int lane = tid & 31, w = tid >> 5;
-    if (w >= 32) return;
-    if (m <= 32) window_w_rpl<T, 1>(Gs, n, P, idx, fk, m, Wx, lane, w);
-    else if (m <= 64) window_w_rpl<T, 2>(Gs, n, P, idx, fk, m, Wx, lane, w);
-    else if (NW > 64 && m <= 96) window_w_rpl<T, (NW > 64 ? 3 : 2)>(Gs, n, P, idx, fk, m, Wx, lane, w);
-    else window_w_rpl<T, NW / 32>(Gs, n, P, idx, fk, m, Wx, lane, w);
+    T v[RU][CU];
+#pragma unroll
+    for (int a = 0; a < RU; ++a) {
+        const int row = w + 32 * a, s = row >= m ? 1 : 0, k = row - s * m;
+#pragma unroll
+        for (int c = 0; c < CU; ++c) {
+            const int kp = lane + 32 * c;
+            if (k < m && kp < m) v[a][c] = Gs[(s * n + idx[k]) * P + idx[kp]] * fk[s][kp];
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int a = 0; a < RU; ++a) {
+        const int row = w + 32 * a, s = row >= m ? 1 : 0, k = row - s * m;
+#pragma unroll
+        for (int c = 0; c < CU; ++c) {
+            const int kp = lane + 32 * c;
+            if (k < m && kp < m) Gs[(s * n + k) * P + kp] = v[a][c];
+        }
+    }
+    __syncthreads();
+}
+
+template <typename T>
+__device__ __forceinline__ void window_w(T* Gs, int n, int P, const int* idx, const T (*fk)[WinCap<T>::NW], int m,
+                                         T* Wx, int tid) {
+    constexpr bool BIG = WinCap<T>::NW > 64;
+    const int lane = tid & 31, w = tid >> 5;
+    if (m <= 64) window_compact<T, 4, 2>(Gs, n, P, idx, fk, m, tid);
+    else window_compact<T, WinCap<T>::NW / 16, WinCap<T>::NW / 32>(Gs, n, P, idx, fk, m, tid);
+    if (m <= 16) window_w_rpl<T, 1, 1>(Gs, n, P, fk, m, Wx, lane, w);
+    else if (m <= 32) window_w_rpl<T, 1, 2>(Gs, n, P, fk, m, Wx, lane, w);
+    else if (m <= 48) window_w_rpl<T, 2, 3>(Gs, n, P, fk, m, Wx, lane, w);
+    else if (m <= 64) window_w_rpl<T, 2, 4>(Gs, n, P, fk, m, Wx, lane, w);
+    else if (BIG && m <= 96) window_w_rpl<T, BIG ? 3 : 2, BIG ? 6 : 4>(Gs, n, P, fk, m, Wx, lane, w);
+    else window_w_rpl<T, BIG ? 4 : 2, BIG ? 8 : 4>(Gs, n, P, fk, m, Wx, lane, w);
+}
+
+// What warp 0 carries through a window's decisions (the same in every lane).
+template <typename T>
+struct WinScan {
+    int m = 0;        // accepts so far
+    int nneg = 0;     // accepted negative ratios (sign parity)
+    T maxr = T(0);    // largest |R| of an accept
+    bool alive = true;  // constrained path: the walker has not been removed
+    bool bad = false;   // a non-finite ratio was met
+    int done = 0;       // sites decided
+};
+
+// The decisions of the sites [b0, b0 + nbk) of the window, one warp for both spins: lane
+// 16 s + r CG + cg holds row r, columns j CG + cg of spin s's sub-block in registers (CG = 16 / B), so
+// a site costs its ratio (one shuffle for the diagonal, one to pair the spins) and an accept B shuffles
+// of its row and as many multiply-adds, with no barrier.  Every lane takes the decision redundantly.
+// An accept a updates the rows and columns after a only, with the products
+// G[r][c] += (Delta/r G[r][a]) G[a][c] (f = -Delta/r) in accept order; row a and column a keep their values of that moment (the frozen coefficients).
+//   Metropolis (AFQMC_MODE_DELAYED): R = s(-x)/s(x) r_up r_dn, r_s = 1 + Delta_s (1 - G_s[q][q]).
+//   Constrained-path heat bath (WIN_MODE_CP, Sec. IV.D, Eq. ptilde): lambda(x) = p(x) s(x) r_up(x) r_dn(x),
+//   negative lambda clamped to zero, x = +1 iff u (lambda(+1) + lambda(-1)) < lambda(+1); the walker is
+//   removed when both vanish; every site is an accept.
+template <typename T, int MODE>
+__device__ __forceinline__ void window_sub_sites(T* Gs, int n, int P, int b0, int nbk, const int8_t* xw, const T* s_u,
+                                                 const uint8_t* s_rep, bool forced, const T (*dflip)[2],
+                                                 const T* sflip, T* s_rat, T* s_det, uint8_t* s_dec, int8_t* s_xch,
+                                                 T (*s_fk)[WinCap<T>::NW], int* idx, WinScan<T>& sc, int lane) {
+    constexpr int B = WinSub<T>::B, CG = 16 / B, CW = B / CG;
+    constexpr unsigned FULL = 0xffffffffu;
+    const int s = lane >> 4, r = (lane & 15) / CG, cg = lane % CG, half = lane & 16;
+    T g[CW];  // columns q0 + j CG + cg of row r, q0 the site the loop is at
+#pragma unroll
+    for (int j = 0; j < CW; ++j) {
+        const int c = j * CG + cg;
+        g[j] = (r < nbk && c < nbk) ? Gs[(s * n + b0 + r) * P + b0 + c] : T(0);
+    }
+    T* col = Gs + (size_t)(s * n + b0 + (r < nbk ? r : 0)) * P + b0 + cg;
+    const int ls = lane < nbk ? lane : 0;  // lane l < nbk keeps the inputs and outputs of site l
+    const T u_l = s_u[b0 + ls];
+    const int x_l = xw[b0 + ls], rep_l = s_rep[b0 + ls];
+    const T d0 = dflip[s][0], d1 = dflip[s][1], sf0 = sflip[0], sf1 = sflip[1];
+    unsigned mask = 0, plus = 0;
+    T rat_l = T(0), det_l = T(0), f_l = T(0);
+    const int m0 = sc.m;
+#pragma unroll 1
+    for (int q0 = 0; q0 < nbk && sc.alive; q0 += CG) {
+#pragma unroll
+        for (int t = 0; t < CG; ++t) {  // the current column sits in g[0] of the lanes cg == t
+            const int q = q0 + t, src = half + q * CG;
+            if (t > 0 && (q >= nbk || !sc.alive)) break;
+            const T a = T(1) - __shfl_sync(FULL, g[0], src + t);
+            const T u = __shfl_sync(FULL, u_l, q);
+            const bool rep = __shfl_sync(FULL, rep_l, q) != 0;
+            bool acc;
+            T f;
+            if (MODE == WIN_MODE_CP) {
+                const T rp = T(1) + d0 * a, rm = T(1) + d1 * a;
+                const T rpo = __shfl_xor_sync(FULL, rp, 16), rmo = __shfl_xor_sync(FULL, rm, 16);
+                const T lp = fmax(sf0 * (s ? rpo : rp) * (s ? rp : rpo), T(0));
+                const T lm = fmax(sf1 * (s ? rmo : rm) * (s ? rm : rmo), T(0));
+                const T nrm = lp + lm;
+                acc = nrm > T(0) && isfinite(nrm);
+                if (!acc) {
+                    sc.alive = false;
+                    if (!isfinite(nrm)) sc.bad = true;
+                }
+                const bool up = forced ? rep : u * nrm < lp;
+                f = -((up ? d0 : d1) / (up ? rp : rm));
+                if (acc && up) plus |= 1u << q;
+                if (lane == q) {
+                    rat_l = nrm;
+                    det_l = up ? rp * rpo : rm * rmo;
+                }
+            } else {
+                const int xi = __shfl_sync(FULL, x_l, q) > 0 ? 0 : 1;
+                const T dl = xi ? d1 : d0;
+                const T rr = T(1) + dl * a, ro = __shfl_xor_sync(FULL, rr, 16);
+                const T R = (xi ? sf1 : sf0) * (s ? ro : rr) * (s ? rr : ro);
+                acc = forced ? rep : u < fabs(R);
+                if (!isfinite(R)) {
+                    acc = false;
+                    sc.bad = true;
+                }
+                f = -(dl / rr);
+                if (lane == q) rat_l = R;
+                if (acc) {
+                    if (R < T(0)) ++sc.nneg;
+                    sc.maxr = fmax(sc.maxr, fabs(R));
+                }
+            }
+            ++sc.done;
+            if (acc) {
+                mask |= 1u << q;
+                if ((lane & 15) == q) f_l = f;
+                const T fc = -f * (CG == 1 ? g[0] : __shfl_sync(FULL, g[0], half + r * CG + t));
+#pragma unroll
+                for (int j = t == CG - 1 ? 1 : 0; j < CW; ++j) {
+                    const T rv = __shfl_sync(FULL, g[j], src + cg);
+                    if (r > q && (j > 0 || cg > t)) g[j] = fma(fc, rv, g[j]);
+                }
+            }
+        }
+        if (r < nbk && q0 + cg < nbk) col[q0] = g[0];  // these columns are never written again
+#pragma unroll
+        for (int j = 0; j + 1 < CW; ++j) g[j] = g[j + 1];
+    }
+    sc.m = m0 + __popc(mask);
+    if (lane < nbk) {
+        s_dec[b0 + lane] = MODE == WIN_MODE_CP ? (plus >> lane) & 1u : (mask >> lane) & 1u;
+        s_rat[b0 + lane] = rat_l;
+        if (MODE == WIN_MODE_CP) s_det[b0 + lane] = det_l;
+    }
+    if ((mask >> (lane & 15)) & 1u) {
+        const int k = m0 + __popc(mask & ((1u << (lane & 15)) - 1u));
+        s_fk[s][k] = f_l;
+        if (s == 0) {
+            idx[k] = b0 + lane;
+            if (MODE == WIN_MODE_CP) s_xch[k] = (plus >> lane) & 1u ? 1 : -1;
+        }
+    }
+}
+
+// The accepts k = 0 .. mk - 1 of the sub-block that ends before site b1 (sites ia[k], factors fa[s][k])
+// applied to the rows and columns [b1, n) of both spins, all threads of the block:
+//   1. the coefficient triangles of the sub-block, shifted to start after the diagonal:
+//      D[0][s][k'][j] = G[a_k'][a_k] and D[1][s][k'][j] = -f_k' G[a_k][a_k'], k = k' + 1 + j (f = -Delta/r);
+//   2. one thread per row (or column) of the panels: column a_k of the rows after the sub-block, and
+//      row a_k of the columns after it, as they stood when a_k was accepted, by the recursion over the
+//      earlier accepts; stored in place (the frozen coefficients) and as pw[s][r][k] = -f_k G[r][a_k],
+//      qv[s][k][c] = G[a_k][c], zero-padded to whole 16-byte vectors;
+//   3. G[r][c] += sum_k pw qv, in accept order, one column and a few rows a thread.
+// The arithmetic is that of one trailing rank-1 update per accept, in the same order.
+template <typename T>
+__device__ __forceinline__ void window_sub_update(T* Gs, int n, int P, int b1, int mk, const int* ia, const T* fu,
+                                                  const T* fd, T* D, T* pw, T* qv, int tid, int nt) {
+    constexpr int B = WinSub<T>::B, VW = Vec16<T>::W;
+    using V = typename Vec16<T>::V;
+    const int rem = n - b1;
+    for (int e = tid; e < 4 * B * B; e += nt) {
+        const int j = e % B, kp = (e / B) % B, s = (e / (B * B)) & 1, kind = e / (2 * B * B), k = kp + 1 + j;
+        T v = T(0);
+        if (k < mk) {
+            const T* Gb = Gs + (size_t)s * n * P;
+            v = kind ? -(s ? fd : fu)[kp] * Gb[ia[k] * P + ia[kp]] : Gb[ia[kp] * P + ia[k]];
+        }
+        D[e] = v;
+    }
+    __syncthreads();
+    for (int e = tid; e < 4 * rem; e += nt) {
+        const int kind = e >= 2 * rem ? 1 : 0, e2 = e - kind * 2 * rem, s = e2 >= rem ? 1 : 0, i = e2 - s * rem;
+        T* line = Gs + (size_t)s * n * P + (kind ? b1 + i : (b1 + i) * P);
+        const int step = kind ? P : 1;
+        const T* Dm = D + (kind * 2 + s) * B * B;
+        const T* f = s ? fd : fu;
+        T* out = kind ? qv + s * B * n + i : pw + (s * n + i) * B;
+        const int ostep = kind ? n : 1;
+        T v[B];  // v[j]: entry kp + j of the line, kp the accept the loop is at
+#pragma unroll
+        for (int k = 0; k < B; ++k) v[k] = k < mk ? line[ia[k] * step] : T(0);
+#pragma unroll 1
+        for (int kp = 0; kp < mk; ++kp) {
+            const T w = kind ? v[0] : -f[kp] * v[0];
+            line[ia[kp] * step] = v[0];
+            out[kp * ostep] = w;
+#pragma unroll
+            for (int j0 = 0; j0 < B; j0 += VW) {
+                T d[VW];
+                *(V*)d = *(const V*)(Dm + kp * B + j0);
+#pragma unroll
+                for (int l = 0; l < VW; ++l)
+                    if (j0 + l + 1 < B) v[j0 + l] = fma(w, d[l], v[j0 + l + 1]);
+            }
+        }
+        for (int kp = mk; kp < (mk + VW - 1) / VW * VW; ++kp) out[kp * ostep] = T(0);
+    }
+    __syncthreads();
+    const int rt = (2 * rem * rem + nt - 1) / nt, ngr = (rem + rt - 1) / rt, tot = 2 * rem * ngr;
+    for (int e = tid; e < tot; e += nt) {
+        const int s = e >= rem * ngr ? 1 : 0, e2 = e - s * rem * ngr, rg = e2 / rem, c = e2 - rg * rem;
+        T q[B];
+#pragma unroll
+        for (int k0 = 0; k0 < B; k0 += VW)
+#pragma unroll
+            for (int l = 0; l < VW; ++l) q[k0 + l] = k0 < mk ? qv[(s * B + k0 + l) * n + c] : T(0);
+        const int rlo = rg * rt, rhi = min(rem, rlo + rt);
+        T* out = Gs + ((size_t)s * n + b1 + rlo) * P + b1 + c;
+        const T* pr = pw + (size_t)(s * n + rlo) * B;
+        for (int r = rlo; r < rhi; ++r, out += P, pr += B) {
+            T acc = *out;
+#pragma unroll
+            for (int k0 = 0; k0 < B; k0 += VW) {
+                if (k0 < mk) {
+                    T w[VW];
+                    *(V*)w = *(const V*)(pr + k0);
+#pragma unroll
+                    for (int l = 0; l < VW; ++l) acc = fma(w[l], q[k0 + l], acc);
+                }
+            }
+            *out = acc;
+        }
+    }
+    __syncthreads();
 }
 
 template <typename T, int MODE>
@@ -500,15 +730,19 @@ __global__ void __launch_bounds__(WIN_THREADS) window_kernel(const T* __restrict
     const WindowBufs wb = wb_walker<T>(wb0, wk, N);
     const T* blk = blk0 ? blk0 + (size_t)wk * 2 * WinCap<T>::NW * WinCap<T>::NW : nullptr;
     T* Gs = (T*)smem_raw;  // [2][n][P]
-    size_t off = 2 * (size_t)n * P * sizeof(T);
+    size_t off = 2 * (size_t)n * P * sizeof(T);  // a multiple of 16: n (n + 1) is even
+    constexpr int SB = WinSub<T>::B;
+    T* Dsub = (T*)(smem_raw + off);    // [2][2][SB][SB] sub-block coefficients (window_sub_update)
+    T* pwsub = Dsub + 4 * SB * SB;     // [2][n][SB]
+    T* qvsub = pwsub + 2 * n * SB;     // [2][SB][n]
+    off += 4 * (size_t)SB * (SB + n) * sizeof(T);
     T* S1 = (T*)(smem_raw + off);  // [2][NBMAX][NBMAX+1]
     off += 2 * (size_t)NBMAX * (NBMAX + 1) * sizeof(T);
     T* stc = (T*)(smem_raw + off);  // staging: col[2][n], row[2][n]
     off += 4 * (size_t)n * sizeof(T);
     T* stb = (T*)(smem_raw + off);  // small staging [2][NBMAX]
     off += 2 * (size_t)NBMAX * sizeof(T);
-    double* dl = (double*)(smem_raw + ((off + 7) & ~(size_t)7));  // [2][n]
-    off = ((off + 7) & ~(size_t)7) + 2 * (size_t)n * sizeof(double);
+    off = (off + 7) & ~(size_t)7;
     double* fb = (double*)(smem_raw + off);  // block-FB scalars [8][NBMAX]
     off += 8 * (size_t)NBMAX * sizeof(double);
     int* idx = (int*)(smem_raw + off);  // accepted positions [n]
@@ -524,29 +758,24 @@ __global__ void __launch_bounds__(WIN_THREADS) window_kernel(const T* __restrict
     const T* G[2] = {Gu, Gd};
     // the n x n diagonal block of both spins: from G, or from the corrected snapshot the
     // previous window's flush prepared (pitch NW, spin stride NW^2)
-    {  // eight loads in flight per thread before their shared-memory stores
-        constexpr int NL = 8;
-        const int nn2 = n * n;
-        for (int e0 = tid; e0 < 2 * nn2; e0 += NL * nt) {
-            T v[NL];
+    {  // warps over rows, lanes over columns; four rows' loads in flight per thread before their stores
+        const int lane = tid & 31;
+        for (int c = lane; c < n; c += 32)
+            for (int row0 = tid >> 5; row0 < 2 * n; row0 += 4 * (nt >> 5)) {
+                T v[4];
 #pragma unroll
-            for (int q = 0; q < NL; ++q) {
-                const int e = e0 + q * nt;
-                if (e < 2 * nn2) {
-                    const int s = e >= nn2 ? 1 : 0, rem = e - s * nn2, a = rem / n, c = rem - a * n;
-                    v[q] = blk ? blk[((size_t)s * WinCap<T>::NW + a) * WinCap<T>::NW + c]
-                               : G[s][(long)(s0 + a) * ld + (s0 + c)];
+                for (int q = 0; q < 4; ++q) {
+                    const int row = row0 + q * (nt >> 5), s = row >= n ? 1 : 0, a = row - s * n;
+                    if (row < 2 * n)
+                        v[q] = blk ? blk[((size_t)s * WinCap<T>::NW + a) * WinCap<T>::NW + c]
+                                   : G[s][(long)(s0 + a) * ld + (s0 + c)];
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int row = row0 + q * (nt >> 5);
+                    if (row < 2 * n) Gs[row * P + c] = v[q];
                 }
             }
-#pragma unroll
-            for (int q = 0; q < NL; ++q) {
-                const int e = e0 + q * nt;
-                if (e < 2 * nn2) {
-                    const int s = e >= nn2 ? 1 : 0, rem = e - s * nn2, a = rem / n, c = rem - a * n;
-                    Gs[(s * n + a) * P + c] = v[q];
-                }
-            }
-        }
     }
     for (int p = tid; p < n; p += nt) xw[p] = xl_g[s0 + p];
     // the window's site uniforms (and forced decisions) live in shared memory: the scan reads
@@ -554,17 +783,11 @@ __global__ void __launch_bounds__(WIN_THREADS) window_kernel(const T* __restrict
     // (in the bulk precision: the delayed scan compares them with ratios computed in T)
     __shared__ T s_u[WinCap<float>::NW];
     __shared__ uint8_t s_rep[WinCap<float>::NW];
-    __shared__ T s_rat[WinCap<float>::NW];    // ratio of every decided site, written out after the scan
+    __shared__ T s_rat[WinCap<float>::NW];    // ratio of every decided site, written out after the decisions
     __shared__ uint8_t s_dec[WinCap<float>::NW];
-    __shared__ int s_nneg;                    // number of accepted negative ratios (sign parity)
-    __shared__ T s_maxrT;
     for (int p = tid; p < n; p += nt) {
         s_u[p] = (T)u[s0 + p];
         s_rep[p] = replay ? replay[s0 + p] : 0;
-    }
-    if (tid == 0) {
-        s_nneg = 0;
-        s_maxrT = T(0);
     }
     __shared__ double c_dflip[2][2], c_dstrip[2][2], c_sflip[2];
     __shared__ T c_dflipT[2][2], c_sflipT[2];  // the same in T for the scan's critical path
@@ -596,144 +819,56 @@ __global__ void __launch_bounds__(WIN_THREADS) window_kernel(const T* __restrict
     }
     __syncthreads();
     if (MODE == AFQMC_MODE_DELAYED || MODE == WIN_MODE_CP) {
-        // Warp-serial Metropolis, one accept ahead of the block update: warp 0 keeps its own copy
-        // of the two diagonals, applies each accept's effect on them itself, and scans the next
-        // sites (32 at a time: a rejection leaves G unchanged, a ballot finds the first
-        // acceptance) while warps 1..31 apply the previous accept's trailing update to the block.
-        // Warp 0 reads only row a and column a of an accept a, which that accept's own update never
-        // writes; the earlier updates that do write them are complete at the barrier before.  One
-        // block barrier per accept.
-        T* dg = stc;  // [2][n] warp 0's diagonals (the block-FB path's column / row staging, unused here)
-        for (int q = tid; q < 2 * n; q += nt) dg[q] = Gs[((q / n) * n + q % n) * P + q % n];
-        __shared__ int s_pend[2];
-        __syncthreads();
-        int pend = -1;  // accept whose block update the workers apply in this iteration
-        int p = 0;      // next site to test (warp 0)
-        int m_w0 = 0;   // accepts so far (warp 0)
-        for (int it = 0;; ++it) {
+        // Two levels: warp 0 decides a sub-block of SB sites in registers (no barrier per accept), then
+        // all warps bring the rest of the window's block up to date with the sub-block's accepts.
+        __shared__ int s_mk[2];
+        __shared__ T s_det[WinCap<float>::NW];  // constrained path: r_up r_dn of every site
+        WinScan<T> sc;
+        sc.alive = !((MODE == WIN_MODE_CP) && s_dead);
+        int m_all = 0;
+        for (int b0 = 0, it = 0; b0 < n; b0 += SB, ++it) {
+            const int b1 = min(n, b0 + SB);
             if (tid < 32) {
-                if (pend >= 0) {  // the pending accept's effect on the later diagonals
-                    const int a = idx[pend];
-                    const T f0 = -s_fk[0][pend], f1 = -s_fk[1][pend];
-                    for (int q = a + 1 + tid; q < n; q += 32) {
-                        dg[q] = fma(f0 * Gs[(0 * n + q) * P + a], Gs[(0 * n + a) * P + q], dg[q]);
-                        dg[n + q] = fma(f1 * Gs[(1 * n + q) * P + a], Gs[(1 * n + a) * P + q], dg[n + q]);
-                    }
-                    __syncwarp();
-                }
-                int next = -1;
-                if (MODE == WIN_MODE_CP) {
-                    // constrained-path heat bath (Sec. IV.D, Eq. ptilde): lane 0 draws the field of
-                    // site p from lambda(x) = p(x) s(x) r_up(x) r_dn(x), r_s(x) = 1 + (e^{c_s x} - 1)
-                    // (1 - G_pp), negative lambda clamped to zero (the constraint); the walker is
-                    // removed when both vanish.  Every site is an accept of the delayed update.
-                    if (p < n && !s_dead) {
-                        if (tid == 0) {
-                            const int q = p;
-                            const T a0 = T(1) - dg[q], a1 = T(1) - dg[n + q];
-                            const T rp0 = T(1) + c_dflipT[0][0] * a0, rp1 = T(1) + c_dflipT[1][0] * a1;
-                            const T rm0 = T(1) + c_dflipT[0][1] * a0, rm1 = T(1) + c_dflipT[1][1] * a1;
-                            const T lp = fmax(c_sflipT[0] * rp0 * rp1, T(0));
-                            const T lm = fmax(c_sflipT[1] * rm0 * rm1, T(0));
-                            const T nrm = lp + lm;
-                            if (!(nrm > T(0)) || !isfinite(nrm)) {
-                                s_dead = 1;
-                                if (!isfinite(nrm)) set_err(err, DEV_NUMERIC);
-                            } else {
-                                const bool plus = replay ? (s_rep[q] != 0) : (s_u[q] < lp / nrm);
-                                const int xi = plus ? 0 : 1;
-                                const T r0 = plus ? rp0 : rm0, r1 = plus ? rp1 : rm1;
-                                s_fk[0][m_w0] = -(c_dflipT[0][xi] / r0);
-                                s_fk[1][m_w0] = -(c_dflipT[1][xi] / r1);
-                                idx[m_w0] = q;
-                                s_xch[m_w0] = plus ? 1 : -1;
-                                s_dec[q] = plus ? 1 : 0;
-                                s_rat[q] = nrm;
-                                s_cpl[0] += log((double)nrm);
-                                s_cpl[1] += log(fabs((double)r0 * (double)r1));
-                                next = m_w0;
-                            }
-                        }
-                        next = __shfl_sync(0xffffffffu, next, 0);
-                        if (next >= 0) {
-                            ++m_w0;
-                            ++n_acc;
-                            ++n_flip;
-                        }
-                        ++n_prop;
-                        p = (next >= 0) ? p + 1 : n;
-                    }
-                }
-                while (MODE == AFQMC_MODE_DELAYED && p < n) {
-                    // ratio arithmetic in the bulk precision T (FP64 division on this critical path
-                    // would cost thousands of cycles on GB300's FP64 pipe)
-                    const int q = p + tid;
-                    bool acc = false;
-                    T R = T(0), rr0 = T(1), rr1 = T(1);
-                    int xi = 0;
-                    if (q < n) {
-                        xi = xw[q] > 0 ? 0 : 1;
-                        rr0 = T(1) + c_dflipT[0][xi] * (T(1) - dg[q]);
-                        rr1 = T(1) + c_dflipT[1][xi] * (T(1) - dg[n + q]);
-                        R = c_sflipT[xi] * rr0 * rr1;
-                        acc = replay ? (s_rep[q] != 0) : (s_u[q] < fabs(R));
-                        if (!isfinite(R)) {
-                            acc = false;
-                            set_err(err, DEV_NUMERIC);
-                        }
-                    }
-                    const unsigned ball = __ballot_sync(0xffffffffu, acc);
-                    const int first = ball ? __ffs(ball) - 1 : 32;
-                    if (q < n && tid <= first) {
-                        s_dec[q] = (tid == first) ? 1 : 0;
-                        s_rat[q] = R;
-                    }
-                    if (tid == first) {
-                        s_fk[0][m_w0] = -(c_dflipT[0][xi] / rr0);  // recursion factor f = -Delta / r
-                        s_fk[1][m_w0] = -(c_dflipT[1][xi] / rr1);
-                        idx[m_w0] = q;
-                        if (R < T(0)) s_nneg = s_nneg + 1;
-                        s_maxrT = fmax(s_maxrT, fabs(R));
-                    }
-                    if (first < 32) {
-                        n_prop += first + 1;
-                        p = p + first + 1;
-                        next = m_w0++;
-                        ++n_acc;
-                        ++n_flip;
-                        break;
-                    }
-                    n_prop += min(32, n - p);
-                    p = min(n, p + 32);
-                }
-                if (tid == 0) {
-                    s_pend[it & 1] = next;
-                    s_m = m_w0;
-                }
-                __syncwarp();
-            } else if (pend >= 0) {
-                // warps 1..31: G[r][c] += f G[r][a] G[a][c] for r, c > a, both spins.  Rows and
-                // columns <= a are never touched again, so the block keeps row a and column a as
-                // they were when site a was accepted (the coefficients of the flush recursion).
-                trailing_update(Gs, n, P, idx[pend], -s_fk[0][pend], -s_fk[1][pend], tid - 32, nt - 32);
+                window_sub_sites<T, MODE>(Gs, n, P, b0, b1 - b0, xw, s_u, s_rep, replay != nullptr, c_dflipT,
+                                          c_sflipT, s_rat, s_det, s_dec, s_xch, s_fk, idx, sc, tid);
+                if (tid == 0) s_mk[it & 1] = sc.m;
             }
             __syncthreads();
-            const int np = s_pend[it & 1];
-            if (np < 0) break;  // nothing accepted in the rest of the window: the last update is applied
-            pend = np;
+            const int mk = s_mk[it & 1] - m_all;
+            if (mk > 0 && b1 < n)
+                window_sub_update<T>(Gs, n, P, b1, mk, idx + m_all, s_fk[0] + m_all, s_fk[1] + m_all, Dsub, pwsub,
+                                     qvsub, tid, nt);
+            m_all += mk;
         }
-        // off the critical path: decisions, ratios, factors and the sign in their ABI types
+        if (tid == 0) {
+            s_m = sc.m;
+            if (sc.bad) set_err(err, DEV_NUMERIC);
+            if (sc.nneg & 1) s_sign = -s_sign;
+            s_maxr = fmax(s_maxr, (double)sc.maxr);
+            n_prop = sc.done;
+            n_acc = n_flip = sc.m;
+            if (MODE == WIN_MODE_CP && !sc.alive) s_dead = 1;
+        }
+        __syncthreads();
+        // decisions and ratios in their ABI types; the walker's weight factors as sums over its sites
         for (int q = tid; q < n; q += nt) {
             so.dec[s0 + q] = s_dec[q];
             so.ratio[s0 + q] = (double)s_rat[q];
         }
-        for (int q = tid; q < s_m; q += nt) {
-            dl[0 * n + q] = (double)s_fk[0][q];
-            dl[1 * n + q] = (double)s_fk[1][q];
-        }
-        if (tid == 0) {
-            if (s_nneg & 1) s_sign = -s_sign;
-            s_maxr = fmax(s_maxr, (double)s_maxrT);
+        if (MODE == WIN_MODE_CP && tid < 32) {
+            double a0 = 0.0, a1 = 0.0;
+            for (int q = tid; q < s_m; q += 32) {
+                a0 += log((double)s_rat[idx[q]]);
+                a1 += log(fabs((double)s_det[idx[q]]));
+            }
+            for (int o = 16; o > 0; o >>= 1) {
+                a0 += __shfl_xor_sync(0xffffffffu, a0, o);
+                a1 += __shfl_xor_sync(0xffffffffu, a1, o);
+            }
+            if (tid == 0) {
+                s_cpl[0] = a0;
+                s_cpl[1] = a1;
+            }
         }
         __syncthreads();
     } else if (MODE == WIN_MODE_CPB) {
@@ -819,8 +954,6 @@ __global__ void __launch_bounds__(WIN_THREADS) window_kernel(const T* __restrict
                     idx[k] = a;
                     s_fk[0][k] = -s_phi2[0][q];
                     s_fk[1][k] = -s_phi2[1][q];
-                    dl[0 * n + k] = -(double)s_phi2[0][q];
-                    dl[1 * n + k] = -(double)s_phi2[1][q];
                 }
                 trailing_update(Gs, n, P, a, s_phi2[0][q], s_phi2[1][q], tid, nt);
                 __syncthreads();
@@ -970,8 +1103,6 @@ __global__ void __launch_bounds__(WIN_THREADS) window_kernel(const T* __restrict
                     idx[k] = a;
                     s_fk[0][k] = -s_phi[0][q];
                     s_fk[1][k] = -s_phi[1][q];
-                    dl[0 * n + k] = -(double)s_phi[0][q];
-                    dl[1 * n + k] = -(double)s_phi[1][q];
                     xw[a] = (int8_t)(-xw[a]);
                 }
                 trailing_update(Gs, n, P, a, s_phi[0][q], s_phi[1][q], tid, nt);
@@ -997,11 +1128,7 @@ __global__ void __launch_bounds__(WIN_THREADS) window_kernel(const T* __restrict
         __syncthreads();
     }
     for (int p = tid; p < n; p += nt) xl_g[s0 + p] = xw[p];
-    for (int q = tid; q < m; q += nt) {
-        wb.idx[q] = s0 + idx[q];
-        wb.dtot[q] = dl[q];
-        wb.dtot[WinCap<T>::NW + q] = dl[n + q];
-    }
+    for (int q = tid; q < m; q += nt) wb.idx[q] = s0 + idx[q];
     // The window's update matrix W (Eq. DelayRgenk in G form).  With C[k][k'] = Gs[idx[k]][idx[k']]
     // the block entries frozen at acceptance time (rows and columns at or before an accepted site
     // are never touched again), f_k = -Delta_k / r_k, L1 = I + Cl F and U1 = I + Cu F (Cl, Cu the
@@ -1009,8 +1136,9 @@ __global__ void __launch_bounds__(WIN_THREADS) window_kernel(const T* __restrict
     // W = -F U1^{-1} L1^{-1}: per column of the identity a forward and a backward substitution,
     //   y_k = b_k - sum_{k'<k} C[k][k'] f_k' y_k',   z_k = y_k - sum_{k'>k} C[k][k'] f_k' z_k',
     //   W_k = -f_k z_k.
-    // Each warp owns WCPW columns of one spin in registers (lane l holds rows l, l + 32, ...) and
-    // broadcasts the finished row of every step with a shuffle: no block-wide barrier per step.
+    // The coefficients are gathered into a dense m x m matrix first; then each warp owns a few columns
+    // of one spin in registers (lane l holds rows l, l + 32, ...) and broadcasts the finished row of
+    // every step with a shuffle: no block-wide barrier per step.
     window_w<T>(Gs, n, P, idx, s_fk, m, (T*)wb.Wx, tid);
     if (tid == 0) {
         *wb.m = m;
