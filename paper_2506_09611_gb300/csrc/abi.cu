@@ -85,7 +85,7 @@ struct Walker {
     GridBar* bar = nullptr;
     int* err = nullptr;
     // window buffers, double-buffered by window parity (the flush of window w overlaps the
-    // decisions of window w + 1), and the corrected snapshots of the next window's block
+    // decisions of window w + 1), and the next window's block after the window's update
     int* wm[2] = {nullptr, nullptr};
     int* widx[2] = {nullptr, nullptr};
     void* Wm[2] = {nullptr, nullptr};
@@ -877,7 +877,7 @@ int afqmc_init_walkers(afqmc_ctx* ctx, int n_walkers, const int* L, const int* n
             CK(dalloc(A, (char**)&w->Wm[q], (size_t)nwk * 2 * NW * NW * es));
             CK(dalloc(A, (char**)&w->Wx[q], (size_t)nwk * 2 * NW * NW * es));
             CK(dalloc(A, (char**)&w->X[q], (size_t)nwk * 2 * N * NW * es));
-            CK(dalloc(A, (char**)&w->Y[q], (size_t)nwk * 4 * NW * N * es));
+            CK(dalloc(A, (char**)&w->Y[q], (size_t)nwk * 2 * NW * N * es));
             CK(dalloc(A, (char**)&w->snap[q], (size_t)nwk * 2 * NW * NW * es));
             CK(cudaEventCreateWithFlags(&w->ev_chain[q], cudaEventDisableTiming));
             CK(cudaEventCreateWithFlags(&w->ev_prod[q], cudaEventDisableTiming));
@@ -951,7 +951,7 @@ int afqmc_init_walkers(afqmc_ctx* ctx, int n_walkers, const int* L, const int* n
             CK(cudaMemsetAsync(w->Wm[q], 0, (size_t)nwk * 2 * NW * NW * es, st));
             CK(cudaMemsetAsync(w->Wx[q], 0, (size_t)nwk * 2 * NW * NW * es, st));
             CK(cudaMemsetAsync(w->X[q], 0, (size_t)nwk * 2 * N * NW * es, st));
-            CK(cudaMemsetAsync(w->Y[q], 0, (size_t)nwk * 4 * NW * N * es, st));
+            CK(cudaMemsetAsync(w->Y[q], 0, (size_t)nwk * 2 * NW * N * es, st));
         }
         // fields: the caller's, else Philox-drawn +-1 per walker
         for (int j = 0; j < nwk; ++j) {
@@ -1224,11 +1224,11 @@ static int sweep_impl(afqmc_ctx* ctx, int gi, int ell, int dir, int mode, int k,
         }
     } else {
         int nw = (mode == AFQMC_MODE_DELAYED) ? k : (NW / nb) * nb;
-        // Window w's decisions and the corrected block of window w + 1 run on st; window w's
-        // panels and rank-m product run on the group's flush stream sf and overlap the
-        // decisions of window w + 1.  Before building window w + 1's block, st waits for the
-        // product of window w - 1 (ev_prod), which is also what frees the window buffers of
-        // parity (w + 1) & 1 for reuse.  Every launch covers all walkers of the group.
+        // Window w's decisions and panels run on st; its rank-m product runs on the group's flush
+        // stream sf and overlaps the decisions of window w + 1, whose block (as window w's update will
+        // leave it) comes with the panels.  Before window w's panels are formed, st waits for the product
+        // of window w - 1 (ev_prod), which also frees the window buffers of parity (w + 1) & 1 for reuse.
+        // Every launch covers all walkers of the group.
         WindowBufs wb[2];
         for (int q = 0; q < 2; ++q) {
             wb[q].m = w->wm[q];
@@ -1247,14 +1247,11 @@ static int sweep_impl(afqmc_ctx* ctx, int gi, int ell, int dir, int mode, int k,
             const T* blk = (wi > 0) ? (const T*)w->snap[par ^ 1] : nullptr;
             CK(launch_window_chain<T>(st, mode, G0, G1, xl, w->u, rep, sp, so, s0, n, nb, wb[par], blk, w->err, bt));
             const int sn = s0 + n, nn = (sn < N) ? ((N - sn < nw) ? N - sn : nw) : 0;
-            if (nn > 0) {  // the next window's block
-                if (wi > 0) CK(cudaStreamWaitEvent(st, w->ev_prod[par ^ 1], 0));
-                CK(launch_next_block<T>(st, G0, G1, sp, wb[par], sn, nn, (T*)w->snap[par], bt));
-            }
+            if (wi > 0) CK(cudaStreamWaitEvent(st, w->ev_prod[par ^ 1], 0));
+            CK(launch_flush_panels<T>(st, G0, sp, wb[par], s0, n, sn, nn, (T*)w->snap[par], bt));
             CK(cudaEventRecord(w->ev_chain[par], st));
             CK(cudaStreamWaitEvent(w->sf, w->ev_chain[par], 0));
             PhaseScope pf(ctx, AFQMC_PHASE_FLUSH, w->sf);
-            CK(launch_flush_panels<T>(w->sf, G0, G1, sp, wb[par], n, bt));
             {
                 PhaseScope pg(ctx, AFQMC_PHASE_FLUSH_GEMM, w->sf);
                 CK(launch_flush_gemm<T>(w->sf, G0, G1, sp, wb[par], n, bt));
@@ -1337,7 +1334,7 @@ __global__ void cp_finish_kernel(double* cpl, double* det, double* out, int nwk)
 
 // The window loop of the T form over the N sites of slice ell (Sec. II.C): per window J the block
 // 1 - (U_R[J, :] T) U_L[:, J], the window kernel (Metropolis modes, or the constrained-path heat bath
-// WIN_MODE_CP), then T <- T - (T U_L[:, I]) (W (U_R[I, :] T)) and the rows I of U_R times
+// WIN_MODE_CP), then T <- T - (T U_L[:, I]) W (U_R[I, :] T) and the rows I of U_R times
 // exp(mul c_s x'_I) (mul = 2 for a flip, 1 for a field set from none).
 template <typename T>
 static int tform_windows(afqmc_ctx* ctx, Walker* w, cudaStream_t st, int8_t* xl, int mode, int k, int nb,
@@ -1395,36 +1392,32 @@ static int tform_windows(afqmc_ctx* ctx, Walker* w, cudaStream_t st, int8_t* xl,
             g2.C = blk; g2.ldc = NW; g2.sC = sB;
             CK(gemm<T>(st, g2));
             CK(launch_identity_minus<T>(st, blk, NW, n, nb2, sB));
-            // decisions and the window's W
+            // decisions
             CK(launch_window_chain<T>(st, mode, (const T*)w->G, nullptr, xl, w->u, rep, sp, so, s0, n, nb, wb, blk,
                                       w->err, bt));
-            // T <- T - (T U_L[:, I]) (W (U_R[I, :] T)), then the rows I of U_R
+            // T <- T + V Y' from V = T U_L[:, I] and Y = U_R[I, :] T by the accepts' recursion (at most n
+            // columns and rows), then the rows I of U_R
             PhaseScope pf(ctx, AFQMC_PHASE_FLUSH, st);
             CK(launch_tform_gather<T>(st, UR, UL, N, ns, ns, fs, fs, wb, ULI, URI, nb2));
             GemmArgs<T> v;
-            v.M = ns; v.N = NW; v.K = ns; v.batch = nb2;
+            v.M = ns; v.N = n; v.K = ns; v.batch = nb2;
             v.A = TT; v.lda = ns; v.sA = sT;
             v.B = ULI; v.ldb = NW; v.sB = (long)ns * NW;
             v.C = V; v.ldc = NW; v.sC = (long)ns * NW;
             CK(gemm<T>(st, v));
             GemmArgs<T> y;
-            y.M = NW; y.N = ns; y.K = ns; y.batch = nb2;
+            y.M = n; y.N = ns; y.K = ns; y.batch = nb2;
             y.A = URI; y.lda = ns; y.sA = sP;
             y.B = TT; y.ldb = ns; y.sB = sT;
             y.C = Y; y.ldc = ns; y.sC = sP;
             CK(gemm<T>(st, y));
-            GemmArgs<T> yp;  // Y' = W Y over the m accepted rows
-            yp.M = NW; yp.N = ns; yp.K = NW; yp.Kdev = wb.m; yp.kdiv = 2; yp.batch = nb2;
-            yp.A = (const T*)wb.Wx; yp.lda = NW; yp.sA = sB;
-            yp.B = Y; yp.ldb = ns; yp.sB = sP;
-            yp.C = Yp; yp.ldc = ns; yp.sC = sP;
-            CK(gemm<T>(st, yp));
-            GemmArgs<T> t;  // T -= V Y'
-            t.M = ns; t.N = ns; t.K = NW; t.Kdev = wb.m; t.kdiv = 2; t.batch = nb2;
+            CK(launch_tform_panels<T>(st, ns, wb, s0, n, V, Y, Yp, nwk));
+            GemmArgs<T> t;  // T += V Y'
+            t.M = ns; t.N = ns; t.K = n; t.Kdev = wb.m; t.kdiv = 2; t.batch = nb2;
             t.A = V; t.lda = NW; t.sA = (long)ns * NW;
             t.B = Yp; t.ldb = ns; t.sB = sP;
             t.C = TT; t.ldc = ns; t.sC = sT;
-            t.alpha = T(-1); t.beta = T(1);
+            t.alpha = T(1); t.beta = T(1);
             {
                 PhaseScope pg(ctx, AFQMC_PHASE_FLUSH_GEMM, st);
                 CK(gemm<T>(st, t));

@@ -243,12 +243,12 @@ cudaError_t launch_local(cudaStream_t st, T* Gu, T* Gd, int8_t* xl, const double
                          int max_blocks);
 
 struct WindowBufs {    // device scratch of the window chain + flush
-    int* m;            // accepted count of the window
+    int* m = nullptr;  // accepted count of the window
     int* idx;          // accepted site indices (global), capacity NW
-    void* Wm;          // per spin NW x NW (T): sweep: frozen block coefficients; apply_flips: W
-    void* Wx;          // per spin NW x NW (T): sweep: the window's update matrix W
+    void* Wm;          // per spin NW x NW (T): sweep: the accepts' scaled columns; apply_flips: W
+    void* Wx;          // per spin NW x NW (T): sweep: the accepts' rows
     void* X;           // per spin N x NW column panel (T)
-    void* Y;           // per spin NW x N row panel (T), plus room for a second product
+    void* Y;           // per spin NW x N row panel (T); apply_flips: plus room for a second product
     int nwk = 1;       // walkers in the group: every buffer above holds nwk back-to-back copies
 };
 
@@ -278,26 +278,29 @@ bool sep_available(int L, int N);          // launch_sep with w = 0 applies (lin
 template <typename T>
 cudaError_t launch_sep(cudaStream_t st, const SepArgs& a);
 
+// Decides the window [s0, s0 + n) of every walker of the group and leaves its accepts with their rows and
+// columns in wb.  The window's block of G comes from G itself (blk null) or from blk (pitch window_max).
 template <typename T>
 cudaError_t launch_window_chain(cudaStream_t st, int mode, const T* Gu, const T* Gd, int8_t* xl, const double* u,
                                 const uint8_t* replay, const SiteParams& sp, SliceOut so, int s0, int n, int nb,
                                 WindowBufs wb, const T* blk, int* err, Batch bt = Batch());
 template <typename T>
 cudaError_t launch_flush(cudaStream_t st, T* Gu, T* Gd, const SiteParams& sp, WindowBufs wb, int nw);
-// Pipelined flush of a window (the window kernel leaves its update matrix W in wb.Wx):
-//   launch_next_block   -- the next window's block [sn, sn + nn) of both spins as it will be
-//                          after this window's update; run right after the window kernel;
-//   launch_flush_panels -- X = G[:, I], Yraw = E_I^T - G[I, :], Y' = W Yraw;
-//   launch_flush_gemm   -- G <- G - X Y'.
+// Pipelined flush of a window (see sweep.cu):
+//   launch_flush_panels -- the update's panels X (N x m) and Y (m x N) of every spin and walker, and the
+//                          next window's block [sn, sn + nn) of G after this update into snap;
+//   launch_flush_gemm   -- G <- G + X Y;
+//   launch_tform_panels -- the same recursion on the T form's V = T U_L[:, I] (ns x m, pitch window_max,
+//                          in place) and R = U_R[I, :] T (m x ns) -> Y, so that T <- T + V Y.
 template <typename T>
-cudaError_t launch_next_block(cudaStream_t st, const T* Gu, const T* Gd, const SiteParams& sp, WindowBufs wb, int sn,
-                              int nn, T* snap, Batch bt = Batch());
-template <typename T>
-cudaError_t launch_flush_panels(cudaStream_t sf, T* Gu, T* Gd, const SiteParams& sp, WindowBufs wb, int nw,
-                                Batch bt = Batch());
+cudaError_t launch_flush_panels(cudaStream_t st, const T* Gu, const SiteParams& sp, WindowBufs wb, int s0, int n,
+                                int sn, int nn, T* snap, Batch bt = Batch());
 template <typename T>
 cudaError_t launch_flush_gemm(cudaStream_t sf, T* Gu, T* Gd, const SiteParams& sp, WindowBufs wb, int nw,
                               Batch bt = Batch());
+template <typename T>
+cudaError_t launch_tform_panels(cudaStream_t st, int ns, WindowBufs wb, int s0, int n, T* V, const T* R, T* Y,
+                                int nwk);
 // T form: the gathers of the window's accepted sites I for every (walker, spin) z of the batch,
 // ULI[z] = UL[z][:, I] (ns x m, pitch window_max<T>()) and URI[z] = UR[z][I, :] (m x ns, pitch ldr),
 // and the row scaling UR[z][I_k, :] *= exp(2 c_s x'_{I_k}) with the slice's new fields.  UR: N x ns

@@ -345,24 +345,18 @@ __device__ __forceinline__ WindowBufs wb_walker(WindowBufs wb, int j, int N) {
     wb.Wm = (T*)wb.Wm + (size_t)j * 2 * NW * NW;
     if (wb.Wx) wb.Wx = (T*)wb.Wx + (size_t)j * 2 * NW * NW;
     wb.X = (T*)wb.X + (size_t)j * 2 * N * NW;
-    wb.Y = (T*)wb.Y + (size_t)j * 2 * NW * N;  // this walker's Yraw (the products follow all walkers' Yraw)
+    wb.Y = (T*)wb.Y + (size_t)j * 2 * NW * N;
     return wb;
 }
 
-// Sites per sub-block of the window (window_sub_sites): what one warp keeps in registers for both
-// spins, 16 FP32 or 4 FP64 elements a lane.
-template <typename T> struct WinSub { static constexpr int B = sizeof(T) == 4 ? 16 : 8; };
-
 template <typename T>
 static size_t window_smem(int n) {
-    constexpr size_t B = WinSub<T>::B;
     size_t P = (size_t)n + 1;
-    size_t g = 2 * (size_t)n * P * sizeof(T);            // Gs[2][n][n+1]
-    size_t pan = 4 * B * (B + (size_t)n) * sizeof(T);    // sub-block coefficients and panels
+    size_t g = 2 * (size_t)n * P * sizeof(T);  // Gs[2][n][n+1]
     size_t s1 = 2 * (size_t)NBMAX * (NBMAX + 1) * sizeof(T);
     size_t vec = 4 * (size_t)n * sizeof(T) + 2 * (size_t)NBMAX * sizeof(T);  // staging vectors
     size_t misc = (size_t)n * (sizeof(int) + 1) + 8 * (size_t)NBMAX * sizeof(double) + 256;
-    return g + pan + s1 + vec + misc;
+    return g + s1 + vec + misc;
 }
 
 // G_s[r][c] += f_s * G_s[r][a] * G_s[a][c] for r, c in (a, n), both spins; 32 x 32 thread tiles.
@@ -379,334 +373,346 @@ __device__ __forceinline__ void trailing_update(T* Gs, int n, int P, int a, T f0
     }
 }
 
-// W = -F U1^{-1} L1^{-1} of the window (see the window kernel's tail); written to Wx[s][k][j] (pitch
-// NW).  Cc[s][k][k'] (pitch P, spin stride n P) holds C[k][k'] f_k'.  32 warps: spin = warp / 16,
-// columns (warp % 16) WC + c; lane l holds rows l + 32 r, r < RPL (RPL >= ceil(m / 32)).  WC is the
-// least count that covers m columns with 16 warps, so all of them work; the next step's coefficient
-// is fetched while the current one is applied, and the forward pass of a warp starts at its first
-// column (identity columns are zero above the diagonal).
-template <typename T, int RPL, int WC>
-__device__ __forceinline__ void window_w_rpl(const T* Cc, int n, int P, const T (*fk)[WinCap<T>::NW], int m, T* Wx,
-                                             int lane, int w) {
+// The window's accepts in sequential form, for panel_kernel: accept k at position a_k of the window with
+// factor f_k = -Delta_k / r_k leaves the row and column of the block as they were at that moment,
+//   Wx[s][k][c] = G[a_k][c] (c > a_k),  Wm[s][k][r] = -f_k G[r][a_k] (r > a_k),  both -f_k at a_k
+// (pitch NW; entries before a_k are never read).  Here from the block's frozen rows and columns.
+template <typename T>
+__device__ __forceinline__ void window_export(const T* Gs, int n, int P, const int* idx,
+                                              const T (*fk)[WinCap<T>::NW], int m, T* Wx, T* Wm, int tid) {
     constexpr int NW = WinCap<T>::NW;
-    const int s = w >> 4, j0 = (w & 15) * WC;
-    if (j0 >= m) return;
-    const T* Cb = Cc + (size_t)s * n * P;
-    T y[RPL][WC];
-#pragma unroll
-    for (int r = 0; r < RPL; ++r)
-#pragma unroll
-        for (int c = 0; c < WC; ++c) y[r][c] = (lane + 32 * r == j0 + c) ? T(1) : T(0);
-    auto coef = [&](int kp, T* cf) {  // C[k][kp] f_kp of this lane's rows
-#pragma unroll
-        for (int r = 0; r < RPL; ++r) {
-            const int k = lane + 32 * r;
-            cf[r] = k < m ? Cb[k * P + kp] : T(0);
-        }
-    };
-    auto bcast = [&](int kp, T* v) {  // row kp of y from the lane that holds it
-        const int ro = kp >> 5, lo = kp & 31;
-#pragma unroll
-        for (int c = 0; c < WC; ++c) {
-            T src = y[0][c];
-#pragma unroll
-            for (int r = 1; r < RPL; ++r)
-                if (ro == r) src = y[r][c];
-            v[c] = __shfl_sync(0xffffffffu, src, lo);
-        }
-    };
-    T cf[RPL], cfn[RPL], v[WC];
-    // forward: rows k > kp
-    if (j0 + 1 < m) coef(j0, cf);
-    for (int kp = j0; kp + 1 < m; ++kp) {
-        if (kp + 2 < m) coef(kp + 1, cfn);
-        bcast(kp, v);
-#pragma unroll
-        for (int r = 0; r < RPL; ++r) {
-            const int k = lane + 32 * r;
-            if (k > kp && k < m) {
-#pragma unroll
-                for (int c = 0; c < WC; ++c) y[r][c] -= cf[r] * v[c];
-            }
-        }
-#pragma unroll
-        for (int r = 0; r < RPL; ++r) cf[r] = cfn[r];
-    }
-    // backward: rows k < kp
-    if (m >= 2) coef(m - 1, cf);
-    for (int kp = m - 1; kp >= 1; --kp) {
-        if (kp >= 2) coef(kp - 1, cfn);
-        bcast(kp, v);
-#pragma unroll
-        for (int r = 0; r < RPL; ++r) {
-            const int k = lane + 32 * r;
-            if (k < kp) {
-#pragma unroll
-                for (int c = 0; c < WC; ++c) y[r][c] -= cf[r] * v[c];
-            }
-        }
-#pragma unroll
-        for (int r = 0; r < RPL; ++r) cf[r] = cfn[r];
-    }
-    T* Wd = Wx + (size_t)s * NW * NW;
-#pragma unroll
-    for (int r = 0; r < RPL; ++r) {
-        const int k = lane + 32 * r;
-        if (k < m) {
-            const T fkk = -fk[s][k];
-#pragma unroll
-            for (int c = 0; c < WC; ++c)
-                if (j0 + c < m) Wd[k * NW + j0 + c] = fkk * y[r][c];
+    for (int row = tid >> 5; row < 2 * m; row += WIN_THREADS / 32) {
+        const int s = row >= m ? 1 : 0, k = row - s * m, a = idx[k];
+        const T* Gb = Gs + (size_t)s * n * P;
+        const T nf = -fk[s][k];
+        const size_t o = ((size_t)s * NW + k) * NW;
+        for (int c = a + (tid & 31); c < n; c += 32) {
+            Wx[o + c] = c == a ? nf : Gb[a * P + c];
+            Wm[o + c] = c == a ? nf : nf * Gb[c * P + a];
         }
     }
 }
 
-// Cc[s][k][k'] = C[k][k'] f_k' in place over the block: every element of the accepted rows and columns
-// is read (RU x CU registers a thread; warps over rows, lanes over columns) before any is written.  The
-// block itself is not needed any more.
-template <typename T, int RU, int CU>
-__device__ __forceinline__ void window_compact(T* Gs, int n, int P, const int* idx, const T (*fk)[WinCap<T>::NW],
-                                               int m, int tid) {
-    const int lane = tid & 31, w = tid >> 5;
-    T v[RU][CU];
-#pragma unroll
-    for (int a = 0; a < RU; ++a) {
-        const int row = w + 32 * a, s = row >= m ? 1 : 0, k = row - s * m;
-#pragma unroll
-        for (int c = 0; c < CU; ++c) {
-            const int kp = lane + 32 * c;
-            if (k < m && kp < m) v[a][c] = Gs[(s * n + idx[k]) * P + idx[kp]] * fk[s][kp];
-        }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int a = 0; a < RU; ++a) {
-        const int row = w + 32 * a, s = row >= m ? 1 : 0, k = row - s * m;
-#pragma unroll
-        for (int c = 0; c < CU; ++c) {
-            const int kp = lane + 32 * c;
-            if (k < m && kp < m) Gs[(s * n + k) * P + kp] = v[a][c];
-        }
-    }
-    __syncthreads();
-}
-
+// Field-change constants in the bulk precision (SiteParams holds them in FP64).
 template <typename T>
-__device__ __forceinline__ void window_w(T* Gs, int n, int P, const int* idx, const T (*fk)[WinCap<T>::NW], int m,
-                                         T* Wx, int tid) {
-    constexpr bool BIG = WinCap<T>::NW > 64;
-    const int lane = tid & 31, w = tid >> 5;
-    if (m <= 64) window_compact<T, 4, 2>(Gs, n, P, idx, fk, m, tid);
-    else window_compact<T, WinCap<T>::NW / 16, WinCap<T>::NW / 32>(Gs, n, P, idx, fk, m, tid);
-    if (m <= 16) window_w_rpl<T, 1, 1>(Gs, n, P, fk, m, Wx, lane, w);
-    else if (m <= 32) window_w_rpl<T, 1, 2>(Gs, n, P, fk, m, Wx, lane, w);
-    else if (m <= 48) window_w_rpl<T, 2, 3>(Gs, n, P, fk, m, Wx, lane, w);
-    else if (m <= 64) window_w_rpl<T, 2, 4>(Gs, n, P, fk, m, Wx, lane, w);
-    else if (BIG && m <= 96) window_w_rpl<T, BIG ? 3 : 2, BIG ? 6 : 4>(Gs, n, P, fk, m, Wx, lane, w);
-    else window_w_rpl<T, BIG ? 4 : 2, BIG ? 8 : 4>(Gs, n, P, fk, m, Wx, lane, w);
-}
-
-// What warp 0 carries through a window's decisions (the same in every lane).
-template <typename T>
-struct WinScan {
-    int m = 0;        // accepts so far
-    int nneg = 0;     // accepted negative ratios (sign parity)
-    T maxr = T(0);    // largest |R| of an accept
-    bool alive = true;  // constrained path: the walker has not been removed
-    bool bad = false;   // a non-finite ratio was met
-    int done = 0;       // sites decided
+struct FlipConsts {
+    T dflip[2][2], sflip[2];
 };
 
-// The decisions of the sites [b0, b0 + nbk) of the window, one warp for both spins: lane
-// 16 s + r CG + cg holds row r, columns j CG + cg of spin s's sub-block in registers (CG = 16 / B), so
-// a site costs its ratio (one shuffle for the diagonal, one to pair the spins) and an accept B shuffles
-// of its row and as many multiply-adds, with no barrier.  Every lane takes the decision redundantly.
-// An accept a updates the rows and columns after a only, with the products
-// G[r][c] += (Delta/r G[r][a]) G[a][c] (f = -Delta/r) in accept order; row a and column a keep their values of that moment (the frozen coefficients).
-//   Metropolis (AFQMC_MODE_DELAYED): R = s(-x)/s(x) r_up r_dn, r_s = 1 + Delta_s (1 - G_s[q][q]).
-//   Constrained-path heat bath (WIN_MODE_CP, Sec. IV.D, Eq. ptilde): lambda(x) = p(x) s(x) r_up(x) r_dn(x),
-//   negative lambda clamped to zero, x = +1 iff u (lambda(+1) + lambda(-1)) < lambda(+1); the walker is
-//   removed when both vanish; every site is an accept.
-template <typename T, int MODE>
-__device__ __forceinline__ void window_sub_sites(T* Gs, int n, int P, int b0, int nbk, const int8_t* xw, const T* s_u,
-                                                 const uint8_t* s_rep, bool forced, const T (*dflip)[2],
-                                                 const T* sflip, T* s_rat, T* s_det, uint8_t* s_dec, int8_t* s_xch,
-                                                 T (*s_fk)[WinCap<T>::NW], int* idx, WinScan<T>& sc, int lane) {
-    constexpr int B = WinSub<T>::B, CG = 16 / B, CW = B / CG;
-    constexpr unsigned FULL = 0xffffffffu;
-    const int s = lane >> 4, r = (lane & 15) / CG, cg = lane % CG, half = lane & 16;
-    T g[CW];  // columns q0 + j CG + cg of row r, q0 the site the loop is at
+// t[k] by a tree of selects: indexing would move the array out of the registers.
+template <typename T, int R>
+__device__ __forceinline__ T reg_pick(T (&t)[R], int k) {
 #pragma unroll
-    for (int j = 0; j < CW; ++j) {
-        const int c = j * CG + cg;
-        g[j] = (r < nbk && c < nbk) ? Gs[(s * n + b0 + r) * P + b0 + c] : T(0);
-    }
-    T* col = Gs + (size_t)(s * n + b0 + (r < nbk ? r : 0)) * P + b0 + cg;
-    const int ls = lane < nbk ? lane : 0;  // lane l < nbk keeps the inputs and outputs of site l
-    const T u_l = s_u[b0 + ls];
-    const int x_l = xw[b0 + ls], rep_l = s_rep[b0 + ls];
-    const T d0 = dflip[s][0], d1 = dflip[s][1], sf0 = sflip[0], sf1 = sflip[1];
-    unsigned mask = 0, plus = 0;
-    T rat_l = T(0), det_l = T(0), f_l = T(0);
-    const int m0 = sc.m;
-#pragma unroll 1
-    for (int q0 = 0; q0 < nbk && sc.alive; q0 += CG) {
+    for (int w = R / 2; w >= 1; w /= 2)
 #pragma unroll
-        for (int t = 0; t < CG; ++t) {  // the current column sits in g[0] of the lanes cg == t
-            const int q = q0 + t, src = half + q * CG;
-            if (t > 0 && (q >= nbk || !sc.alive)) break;
-            const T a = T(1) - __shfl_sync(FULL, g[0], src + t);
-            const T u = __shfl_sync(FULL, u_l, q);
-            const bool rep = __shfl_sync(FULL, rep_l, q) != 0;
-            bool acc;
-            T f;
-            if (MODE == WIN_MODE_CP) {
-                const T rp = T(1) + d0 * a, rm = T(1) + d1 * a;
-                const T rpo = __shfl_xor_sync(FULL, rp, 16), rmo = __shfl_xor_sync(FULL, rm, 16);
-                const T lp = fmax(sf0 * (s ? rpo : rp) * (s ? rp : rpo), T(0));
-                const T lm = fmax(sf1 * (s ? rmo : rm) * (s ? rm : rmo), T(0));
-                const T nrm = lp + lm;
-                acc = nrm > T(0) && isfinite(nrm);
-                if (!acc) {
-                    sc.alive = false;
-                    if (!isfinite(nrm)) sc.bad = true;
-                }
-                const bool up = forced ? rep : u * nrm < lp;
-                f = -((up ? d0 : d1) / (up ? rp : rm));
-                if (acc && up) plus |= 1u << q;
-                if (lane == q) {
-                    rat_l = nrm;
-                    det_l = up ? rp * rpo : rm * rmo;
-                }
-            } else {
-                const int xi = __shfl_sync(FULL, x_l, q) > 0 ? 0 : 1;
-                const T dl = xi ? d1 : d0;
-                const T rr = T(1) + dl * a, ro = __shfl_xor_sync(FULL, rr, 16);
-                const T R = (xi ? sf1 : sf0) * (s ? ro : rr) * (s ? rr : ro);
-                acc = forced ? rep : u < fabs(R);
-                if (!isfinite(R)) {
-                    acc = false;
-                    sc.bad = true;
-                }
-                f = -(dl / rr);
-                if (lane == q) rat_l = R;
-                if (acc) {
-                    if (R < T(0)) ++sc.nneg;
-                    sc.maxr = fmax(sc.maxr, fabs(R));
-                }
-            }
-            ++sc.done;
-            if (acc) {
-                mask |= 1u << q;
-                if ((lane & 15) == q) f_l = f;
-                const T fc = -f * (CG == 1 ? g[0] : __shfl_sync(FULL, g[0], half + r * CG + t));
-#pragma unroll
-                for (int j = t == CG - 1 ? 1 : 0; j < CW; ++j) {
-                    const T rv = __shfl_sync(FULL, g[j], src + cg);
-                    if (r > q && (j > 0 || cg > t)) g[j] = fma(fc, rv, g[j]);
-                }
-            }
-        }
-        if (r < nbk && q0 + cg < nbk) col[q0] = g[0];  // these columns are never written again
-#pragma unroll
-        for (int j = 0; j + 1 < CW; ++j) g[j] = g[j + 1];
-    }
-    sc.m = m0 + __popc(mask);
-    if (lane < nbk) {
-        s_dec[b0 + lane] = MODE == WIN_MODE_CP ? (plus >> lane) & 1u : (mask >> lane) & 1u;
-        s_rat[b0 + lane] = rat_l;
-        if (MODE == WIN_MODE_CP) s_det[b0 + lane] = det_l;
-    }
-    if ((mask >> (lane & 15)) & 1u) {
-        const int k = m0 + __popc(mask & ((1u << (lane & 15)) - 1u));
-        s_fk[s][k] = f_l;
-        if (s == 0) {
-            idx[k] = b0 + lane;
-            if (MODE == WIN_MODE_CP) s_xch[k] = (plus >> lane) & 1u ? 1 : -1;
-        }
-    }
+        for (int i = 0; i < w; ++i) t[i] = (k & w) ? t[i + w] : t[i];
+    return t[0];
 }
 
-// The accepts k = 0 .. mk - 1 of the sub-block that ends before site b1 (sites ia[k], factors fa[s][k])
-// applied to the rows and columns [b1, n) of both spins, all threads of the block:
-//   1. the coefficient triangles of the sub-block, shifted to start after the diagonal:
-//      D[0][s][k'][j] = G[a_k'][a_k] and D[1][s][k'][j] = -f_k' G[a_k][a_k'], k = k' + 1 + j (f = -Delta/r);
-//   2. one thread per row (or column) of the panels: column a_k of the rows after the sub-block, and
-//      row a_k of the columns after it, as they stood when a_k was accepted, by the recursion over the
-//      earlier accepts; stored in place (the frozen coefficients) and as pw[s][r][k] = -f_k G[r][a_k],
-//      qv[s][k][c] = G[a_k][c], zero-padded to whole 16-byte vectors;
-//   3. G[r][c] += sum_k pw qv, in accept order, one column and a few rows a thread.
-// The arithmetic is that of one trailing rank-1 update per accept, in the same order.
-template <typename T>
-__device__ __forceinline__ void window_sub_update(T* Gs, int n, int P, int b1, int mk, const int* ia, const T* fu,
-                                                  const T* fd, T* D, T* pw, T* qv, int tid, int nt) {
-    constexpr int B = WinSub<T>::B, VW = Vec16<T>::W;
-    using V = typename Vec16<T>::V;
-    const int rem = n - b1;
-    for (int e = tid; e < 4 * B * B; e += nt) {
-        const int j = e % B, kp = (e / B) % B, s = (e / (B * B)) & 1, kind = e / (2 * B * B), k = kp + 1 + j;
-        T v = T(0);
-        if (k < mk) {
-            const T* Gb = Gs + (size_t)s * n * P;
-            v = kind ? -(s ? fd : fu)[kp] * Gb[ia[k] * P + ia[kp]] : Gb[ia[kp] * P + ia[k]];
-        }
-        D[e] = v;
-    }
-    __syncthreads();
-    for (int e = tid; e < 4 * rem; e += nt) {
-        const int kind = e >= 2 * rem ? 1 : 0, e2 = e - kind * 2 * rem, s = e2 >= rem ? 1 : 0, i = e2 - s * rem;
-        T* line = Gs + (size_t)s * n * P + (kind ? b1 + i : (b1 + i) * P);
-        const int step = kind ? P : 1;
-        const T* Dm = D + (kind * 2 + s) * B * B;
-        const T* f = s ? fd : fu;
-        T* out = kind ? qv + s * B * n + i : pw + (s * n + i) * B;
-        const int ostep = kind ? n : 1;
-        T v[B];  // v[j]: entry kp + j of the line, kp the accept the loop is at
+// x / y for the accept factor.  FP32: the approximate reciprocal of the device and one step of residual
+// correction (q += (x - q y) / y), straight-line code that overlaps the block's update.  FP64: a 22-bit
+// reciprocal of y's leading bits, taken in FP32 from its bit pattern, and one step of Halley's iteration
+// (1/y = s (1 + e + e^2 + ...), e = 1 - s y, error e^3 < 2^-63): four dependent FP64 operations, where each
+// costs about 100 cycles and a full division about 740.  Outside the FP32 exponent range: the division.
+__device__ __forceinline__ float accept_quot(float x, float y) {
+    const float rc = __fdividef(1.0f, y), q = x * rc;
+    return fmaf(fmaf(-q, y, x), rc, q);
+}
+__device__ __forceinline__ double accept_quot(double x, double y) {
+    const unsigned hi = (unsigned)__double2hiint(y), lo = (unsigned)__double2loint(y);
+    const int ex = (int)((hi >> 20) & 0x7ffu) - 1023;
+    if (ex < -100 || ex > 100) return x / y;
+    // y = +-1.m 2^ex: the float 1.m (23 bits), its reciprocal in (0.5, 1], back with exponent -ex
+    const float ym = __uint_as_float(0x3f800000u | ((hi & 0xfffffu) << 3) | (lo >> 29));
+    const unsigned rb = __float_as_uint(__fdividef(1.0f, ym));
+    const int re = (int)((rb >> 23) & 0xffu) - 127 - ex + 1023;
+    const double sd = __hiloint2double((int)((hi & 0x80000000u) | ((unsigned)re << 20) | ((rb & 0x7fffffu) >> 3)),
+                                       (int)(rb << 29));
+    const double e = fma(-y, sd, 1.0);
+    return x * fma(sd, fma(e, e, e), sd);
+}
+
+// Warps and register tile of window_reg_kernel for windows of up to NP sites.  Warp 0 decides, TW tile warps
+// hold the block (RG row groups x 8 column groups of threads per spin, a thread rows rg + RG i and columns
+// cg + 8 j), one warp exports the accepts.  Up to 64 sites warps 4, 8, ... exit at once, so the deciding
+// warp has its SM partition to itself (with 128 sites their registers are needed).
+template <typename T, int NP>
+struct WinTile {
+    static constexpr int TW = 8, WPS = TW / 2;
+    static constexpr int RG = 4 * WPS, TR = NP / RG, TC = NP / 8, NJ = NP / 32;
+    static constexpr bool IDLE = NP <= 64;
+    static constexpr int ACTIVE = 32 * (TW + 2);                              // threads at the barriers
+    static constexpr int THREADS = ACTIVE + (IDLE ? 32 * ((TW + 1) / 3) : 0);  // with the exiting warps
+};
+
+// One window of the delayed update (AFQMC_MODE_DELAYED) or of the constrained-path heat bath
+// (WIN_MODE_CP), one block per walker.
+//
+// The n x n block of both spins (n <= NP) lives in the registers of the tile warps.  Per accept a, two
+// barriers: the deciding warp names a; the threads that hold row a and column a put them into shared memory
+// (double-buffered by accept parity); every tile thread applies G[r][c] += (-f G[r][a]) G[a][c] to its
+// elements while the deciding warp goes on from the same two vectors and the export warp writes them out for
+// panel_kernel.  Rows and columns at or before a are never looked at again.
+//
+// Decisions: lane l keeps 1 - G[q][q] of both spins, the uniform, the field and the ratio of the sites
+// q = l + 32 j, and tests 32 sites at a time; a ballot finds the next accept (a rejection leaves G unchanged).
+//   Metropolis: R = s(-x)/s(x) r_up r_dn, r_s = 1 + Delta_s (1 - G_s[q][q]), accept iff u < |R|.
+//   Constrained-path heat bath (Sec. IV.D, Eq. ptilde): lambda(x) = p(x) s(x) r_up(x) r_dn(x), negative
+//   lambda clamped to zero, x = +1 iff u (lambda(+1) + lambda(-1)) < lambda(+1); the walker is removed when
+//   both vanish; every site is an accept.
+//
+// Bound by the latency of the accept chain, one warp's instruction stream: roles are split over warps so
+// that each has little to issue per accept.
+template <typename T, int MODE, int NP>
+__global__ void __launch_bounds__(WinTile<T, NP>::THREADS) window_reg_kernel(
+    const T* __restrict__ Gu0, int8_t* xl0, const double* __restrict__ u0, const uint8_t* __restrict__ replay0,
+    int N, long ld, FlipConsts<T> fc, SliceOut so0, int s0, int n, WindowBufs wb0, const T* __restrict__ blk0,
+    int* err, Batch bt) {
+    using W = WinTile<T, NP>;
+    constexpr int NW = WinCap<T>::NW, RG = W::RG, TR = W::TR, TC = W::TC, NJ = W::NJ;
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, hw = __shfl_sync(FULL, threadIdx.x >> 5, 0), wk = blockIdx.x;
+    if (W::IDLE && hw > 0 && (hw & 3) == 0) return;
+    const int warp = W::IDLE ? hw - 1 - hw / 4 : hw - 1;  // -1: decides, < TW: tile, TW: export
+    auto block_sync = [&] {
+        __syncwarp();  // the barrier counts whole warps
+        named_barrier_sync(1, W::ACTIVE);
+    };
+    const WindowBufs wb = wb_walker<T>(wb0, wk, N);
+    const T* G = Gu0 + (size_t)wk * bt.gstride;
+    const T* src0 = blk0 ? blk0 + (size_t)wk * 2 * NW * NW : G + (size_t)s0 * ld + s0;  // the block, spin up
+    const T* src1 = blk0 ? src0 + NW * NW : src0 + (size_t)N * ld;
+    const long lds = blk0 ? NW : ld;
+    __shared__ T srow[2][2][NP], scol[2][2][NP];  // [accept parity][spin]: G[a][:], G[:, a]
+    __shared__ T s_f[2][2];                       // [accept parity][spin]: f = -Delta / r
+    __shared__ int s_a[2];                        // [accept parity]: the accept, -1 at the end
+
+    if (warp >= 0 && warp < W::TW) {  // ---- tile warps ----
+        const int s = warp >= W::WPS ? 1 : 0, rg = (warp - s * W::WPS) * 4 + (lane >> 3), cg = lane & 7;
+        const T* sp = s ? src1 : src0;
+        T g[TR][TC];
 #pragma unroll
-        for (int k = 0; k < B; ++k) v[k] = k < mk ? line[ia[k] * step] : T(0);
-#pragma unroll 1
-        for (int kp = 0; kp < mk; ++kp) {
-            const T w = kind ? v[0] : -f[kp] * v[0];
-            line[ia[kp] * step] = v[0];
-            out[kp * ostep] = w;
+        for (int i = 0; i < TR; ++i)
 #pragma unroll
-            for (int j0 = 0; j0 < B; j0 += VW) {
-                T d[VW];
-                *(V*)d = *(const V*)(Dm + kp * B + j0);
-#pragma unroll
-                for (int l = 0; l < VW; ++l)
-                    if (j0 + l + 1 < B) v[j0 + l] = fma(w, d[l], v[j0 + l + 1]);
+            for (int j = 0; j < TC; ++j) {
+                const int r = rg + RG * i, c = cg + 8 * j;
+                g[i][j] = (r < n && c < n) ? sp[r * lds + c] : T(0);
             }
-        }
-        for (int kp = mk; kp < (mk + VW - 1) / VW * VW; ++kp) out[kp * ostep] = T(0);
-    }
-    __syncthreads();
-    const int rt = (2 * rem * rem + nt - 1) / nt, ngr = (rem + rt - 1) / rt, tot = 2 * rem * ngr;
-    for (int e = tid; e < tot; e += nt) {
-        const int s = e >= rem * ngr ? 1 : 0, e2 = e - s * rem * ngr, rg = e2 / rem, c = e2 - rg * rem;
-        T q[B];
+        for (int par = 0;; par ^= 1) {
+            block_sync();
+            const int a = s_a[par];
+            if (a < 0) return;
+            if (rg == (a & (RG - 1))) {
 #pragma unroll
-        for (int k0 = 0; k0 < B; k0 += VW)
+                for (int j = 0; j < TC; ++j) {
+                    T t[TR];
 #pragma unroll
-            for (int l = 0; l < VW; ++l) q[k0 + l] = k0 < mk ? qv[(s * B + k0 + l) * n + c] : T(0);
-        const int rlo = rg * rt, rhi = min(rem, rlo + rt);
-        T* out = Gs + ((size_t)s * n + b1 + rlo) * P + b1 + c;
-        const T* pr = pw + (size_t)(s * n + rlo) * B;
-        for (int r = rlo; r < rhi; ++r, out += P, pr += B) {
-            T acc = *out;
-#pragma unroll
-            for (int k0 = 0; k0 < B; k0 += VW) {
-                if (k0 < mk) {
-                    T w[VW];
-                    *(V*)w = *(const V*)(pr + k0);
-#pragma unroll
-                    for (int l = 0; l < VW; ++l) acc = fma(w[l], q[k0 + l], acc);
+                    for (int i = 0; i < TR; ++i) t[i] = g[i][j];
+                    srow[par][s][cg + 8 * j] = reg_pick<T, TR>(t, a / RG);
                 }
             }
-            *out = acc;
+            if (cg == (a & 7)) {
+#pragma unroll
+                for (int i = 0; i < TR; ++i) {
+                    T t[TC];
+#pragma unroll
+                    for (int j = 0; j < TC; ++j) t[j] = g[i][j];
+                    scol[par][s][rg + RG * i] = reg_pick<T, TC>(t, a >> 3);
+                }
+            }
+            block_sync();
+            const T nf = -s_f[par][s];
+            T rv[TC];
+#pragma unroll
+            for (int j = 0; j < TC; ++j) rv[j] = srow[par][s][cg + 8 * j];
+#pragma unroll
+            for (int i = 0; i < TR; ++i) {
+                // an FP64 or 128-site update is bound by its multiply-adds: rows (and columns) at or before
+                // a in every thread are left out
+                if ((sizeof(T) == 8 || NP > 64) && RG * i + RG - 1 <= a) continue;
+                const T wv = nf * scol[par][s][rg + RG * i];
+#pragma unroll
+                for (int j = 0; j < TC; ++j) {
+                    if (sizeof(T) == 8 && 8 * j + 7 <= a) continue;
+                    g[i][j] = fma(wv, rv[j], g[i][j]);
+                }
+            }
         }
     }
-    __syncthreads();
+    if (warp == W::TW) {  // ---- export warp: row a and -f column a of accept m, -f at position a ----
+        for (int m = 0;; ++m) {
+            const int par = m & 1;
+            block_sync();
+            const int a = s_a[par];
+            if (a < 0) return;
+            block_sync();
+            if (lane == 0) wb.idx[m] = s0 + a;
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                const T nf = -s_f[par][s];
+                T* wx = (T*)wb.Wx + ((size_t)s * NW + m) * NW;
+                T* wm = (T*)wb.Wm + ((size_t)s * NW + m) * NW;
+#pragma unroll
+                for (int j = 0; j < NJ; ++j) {
+                    const int q = lane + 32 * j;
+                    wx[q] = q == a ? nf : srow[par][s][q];
+                    wm[q] = q == a ? nf : nf * scol[par][s][q];
+                }
+            }
+        }
+    }
+    // ---- deciding warp ----
+    int8_t* xl = xl0 + (size_t)wk * bt.xstride + s0;
+    const double* u = u0 + (size_t)wk * 2 * N + s0;
+    const uint8_t* rep = replay0 ? replay0 + (size_t)wk * 2 * N + s0 : nullptr;
+    const SliceOut so = so_walker(so0, wk, N);
+    const bool forced = rep != nullptr;
+    T b0[NJ], b1[NJ], ul[NJ], rat[NJ], det[NJ];  // 1 - G[q][q] up and down, uniform, ratio (norm), r_up r_dn
+    int xs[NJ];
+    unsigned repm[NJ], accm[NJ], upm[NJ], valid[NJ];  // lane masks: forced, accepted, x = +1 drawn, q < n
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+        const int q = lane + 32 * j;
+        const bool in = q < n;
+        b0[j] = in ? T(1) - src0[q * lds + q] : T(0);
+        b1[j] = in ? T(1) - src1[q * lds + q] : T(0);
+        ul[j] = in ? (T)u[q] : T(0);
+        xs[j] = in ? xl[q] : 1;
+        valid[j] = __ballot_sync(FULL, in);
+        repm[j] = __ballot_sync(FULL, in && forced && rep[q] != 0);
+        accm[j] = upm[j] = 0u;
+        rat[j] = det[j] = T(0);
+    }
+    bool dead = MODE == WIN_MODE_CP && so.cp && so.cp[2] != 0.0;
+    int m = 0;
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+        // field-change constants of this chunk's sites (Metropolis)
+        const bool xp = xs[j] > 0;
+        const T x0 = xp ? fc.dflip[0][0] : fc.dflip[0][1], x1 = xp ? fc.dflip[1][0] : fc.dflip[1][1];
+        const T sf = xp ? fc.sflip[0] : fc.sflip[1];
+        unsigned open = dead ? 0u : valid[j];  // sites of the chunk not decided yet
+        while (open) {
+            T e0 = x0, e1 = x1, r0, r1, R;
+            unsigned ball;
+            if (MODE == WIN_MODE_CP) {
+                const T p0 = T(1) + fc.dflip[0][0] * b0[j], p1 = T(1) + fc.dflip[1][0] * b1[j];
+                const T m0 = T(1) + fc.dflip[0][1] * b0[j], m1 = T(1) + fc.dflip[1][1] * b1[j];
+                const T lp = fmax(fc.sflip[0] * p0 * p1, T(0)), lm = fmax(fc.sflip[1] * m0 * m1, T(0));
+                R = lp + lm;
+                const bool up = forced ? ((repm[j] >> lane) & 1u) != 0 : ul[j] * R < lp;
+                r0 = up ? p0 : m0;
+                r1 = up ? p1 : m1;
+                e0 = up ? fc.dflip[0][0] : fc.dflip[0][1];
+                e1 = up ? fc.dflip[1][0] : fc.dflip[1][1];
+                const unsigned site = open & (0u - open);  // one site at a time
+                ball = __ballot_sync(FULL, R > T(0) && isfinite(R)) & site;
+                upm[j] |= __ballot_sync(FULL, up) & ball;
+                if ((site >> lane) & 1u) {
+                    rat[j] = R;
+                    det[j] = r0 * r1;
+                }
+                if (!ball) {
+                    dead = true;
+                    break;
+                }
+            } else {
+                r0 = T(1) + e0 * b0[j];
+                r1 = T(1) + e1 * b1[j];
+                R = sf * r0 * r1;
+                const unsigned yes = __ballot_sync(FULL, ul[j] < fabs(R) && isfinite(R));
+                ball = (forced ? repm[j] : yes) & open;
+            }
+            // sites before the first accept are rejected; it and they are decided now
+            const unsigned bit = ball & (0u - ball), done = ball ? open & (bit | (bit - 1u)) : open;
+            if (MODE != WIN_MODE_CP && ((done >> lane) & 1u)) rat[j] = R;
+            open &= ~done;
+            if (!ball) break;
+            accm[j] |= bit;
+            const int first = __ffs(ball) - 1, par = m & 1;
+            T f0, f1;
+            if (sizeof(T) == 4) {  // every lane's factors, under the ballot's latency
+                const T q0 = -accept_quot(e0, r0), q1 = -accept_quot(e1, r1);
+                if (lane == first) {
+                    s_a[par] = 32 * j + first;
+                    s_f[par][0] = q0;
+                    s_f[par][1] = q1;
+                }
+                block_sync();
+                f0 = __shfl_sync(FULL, q0, first);
+                f1 = __shfl_sync(FULL, q1, first);
+            } else {  // one quotient for both spins while the tile warps store: even lanes up, odd lanes down
+                if (lane == 0) s_a[par] = 32 * j + first;
+                block_sync();
+                const T n0 = __shfl_sync(FULL, e0, first), n1 = __shfl_sync(FULL, e1, first);
+                const T d0 = __shfl_sync(FULL, r0, first), d1 = __shfl_sync(FULL, r1, first);
+                const T fq = -accept_quot((lane & 1) ? n1 : n0, (lane & 1) ? d1 : d0);
+                if (lane < 2) s_f[par][lane] = fq;
+                f0 = __shfl_sync(FULL, fq, 0);
+                f1 = __shfl_sync(FULL, fq, 1);
+            }
+            block_sync();
+#pragma unroll
+            for (int i = j; i < NJ; ++i) {
+                const int q = lane + 32 * i;
+                b0[i] = fma(f0 * scol[par][0][q], srow[par][0][q], b0[i]);
+                b1[i] = fma(f1 * scol[par][1][q], srow[par][1][q], b1[i]);
+            }
+            ++m;
+        }
+    }
+    if (lane == 0) s_a[m & 1] = -1;
+    block_sync();
+    // decisions, ratios, fields and the walker's sums
+    double c0 = 0.0, c1 = 0.0;
+    int nneg = 0;
+    T maxr = T(0);
+    bool bad = false;
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+        const int q = lane + 32 * j;
+        const bool acc = ((accm[j] >> lane) & 1u) != 0, up = ((upm[j] >> lane) & 1u) != 0;
+        if (q < n) {
+            so.dec[s0 + q] = MODE == WIN_MODE_CP ? up : acc;
+            so.ratio[s0 + q] = (double)rat[j];
+            bad = bad || !isfinite(rat[j]);
+            if (acc) {
+                xl[q] = (int8_t)(MODE == WIN_MODE_CP ? (up ? 1 : -1) : -xs[j]);
+                if (MODE == WIN_MODE_CP) {
+                    c0 += log((double)rat[j]);
+                    c1 += log(fabs((double)det[j]));
+                } else {
+                    if (rat[j] < T(0)) ++nneg;
+                    maxr = fmax(maxr, fabs(rat[j]));
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        nneg += __shfl_xor_sync(FULL, nneg, o);
+        maxr = fmax(maxr, __shfl_xor_sync(FULL, maxr, o));
+        if (MODE == WIN_MODE_CP) {
+            c0 += __shfl_xor_sync(FULL, c0, o);
+            c1 += __shfl_xor_sync(FULL, c1, o);
+        }
+    }
+    bad = __any_sync(FULL, bad);
+    if (lane == 0) {
+        *wb.m = m;
+        if (bad) set_err(err, DEV_NUMERIC);
+        if (so.sign && (nneg & 1)) *so.sign = -*so.sign;
+        if (MODE == WIN_MODE_CP && so.cp) {
+            so.cp[0] += c0;
+            so.cp[1] += c1;
+            if (dead) so.cp[2] = 1.0;
+        }
+        so.stats[0] += n;
+        so.stats[1] += m;
+        so.stats[2] += m;
+        so.stats[3] += (m > 0) ? 1 : 0;
+        *so.maxr = fmax(*so.maxr, (double)maxr);
+    }
 }
 
 template <typename T, int MODE>
@@ -730,12 +736,7 @@ __global__ void __launch_bounds__(WIN_THREADS) window_kernel(const T* __restrict
     const WindowBufs wb = wb_walker<T>(wb0, wk, N);
     const T* blk = blk0 ? blk0 + (size_t)wk * 2 * WinCap<T>::NW * WinCap<T>::NW : nullptr;
     T* Gs = (T*)smem_raw;  // [2][n][P]
-    size_t off = 2 * (size_t)n * P * sizeof(T);  // a multiple of 16: n (n + 1) is even
-    constexpr int SB = WinSub<T>::B;
-    T* Dsub = (T*)(smem_raw + off);    // [2][2][SB][SB] sub-block coefficients (window_sub_update)
-    T* pwsub = Dsub + 4 * SB * SB;     // [2][n][SB]
-    T* qvsub = pwsub + 2 * n * SB;     // [2][SB][n]
-    off += 4 * (size_t)SB * (SB + n) * sizeof(T);
+    size_t off = 2 * (size_t)n * P * sizeof(T);
     T* S1 = (T*)(smem_raw + off);  // [2][NBMAX][NBMAX+1]
     off += 2 * (size_t)NBMAX * (NBMAX + 1) * sizeof(T);
     T* stc = (T*)(smem_raw + off);  // staging: col[2][n], row[2][n]
@@ -778,17 +779,6 @@ __global__ void __launch_bounds__(WIN_THREADS) window_kernel(const T* __restrict
             }
     }
     for (int p = tid; p < n; p += nt) xw[p] = xl_g[s0 + p];
-    // the window's site uniforms (and forced decisions) live in shared memory: the scan reads
-    // them on its critical path
-    // (in the bulk precision: the delayed scan compares them with ratios computed in T)
-    __shared__ T s_u[WinCap<float>::NW];
-    __shared__ uint8_t s_rep[WinCap<float>::NW];
-    __shared__ T s_rat[WinCap<float>::NW];    // ratio of every decided site, written out after the decisions
-    __shared__ uint8_t s_dec[WinCap<float>::NW];
-    for (int p = tid; p < n; p += nt) {
-        s_u[p] = (T)u[s0 + p];
-        s_rep[p] = replay ? replay[s0 + p] : 0;
-    }
     __shared__ double c_dflip[2][2], c_dstrip[2][2], c_sflip[2];
     __shared__ T c_dflipT[2][2], c_sflipT[2];  // the same in T for the scan's critical path
     if (tid < 4) {
@@ -812,66 +802,13 @@ __global__ void __launch_bounds__(WIN_THREADS) window_kernel(const T* __restrict
     __shared__ int8_t s_xch[WinCap<float>::NW];  // constrained path: the field chosen at each site
     __shared__ double s_cpl[2];                  // constrained path: sum ln N_i, sum ln |r_up r_dn|
     __shared__ int s_dead;
-    if ((MODE == WIN_MODE_CP || MODE == WIN_MODE_CPB) && tid == 0) {
+    if (MODE == WIN_MODE_CPB && tid == 0) {
         s_cpl[0] = 0.0;
         s_cpl[1] = 0.0;
         s_dead = so.cp ? (so.cp[2] != 0.0) : 0;
     }
     __syncthreads();
-    if (MODE == AFQMC_MODE_DELAYED || MODE == WIN_MODE_CP) {
-        // Two levels: warp 0 decides a sub-block of SB sites in registers (no barrier per accept), then
-        // all warps bring the rest of the window's block up to date with the sub-block's accepts.
-        __shared__ int s_mk[2];
-        __shared__ T s_det[WinCap<float>::NW];  // constrained path: r_up r_dn of every site
-        WinScan<T> sc;
-        sc.alive = !((MODE == WIN_MODE_CP) && s_dead);
-        int m_all = 0;
-        for (int b0 = 0, it = 0; b0 < n; b0 += SB, ++it) {
-            const int b1 = min(n, b0 + SB);
-            if (tid < 32) {
-                window_sub_sites<T, MODE>(Gs, n, P, b0, b1 - b0, xw, s_u, s_rep, replay != nullptr, c_dflipT,
-                                          c_sflipT, s_rat, s_det, s_dec, s_xch, s_fk, idx, sc, tid);
-                if (tid == 0) s_mk[it & 1] = sc.m;
-            }
-            __syncthreads();
-            const int mk = s_mk[it & 1] - m_all;
-            if (mk > 0 && b1 < n)
-                window_sub_update<T>(Gs, n, P, b1, mk, idx + m_all, s_fk[0] + m_all, s_fk[1] + m_all, Dsub, pwsub,
-                                     qvsub, tid, nt);
-            m_all += mk;
-        }
-        if (tid == 0) {
-            s_m = sc.m;
-            if (sc.bad) set_err(err, DEV_NUMERIC);
-            if (sc.nneg & 1) s_sign = -s_sign;
-            s_maxr = fmax(s_maxr, (double)sc.maxr);
-            n_prop = sc.done;
-            n_acc = n_flip = sc.m;
-            if (MODE == WIN_MODE_CP && !sc.alive) s_dead = 1;
-        }
-        __syncthreads();
-        // decisions and ratios in their ABI types; the walker's weight factors as sums over its sites
-        for (int q = tid; q < n; q += nt) {
-            so.dec[s0 + q] = s_dec[q];
-            so.ratio[s0 + q] = (double)s_rat[q];
-        }
-        if (MODE == WIN_MODE_CP && tid < 32) {
-            double a0 = 0.0, a1 = 0.0;
-            for (int q = tid; q < s_m; q += 32) {
-                a0 += log((double)s_rat[idx[q]]);
-                a1 += log(fabs((double)s_det[idx[q]]));
-            }
-            for (int o = 16; o > 0; o >>= 1) {
-                a0 += __shfl_xor_sync(0xffffffffu, a0, o);
-                a1 += __shfl_xor_sync(0xffffffffu, a1, o);
-            }
-            if (tid == 0) {
-                s_cpl[0] = a0;
-                s_cpl[1] = a1;
-            }
-        }
-        __syncthreads();
-    } else if (MODE == WIN_MODE_CPB) {
+    if (MODE == WIN_MODE_CPB) {
         // ---- constrained-path block force bias (Sec. IV.D) ----
         // Per block S of nb sites (no field set yet): the force bias F_i of the current block's
         // diagonal (spin channel sum_s c_s A_s[i][i], charge channel lam (A_up + A_dn - 1)[i][i]),
@@ -1114,11 +1051,7 @@ __global__ void __launch_bounds__(WIN_THREADS) window_kernel(const T* __restrict
     }
     __syncthreads();
     const int m = s_m;
-    if (MODE == AFQMC_MODE_DELAYED) {  // apply the accepted flips (deferred: xw[p] was read by every thread)
-        for (int q = tid; q < m; q += nt) xw[idx[q]] = (int8_t)(-xw[idx[q]]);
-        __syncthreads();
-    }
-    if (MODE == WIN_MODE_CP || MODE == WIN_MODE_CPB) {  // the chosen fields, and the walker's weight factors
+    if (MODE == WIN_MODE_CPB) {  // the chosen fields, and the walker's weight factors
         for (int q = tid; q < m; q += nt) xw[idx[q]] = s_xch[q];
         if (tid == 0 && so.cp) {
             so.cp[0] += s_cpl[0];
@@ -1129,17 +1062,8 @@ __global__ void __launch_bounds__(WIN_THREADS) window_kernel(const T* __restrict
     }
     for (int p = tid; p < n; p += nt) xl_g[s0 + p] = xw[p];
     for (int q = tid; q < m; q += nt) wb.idx[q] = s0 + idx[q];
-    // The window's update matrix W (Eq. DelayRgenk in G form).  With C[k][k'] = Gs[idx[k]][idx[k']]
-    // the block entries frozen at acceptance time (rows and columns at or before an accepted site
-    // are never touched again), f_k = -Delta_k / r_k, L1 = I + Cl F and U1 = I + Cu F (Cl, Cu the
-    // strictly lower / upper parts of C, F = diag f), the delayed-update recursions give
-    // W = -F U1^{-1} L1^{-1}: per column of the identity a forward and a backward substitution,
-    //   y_k = b_k - sum_{k'<k} C[k][k'] f_k' y_k',   z_k = y_k - sum_{k'>k} C[k][k'] f_k' z_k',
-    //   W_k = -f_k z_k.
-    // The coefficients are gathered into a dense m x m matrix first; then each warp owns a few columns
-    // of one spin in registers (lane l holds rows l, l + 32, ...) and broadcasts the finished row of
-    // every step with a shuffle: no block-wide barrier per step.
-    window_w<T>(Gs, n, P, idx, s_fk, m, (T*)wb.Wx, tid);
+    // The accepts' rows and columns, from which panel_kernel forms the window's update of all of G
+    window_export<T>(Gs, n, P, idx, s_fk, m, (T*)wb.Wx, (T*)wb.Wm, tid);
     if (tid == 0) {
         *wb.m = m;
         if (so.sign) *so.sign = s_sign;
@@ -1151,34 +1075,60 @@ __global__ void __launch_bounds__(WIN_THREADS) window_kernel(const T* __restrict
     }
 }
 
+template <typename T, int MODE, int NP>
+static cudaError_t launch_window_reg(cudaStream_t st, const T* Gu, int8_t* xl, const double* u, const uint8_t* replay,
+                                     const SiteParams& sp, SliceOut so, int s0, int n, WindowBufs wb, const T* blk,
+                                     int* err, Batch bt) {
+    FlipConsts<T> fc;
+    for (int xi = 0; xi < 2; ++xi) {
+        for (int s = 0; s < 2; ++s) fc.dflip[s][xi] = (T)sp.dflip[s][xi];
+        fc.sflip[xi] = (T)sp.sflip[xi];
+    }
+    count_launch();
+    window_reg_kernel<T, MODE, NP><<<bt.nwk, WinTile<T, NP>::THREADS, 0, st>>>(Gu, xl, u, replay, sp.N, sp.ld, fc, so, s0,
+                                                                               n, wb, blk, err, bt);
+    return cudaGetLastError();
+}
+
 template <typename T>
 cudaError_t launch_window_chain(cudaStream_t st, int mode, const T* Gu, const T* Gd, int8_t* xl,
                                 const double* u, const uint8_t* replay, const SiteParams& sp, SliceOut so,
                                 int s0, int n, int nb, WindowBufs wb, const T* blk, int* err, Batch bt) {
     (void)Gd;  // spin down follows spin up (N x ld) in every walker's G
-    size_t shm = window_smem<T>(n);
-    auto kfn = (mode == AFQMC_MODE_DELAYED) ? (const void*)window_kernel<T, AFQMC_MODE_DELAYED>
-               : (mode == WIN_MODE_CP)     ? (const void*)window_kernel<T, WIN_MODE_CP>
-               : (mode == WIN_MODE_CPB)    ? (const void*)window_kernel<T, WIN_MODE_CPB>
-                                            : (const void*)window_kernel<T, AFQMC_MODE_BLOCKFB>;
-    {
-        cudaError_t e = ensure_smem_attr(kfn, window_smem<T>(WinCap<T>::NW));
-        if (e != cudaSuccess) return e;
-    }
     if (bt.nwk < 1) bt.nwk = 1;
+    // one accept at a time: the register-tile kernel of the smallest tile that holds the window
+    if (mode == AFQMC_MODE_DELAYED) {
+        if (n <= 32)
+            return launch_window_reg<T, AFQMC_MODE_DELAYED, 32>(st, Gu, xl, u, replay, sp, so, s0, n, wb, blk, err, bt);
+        if (n <= 64)
+            return launch_window_reg<T, AFQMC_MODE_DELAYED, 64>(st, Gu, xl, u, replay, sp, so, s0, n, wb, blk, err, bt);
+        if constexpr (WinCap<T>::NW > 64)
+            return launch_window_reg<T, AFQMC_MODE_DELAYED, 128>(st, Gu, xl, u, replay, sp, so, s0, n, wb, blk, err,
+                                                                 bt);
+        return cudaErrorInvalidValue;
+    }
+    if constexpr (sizeof(T) == 8) {  // the constrained path runs in FP64 only
+        if (mode == WIN_MODE_CP) {
+            if (n <= 32)
+                return launch_window_reg<T, WIN_MODE_CP, 32>(st, Gu, xl, u, replay, sp, so, s0, n, wb, blk, err, bt);
+            return launch_window_reg<T, WIN_MODE_CP, 64>(st, Gu, xl, u, replay, sp, so, s0, n, wb, blk, err, bt);
+        }
+        if (mode == WIN_MODE_CPB) {
+            cudaError_t e = ensure_smem_attr((const void*)window_kernel<T, WIN_MODE_CPB>,
+                                             window_smem<T>(WinCap<T>::NW));
+            if (e != cudaSuccess) return e;
+            count_launch();
+            window_kernel<T, WIN_MODE_CPB><<<bt.nwk, WIN_THREADS, window_smem<T>(n), st>>>(
+                Gu, xl, u, replay, sp, so, s0, n, nb, wb, blk, err, bt);
+            return cudaGetLastError();
+        }
+    }
+    if (mode != AFQMC_MODE_BLOCKFB) return cudaErrorInvalidValue;
+    cudaError_t e = ensure_smem_attr((const void*)window_kernel<T, AFQMC_MODE_BLOCKFB>, window_smem<T>(WinCap<T>::NW));
+    if (e != cudaSuccess) return e;
     count_launch();
-    if (mode == AFQMC_MODE_DELAYED)
-        window_kernel<T, AFQMC_MODE_DELAYED><<<bt.nwk, WIN_THREADS, shm, st>>>(Gu, xl, u, replay, sp, so, s0, n, nb,
-                                                                              wb, blk, err, bt);
-    else if (mode == WIN_MODE_CP)
-        window_kernel<T, WIN_MODE_CP><<<bt.nwk, WIN_THREADS, shm, st>>>(Gu, xl, u, replay, sp, so, s0, n, nb, wb,
-                                                                       blk, err, bt);
-    else if (mode == WIN_MODE_CPB)
-        window_kernel<T, WIN_MODE_CPB><<<bt.nwk, WIN_THREADS, shm, st>>>(Gu, xl, u, replay, sp, so, s0, n, nb, wb,
-                                                                        blk, err, bt);
-    else
-        window_kernel<T, AFQMC_MODE_BLOCKFB><<<bt.nwk, WIN_THREADS, shm, st>>>(Gu, xl, u, replay, sp, so, s0, n, nb,
-                                                                              wb, blk, err, bt);
+    window_kernel<T, AFQMC_MODE_BLOCKFB><<<bt.nwk, WIN_THREADS, window_smem<T>(n), st>>>(
+        Gu, xl, u, replay, sp, so, s0, n, nb, wb, blk, err, bt);
     return cudaGetLastError();
 }
 
@@ -1247,159 +1197,279 @@ template cudaError_t launch_window_chain<double>(cudaStream_t, int, const double
 // ---------------------------------------------------------------------------
 // Pipelined flush of one window.
 //
-// The window kernel leaves W (m x m) in wb.Wm: the accumulated update of the window is
-// G <- G - X W Yraw with X = G[:, I] and Yraw = E_I^T - G[I, :] (I the accepted sites).
-//   * next_block_kernel (main stream, right after the window): the next window's n' x n' block
-//     of G as it will be after this window's update, from three small gathers of G and two
-//     small products in shared memory.  The next window starts from it at once.
-//   * launch_flush_panels + launch_flush_gemm (flush stream): the panel gathers, Y' = W Yraw
-//     and the rank-m product over all of G, overlapping the next window's decisions.
+// A window's accepts a_0, a_1, ... in order are the rank-1 updates G += w_k q_k with
+//   w_k[r] = -f_k (G[r][a_k] + sum_{k'<k} w_k'[r] C[k'][k]),
+//   q_k[c] = G[a_k][c] - delta_{c a_k} + sum_{k'<k} (-f_k' C[k][k']) q_k'[c],
+// G the matrix before the window and C[k][k'] = G[a_k][a_k'] as it was when the earlier of the two was
+// accepted (Wx, Wm of the window kernel): every row's w and every column's q is a short recursion of its
+// own, so no update matrix has to be formed on the decisions' critical path.
+//   * panel_kernel (main stream, right after the window): w -> X (N x NW), q -> Y (NW x N), and the next
+//     window's block of G as this window's update will leave it;
+//   * launch_flush_gemm (flush stream): the rank-m product G += X Y over all of G, overlapping the next
+//     window's decisions.
+// In the T form the raw columns and rows are those of V = T U_L[:, I] and -(U_R[I, :] T).
 // ---------------------------------------------------------------------------
-
-// snap[s][a][c] = G[sn + a][sn + c] - sum_k X[sn + a][k] Y'[k][sn + c], with X = G[:, I],
-// Y' = W Yraw and Yraw[l][sn + c] = -G[I_l][sn + c] (the next window's sites are not in I): the
-// block of the next window as it will be after this window's product.  Grid (row blocks of
-// NB_ROWS, spin); each CTA forms (X_blk W) and then (X_blk W) Yraw_n for its rows.
-constexpr int NB_ROWS = 4;
-constexpr int NB_THREADS = 512;
-// One CTA per (row block of NB_ROWS rows, spin, walker).  The gathers depend on the accepted sites,
-// so the kernel takes two rounds of global loads: the sites, then W, Yraw_n, X_blk and the block's
-// own rows of G, each mapped as warps over rows and lanes over columns (no index divisions, every
-// load of a thread in flight before its shared-memory stores).  The two products split each
-// output's sum over four consecutive lanes (strided partial sums, combined by shuffles), so every
-// warp works on them.
 template <typename T>
-__global__ void __launch_bounds__(NB_THREADS) next_block_kernel(const T* __restrict__ Gu0, long ld, int N,
-                                                                WindowBufs wb0, int sn, int nn, T* snap0,
-                                                                long gstride) {
-    constexpr int NW = WinCap<T>::NW, PP = NW + 1;
-    const int wk = blockIdx.z;
-    const WindowBufs wb = wb_walker<T>(wb0, wk, N);
-    const int m = *wb.m;
-    const int s = blockIdx.y, a0 = blockIdx.x * NB_ROWS, tid = threadIdx.x, nt = blockDim.x;
-    const int ra = min(NB_ROWS, nn - a0);
-    const T* G = Gu0 + (size_t)wk * gstride + (size_t)s * N * ld;
-    T* out = snap0 + (size_t)wk * 2 * NW * NW + (size_t)s * NW * NW;
-    extern __shared__ __align__(16) unsigned char nb_smem[];
-    T* Ws = (T*)nb_smem;         // [m][PP]
-    T* Ys = Ws + NW * PP;        // [m][PP]   Yraw_n
-    T* Xs = Ys + NW * PP;        // [NB_ROWS][PP]
-    T* Ts = Xs + NB_ROWS * PP;   // [NB_ROWS][PP]  X_blk W
-    T* Gr = Ts + NB_ROWS * PP;   // [NB_ROWS][PP]  G[sn + a0 + a][sn + c]
-    constexpr int CS = NW / 32;
-    const int lane = tid & 31, warp = tid >> 5, nwarp = nt >> 5;
-    __shared__ int sidx[NW];
-    for (int q = tid; q < m; q += nt) sidx[q] = wb.idx[q];
-    __syncthreads();
-    const T* W = (const T*)wb.Wx + (size_t)s * NW * NW;
-    // rows r of W and Yraw_n (r < m), of X_blk and of the block's own rows (r < ra) by warps,
-    // columns by lanes
-    for (int r = warp; r < m; r += nwarp) {
-        const T* wrow = W + (size_t)r * NW;
-        const T* grow = G + (long)sidx[r] * ld + sn;
-        T vw[CS], vy[CS];
-#pragma unroll
-        for (int j = 0; j < CS; ++j) {
-            const int c = lane + 32 * j;
-            vw[j] = c < m ? wrow[c] : T(0);
-            vy[j] = c < nn ? grow[c] : T(0);
-        }
-#pragma unroll
-        for (int j = 0; j < CS; ++j) {
-            const int c = lane + 32 * j;
-            if (c < m) Ws[r * PP + c] = vw[j];
-            if (c < nn) Ys[r * PP + c] = -vy[j];
-        }
-    }
-    for (int a = warp; a < ra; a += nwarp) {
-        const T* grow = G + (long)(sn + a0 + a) * ld;
-        T vx[CS], vg[CS];
-#pragma unroll
-        for (int j = 0; j < CS; ++j) {
-            const int k = lane + 32 * j;
-            vx[j] = k < m ? grow[sidx[k]] : T(0);
-            vg[j] = k < nn ? grow[sn + k] : T(0);
-        }
-#pragma unroll
-        for (int j = 0; j < CS; ++j) {
-            const int k = lane + 32 * j;
-            if (k < m) Xs[a * PP + k] = vx[j];
-            if (k < nn) Gr[a * PP + k] = vg[j];
-        }
-    }
-    __syncthreads();
-    // Ts = X_blk W: output (a, k) summed over l = part, part + 4, ... by lanes 4 g + part
-    {
-        const int nout = ra * m, iters = (4 * nout + nt - 1) / nt;
-        for (int it = 0; it < iters; ++it) {
-            const int o4 = tid + it * nt, g = o4 >> 2, part = o4 & 3;
-            T acc = T(0);
-            if (g < nout) {
-                const int a = g / m, k = g - a * m;
-                for (int l = part; l < m; l += 4) acc += Xs[a * PP + l] * Ws[l * PP + k];
-            }
-            acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-            acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-            if (g < nout && part == 0) Ts[(g / m) * PP + g % m] = acc;
-        }
-    }
-    __syncthreads();
-    // snap rows = G[rows, J] - Ts Yraw_n, the same split
-    {
-        const int nout = ra * nn, iters = (4 * nout + nt - 1) / nt;
-        for (int it = 0; it < iters; ++it) {
-            const int o4 = tid + it * nt, g = o4 >> 2, part = o4 & 3;
-            T acc = T(0);
-            int a = 0, c = 0;
-            if (g < nout) {
-                a = g / nn;
-                c = g - a * nn;
-                for (int l = part; l < m; l += 4) acc += Ts[a * PP + l] * Ys[l * PP + c];
-            }
-            acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-            acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-            if (g < nout && part == 0) out[(a0 + a) * NW + c] = Gr[a * PP + c] - acc;
+struct PanelArgs {
+    const T* G = nullptr; long ld = 0, gw = 0, gs = 0;  // G form: matrix, walker and spin strides
+    const T* V = nullptr;  // T form: raw columns [N][NW] and rows [NW][ldy] per (walker, spin)
+    const T* R = nullptr;
+    int N = 0;             // rows (columns) of the panels
+    int s0 = 0, n = 0;     // the window
+    int sn = 0, nn = 0;    // the next window (nn = 0: none)
+    T* snap = nullptr;
+    T* X = nullptr;        // [walker][spin][N][NW]
+    T* Y = nullptr;        // [walker][spin][NW][ldy]
+    long ldy = 0;
+    WindowBufs wb;
+};
+
+// Threads per block (four per line) and rows of the next window's block per block.
+template <typename T> struct PanelCfg { static constexpr int LT = sizeof(T) == 4 ? 512 : 128, RB = sizeof(T) == 4 ? 16 : 8; };
+constexpr int PL_B = 16;  // accepts a line takes at a time (four per thread)
+
+// Elements of the packed coefficient triangle of m accepts: the rows of the b-th group of PL_B accepts hold
+// the columns from PL_B b on.
+__host__ __device__ inline int panel_tri(int m) {
+    const int nb = (m + PL_B - 1) / PL_B;
+    return PL_B * PL_B * (nb * (nb + 1) / 2);
+}
+
+template <typename T>
+static size_t panel_smem(int n, int nn) {
+    constexpr size_t LN = PanelCfg<T>::LT / 4, RB = PanelCfg<T>::RB;
+    const size_t lines = (size_t)panel_tri(n) + LN * (n + 1);
+    const size_t block = nn > 0 ? 2 * (size_t)panel_tri(n) + RB * (n + 1) + (size_t)n * nn + RB * nn : 0;
+    return (lines > block ? lines : block) * sizeof(T) + 3 * WinCap<T>::NW * sizeof(int);
+}
+
+// Asynchronous copy of one element from global to shared memory (zero where !in).
+template <typename T>
+__device__ __forceinline__ void cp_async_elem(T* dst, const T* src, bool in) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    const int sz = in ? (int)sizeof(T) : 0;
+    if (sizeof(T) == 4) asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(sz) : "memory");
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(src), "r"(sz) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() {
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+}
+
+// The packed triangle E[k'][k] = W[k'][pos[k]], k >= k' (zero elsewhere), W = Wx or Wm of one spin.
+template <typename T>
+__device__ __forceinline__ void panel_load_tri(T* E, const T* W, const int* pos, int m, int tid, int nt) {
+    constexpr int NW = WinCap<T>::NW;
+    const int ep = (m + PL_B - 1) / PL_B * PL_B, lane = tid & 31;
+    for (int kp = tid >> 5; kp < ep; kp += nt >> 5) {
+        const int b = kp / PL_B, k0 = b * PL_B;
+        T* row = E + PL_B * (b * ep - PL_B * (b * (b - 1) / 2)) + (kp - k0) * (ep - k0);
+        for (int k = k0 + lane; k < ep; k += 32) {
+            const bool in = k >= kp && k < m;
+            cp_async_elem(row + k - k0, in ? W + (size_t)kp * NW + pos[k] : W, in);
         }
     }
 }
 
+// One line through the recursion, in place, by four lanes (h = lane & 3): entry k at line[off[k]]; column
+// lines (col) scale by the diagonal, row lines subtract the identity at their own column (gi, global index
+// of accept k in gidx[k]) first; neg: the raw line enters negated.  All lanes of a warp call this together.
 template <typename T>
-cudaError_t launch_next_block(cudaStream_t st, const T* Gu, const T* Gd, const SiteParams& sp, WindowBufs wb, int sn,
-                              int nn, T* snap, Batch bt) {
-    (void)Gd;
-    constexpr int NW = WinCap<T>::NW;
-    const size_t shm = (2 * (size_t)NW + 3 * NB_ROWS) * (NW + 1) * sizeof(T);
-    {
-        cudaError_t ea = ensure_smem_attr((const void*)next_block_kernel<T>, shm);
-        if (ea != cudaSuccess) return ea;
+__device__ __forceinline__ void panel_line(T* line, const int* off, int step, const T* E, int m, bool col, bool neg,
+                                           const int* gidx, int gi, bool own, int lane) {
+    constexpr int VW = Vec16<T>::W;
+    using V = typename Vec16<T>::V;
+    constexpr unsigned FULL = 0xffffffffu;
+    const int h = lane & 3, ep = (m + PL_B - 1) / PL_B * PL_B;
+    const T* Eb = E;  // rows of group b
+    for (int kb = 0; kb < m; kb += PL_B) {
+        T v[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const int k = kb + 4 * h + t;
+            T x = T(0);
+            if (k < m) {
+                x = line[off[k] * step];
+                if (neg) x = -x;
+                if (!col && gidx && gidx[k] == gi) x -= T(1);
+            }
+            v[t] = x;
+        }
+        const T* Ep = E + kb + 4 * h;  // columns kb + 4 h .. of the finished accepts' rows
+        for (int k0 = 0, w = ep; k0 < kb; k0 += PL_B, w -= PL_B) {
+#pragma unroll
+            for (int j = 0; j < PL_B; ++j) {
+                const T x = line[off[k0 + j] * step];
+                T d[4];
+#pragma unroll
+                for (int t = 0; t < 4; t += VW) *(V*)(d + t) = *(const V*)(Ep + j * w + t);
+#pragma unroll
+                for (int t = 0; t < 4; ++t) v[t] = fma(x, d[t], v[t]);
+            }
+            Ep += PL_B * w - PL_B;
+        }
+        const int w = ep - kb;
+#pragma unroll
+        for (int j = 0; j < PL_B; ++j) {
+            if (kb + j < m) {
+                T x = __shfl_sync(FULL, v[j & 3], (lane & ~3) | (j >> 2));
+                if (col) x *= Eb[j * w + j];
+                if (own && h == 0) line[off[kb + j] * step] = x;
+                T d[4];
+#pragma unroll
+                for (int t = 0; t < 4; t += VW) *(V*)(d + t) = *(const V*)(Eb + j * w + 4 * h + t);
+#pragma unroll
+                for (int t = 0; t < 4; ++t) v[t] = fma(x, d[t], v[t]);  // entries up to j are not read again
+            }
+        }
+        __syncwarp();
+        Eb += PL_B * w;
     }
+}
+
+// Grid (row blocks, then column blocks of N lines, then blocks of the next window; spin; walker).  A block
+// stages raw lines and the coefficient triangle in shared memory by asynchronous copies and takes each
+// line through the recursion with four lanes.  A block of the next window forms the w of its RB rows and
+// the q of all nn columns and writes G[J][J] + w_J q_J.  Bound by the latency of the recursion (m^2 / 2
+// multiply-adds per line).
+template <typename T, bool TF>
+__global__ void __launch_bounds__(PanelCfg<T>::LT) panel_kernel(PanelArgs<T> a) {
+    constexpr int NW = WinCap<T>::NW, LT = PanelCfg<T>::LT, LN = LT / 4, RB = PanelCfg<T>::RB;
+    const int wk = blockIdx.z, s = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int N = a.N, n = a.n, nl = (N + LN - 1) / LN, z = 2 * wk + s, bx = blockIdx.x;
+    const WindowBufs wb = wb_walker<T>(a.wb, wk, N);
+    const T* G = TF ? nullptr : a.G + (size_t)wk * a.gw + (size_t)s * a.gs;
+    const int m = *wb.m;
+    extern __shared__ __align__(16) unsigned char pl_smem[];
+    T* E = (T*)pl_smem;
+    const T* W0 = (const T*)wb.Wx + (size_t)s * NW * NW;
+    const T* W1 = (const T*)wb.Wm + (size_t)s * NW * NW;
+    const int tri = panel_tri(m);
+    if (bx >= 2 * nl) {  // rows r0 .. r0 + RB - 1 of the next window's block
+        T* E1 = E + tri;
+        T* bw = E1 + tri;                    // w lines [RB][n + 1]
+        T* bq = bw + RB * (n + 1);           // q lines [m][nn]
+        T* gb = bq + (size_t)n * a.nn;       // G[J rows][J] [RB][nn]
+        int* gidx = (int*)(gb + RB * a.nn);  // accepts: global index, position in the window, own index
+        int *pos = gidx + NW, *idn = pos + NW;
+        const int r0 = (bx - 2 * nl) * RB, nr = min(RB, a.nn - r0), nn = a.nn;
+        for (int k = tid; k < m; k += LT) {
+            gidx[k] = wb.idx[k];
+            pos[k] = wb.idx[k] - a.s0;
+            idn[k] = k;
+        }
+        __syncthreads();
+        const T* rows = G + (long)(a.sn + r0) * a.ld;
+        for (int r = warp; r < nr; r += LT / 32) {
+            for (int c = lane; c < nn; c += 32) cp_async_elem(gb + r * nn + c, rows + r * a.ld + a.sn + c, true);
+            for (int k = lane; k < m; k += 32) cp_async_elem(bw + r * (n + 1) + k, rows + r * a.ld + gidx[k], true);
+        }
+        for (int k = warp; k < m; k += LT / 32)
+            for (int c = lane; c < nn; c += 32)
+                cp_async_elem(bq + k * nn + c, G + (long)gidx[k] * a.ld + a.sn + c, true);
+        panel_load_tri<T>(E, W0, pos, m, tid, LT);
+        panel_load_tri<T>(E1, W1, pos, m, tid, LT);
+        cp_async_wait_all();
+        __syncthreads();
+        // the next window's sites are not among the accepts: no identity term.  Row lines fill whole warps
+        // (8 lines each) so that a warp has lines of one kind.
+        constexpr int RW = RB / 8;
+        for (int wv = warp; wv * 8 < 8 * RW + nn; wv += LT / 32) {
+            const bool col = wv < RW;
+            const int l0 = (col ? wv : wv - RW) * 8, l = l0 + (lane >> 2), lim = col ? nr : nn, lc = min(l, lim - 1);
+            if (l0 < lim)
+                panel_line<T>(col ? bw + lc * (n + 1) : bq + lc, idn, col ? 1 : nn, col ? E : E1, m, col, false, nullptr,
+                              0, l < lim, lane);
+        }
+        __syncthreads();
+        T* out = a.snap + (size_t)z * NW * NW + (size_t)r0 * NW;
+        for (int r = warp; r < nr; r += LT / 32)
+            for (int c = lane; c < nn; c += 32) {
+                T acc = gb[r * nn + c];
+                const T* wr = bw + r * (n + 1);
+#pragma unroll 8
+                for (int k = 0; k < m; ++k) acc = fma(wr[k], bq[k * nn + c], acc);
+                out[r * NW + c] = acc;
+            }
+        return;
+    }
+    if (m == 0) return;
+    const bool col = bx < nl;  // column lines: one per row of G
+    const int i0 = (col ? bx : bx - nl) * LN, cnt = min(LN, N - i0);
+    T* buf = E + tri;  // column lines [LN][n + 1], row lines [m][LN]
+    int* gidx = (int*)(buf + (size_t)LN * (n + 1));
+    int *pos = gidx + NW, *idn = pos + NW;
+    for (int k = tid; k < m; k += LT) {
+        gidx[k] = TF ? -1 : wb.idx[k];
+        pos[k] = wb.idx[k] - a.s0;
+        idn[k] = k;
+    }
+    __syncthreads();
+    if (col) {
+        for (int r = warp; r < cnt; r += LT / 32)
+            for (int k = lane; k < m; k += 32)
+                cp_async_elem(buf + r * (n + 1) + k,
+                              TF ? a.V + ((size_t)z * N + i0 + r) * NW + k : G + (long)(i0 + r) * a.ld + gidx[k], true);
+    } else {
+        for (int k = warp; k < m; k += LT / 32)
+            for (int c = lane; c < cnt; c += 32)
+                cp_async_elem(buf + k * LN + c,
+                              TF ? a.R + ((size_t)z * NW + k) * a.ldy + i0 + c : G + (long)gidx[k] * a.ld + i0 + c, true);
+    }
+    panel_load_tri<T>(E, col ? W0 : W1, pos, m, tid, LT);
+    cp_async_wait_all();
+    __syncthreads();
+    if (warp * 8 < cnt) {
+        const int l = tid >> 2, lc = min(l, cnt - 1);
+        panel_line<T>(col ? buf + lc * (n + 1) : buf + lc, idn, col ? 1 : LN, E, m, col, TF && !col, gidx, i0 + lc,
+                      l < cnt, lane);
+    }
+    __syncthreads();
+    if (col) {
+        T* out = a.X + ((size_t)z * N + i0) * NW;
+        for (int r = warp; r < cnt; r += LT / 32)
+            for (int k = lane; k < m; k += 32) out[r * NW + k] = buf[r * (n + 1) + k];
+    } else {
+        for (int k = warp; k < m; k += LT / 32)
+            for (int c = lane; c < cnt; c += 32) a.Y[((size_t)z * NW + k) * a.ldy + i0 + c] = buf[k * LN + c];
+    }
+}
+
+template <typename T, bool TF>
+static cudaError_t launch_panel_kernel(cudaStream_t st, const PanelArgs<T>& a, int nwk) {
+    cudaError_t e = ensure_smem_attr((const void*)panel_kernel<T, TF>, panel_smem<T>(WinCap<T>::NW, WinCap<T>::NW));
+    if (e != cudaSuccess) return e;
+    constexpr int LN = PanelCfg<T>::LT / 4, RB = PanelCfg<T>::RB;
     count_launch();
-    const int nbx = (nn + NB_ROWS - 1) / NB_ROWS;
-    next_block_kernel<T><<<dim3(nbx, 2, bt.nwk), NB_THREADS, shm, st>>>(Gu, sp.ld, sp.N, wb, sn, nn, snap,
-                                                                         bt.gstride);
+    panel_kernel<T, TF><<<dim3(2 * ((a.N + LN - 1) / LN) + (a.nn + RB - 1) / RB, 2, nwk), PanelCfg<T>::LT,
+                          panel_smem<T>(a.n, a.nn), st>>>(a);
     return cudaGetLastError();
 }
 
-// The panel gathers X = G[:, I], Yraw = E_I^T - G[I, :] and Y' = W Yraw of one window.
 template <typename T>
-cudaError_t launch_flush_panels(cudaStream_t sf, T* Gu, T* Gd, const SiteParams& sp, WindowBufs wb, int nw, Batch bt) {
-    (void)Gd;
-    constexpr int NW = WinCap<T>::NW;
-    const int N = sp.N;
-    count_launch();
-    gather_kernel<T><<<dim3(256, 2, bt.nwk), 256, 0, sf>>>(Gu, sp.ld, N, wb, NW, bt.gstride, (long)N * sp.ld);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    GemmArgs<T> g;  // Y' = W Yraw, batch (walker, spin)
-    g.M = nw; g.N = N; g.K = nw; g.Kdev = wb.m; g.kdiv = 2;
-    g.A = (const T*)wb.Wx; g.lda = NW; g.sA = (long)NW * NW;
-    g.B = (const T*)wb.Y; g.ldb = N; g.sB = (long)NW * N;
-    g.C = (T*)wb.Y + (size_t)2 * bt.nwk * NW * N; g.ldc = N; g.sC = (long)NW * N;
-    g.batch = 2 * bt.nwk;
-    return gemm<T>(sf, g);
+cudaError_t launch_flush_panels(cudaStream_t st, const T* Gu, const SiteParams& sp, WindowBufs wb, int s0, int n,
+                                int sn, int nn, T* snap, Batch bt) {
+    PanelArgs<T> a;
+    a.G = Gu; a.ld = sp.ld; a.gw = bt.gstride; a.gs = (long)sp.N * sp.ld;
+    a.N = sp.N; a.s0 = s0; a.n = n; a.sn = sn; a.nn = nn;
+    a.snap = snap;
+    a.X = (T*)wb.X; a.Y = (T*)wb.Y; a.ldy = sp.N;
+    a.wb = wb;
+    return launch_panel_kernel<T, false>(st, a, bt.nwk);
 }
 
-// G <- G - X Y' (the N x N rank-m product, after launch_flush_panels on the same stream).
+template <typename T>
+cudaError_t launch_tform_panels(cudaStream_t st, int ns, WindowBufs wb, int s0, int n, T* V, const T* R, T* Y,
+                                int nwk) {
+    PanelArgs<T> a;
+    a.V = V; a.R = R;
+    a.N = ns; a.s0 = s0; a.n = n;
+    a.X = V; a.Y = Y; a.ldy = ns;
+    a.wb = wb;
+    return launch_panel_kernel<T, true>(st, a, nwk);
+}
+
+// G <- G + X Y (the N x N rank-m product of launch_flush_panels' panels).
 template <typename T>
 cudaError_t launch_flush_gemm(cudaStream_t sf, T* Gu, T* Gd, const SiteParams& sp, WindowBufs wb, int nw, Batch bt) {
     (void)Gd;
@@ -1408,9 +1478,9 @@ cudaError_t launch_flush_gemm(cudaStream_t sf, T* Gu, T* Gd, const SiteParams& s
     GemmArgs<T> h;
     h.M = N; h.N = N; h.K = nw; h.Kdev = wb.m; h.kdiv = 2;
     h.A = (const T*)wb.X; h.lda = NW; h.sA = (long)N * NW;
-    h.B = (const T*)wb.Y + (size_t)2 * bt.nwk * NW * N; h.ldb = N; h.sB = (long)NW * N;
+    h.B = (const T*)wb.Y; h.ldb = N; h.sB = (long)NW * N;
     h.C = Gu; h.ldc = sp.ld; h.sC = (long)N * sp.ld;
-    h.alpha = T(-1); h.beta = T(1);
+    h.alpha = T(1); h.beta = T(1);
     h.batch = 2 * bt.nwk;
     return gemm<T>(sf, h);
 }
@@ -1482,17 +1552,17 @@ template cudaError_t launch_tform_scale_rows<float>(cudaStream_t, float*, int, i
                                                     const int8_t*, long, const double*, int);
 template cudaError_t launch_tform_scale_rows<double>(cudaStream_t, double*, int, int, long, long, WindowBufs,
                                                      const int8_t*, long, const double*, int);
-template cudaError_t launch_flush_panels<float>(cudaStream_t, float*, float*, const SiteParams&, WindowBufs, int,
-                                               Batch);
-template cudaError_t launch_flush_panels<double>(cudaStream_t, double*, double*, const SiteParams&, WindowBufs, int,
-                                                Batch);
+template cudaError_t launch_flush_panels<float>(cudaStream_t, const float*, const SiteParams&, WindowBufs, int, int,
+                                               int, int, float*, Batch);
+template cudaError_t launch_flush_panels<double>(cudaStream_t, const double*, const SiteParams&, WindowBufs, int, int,
+                                                int, int, double*, Batch);
+template cudaError_t launch_tform_panels<float>(cudaStream_t, int, WindowBufs, int, int, float*, const float*, float*,
+                                               int);
+template cudaError_t launch_tform_panels<double>(cudaStream_t, int, WindowBufs, int, int, double*, const double*,
+                                                double*, int);
 template cudaError_t launch_flush_gemm<float>(cudaStream_t, float*, float*, const SiteParams&, WindowBufs, int, Batch);
 template cudaError_t launch_flush_gemm<double>(cudaStream_t, double*, double*, const SiteParams&, WindowBufs, int,
                                               Batch);
-template cudaError_t launch_next_block<float>(cudaStream_t, const float*, const float*, const SiteParams&, WindowBufs,
-                                              int, int, float*, Batch);
-template cudaError_t launch_next_block<double>(cudaStream_t, const double*, const double*, const SiteParams&,
-                                               WindowBufs, int, int, double*, Batch);
 template cudaError_t launch_flush<float>(cudaStream_t, float*, float*, const SiteParams&, WindowBufs, int);
 template cudaError_t launch_flush<double>(cudaStream_t, double*, double*, const SiteParams&, WindowBufs, int);
 
