@@ -124,12 +124,12 @@ int afqmc_soc_measure_energy(afqmc_soc_ctx* ctx, double* energy, void* stream);
  *   scalars  host, 4 doubles per walker: Re D, Im D, Re <Delta^2>, Im <Delta^2>.
  *   nk       host, nullable: 4N doubles per walker, <n_ku> (N complex) then <n_kd> (N complex).
  *   Mk       host, nullable: N x N complex (re, im interleaved) per walker.
- * The first call allocates the DFT tables (2 x (2 ldz)^2 + 2N 2 ldz doubles, ldz = 2N rounded up to
- * 32) and scratch of the same order.  Syncs the stream.  AFQMC_ERR_ARG before init or for a NULL
+ * The first call allocates scratch (2 x 2N x 2 ldz doubles, ldz = 2N rounded up to 32) and the pairing
+ * matrices.  Syncs the stream.  AFQMC_ERR_ARG before init or for a NULL
  * scalars. */
 int afqmc_soc_measure_pairing(afqmc_soc_ctx* ctx, double* scalars, double* nk, double* Mk, void* stream);
 
-/* Accessors (sync the stream of the last call). *//* Accessors (sync the stream of the last call). */
+/* Accessors (sync the stream of the last call). */
 int afqmc_soc_get_G(afqmc_soc_ctx* ctx, int walker, double* host_out);       /* 2N x 2N complex */
 int afqmc_soc_set_G(afqmc_soc_ctx* ctx, int walker, const double* host_in);  /* 2N x 2N complex */
 int afqmc_soc_get_fields(afqmc_soc_ctx* ctx, int walker, int8_t* host_out);  /* M x N */

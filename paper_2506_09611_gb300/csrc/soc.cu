@@ -1131,6 +1131,65 @@ __global__ void __launch_bounds__(256) soc_pair_scalars_kernel(const double* A, 
     }
 }
 
+// Two-dimensional lattice DFT, in FP64, of vectors of N = L^2 complex elements of a row-split matrix: element
+// i = x + L y of vector v of block b at in[v vs + i es + b bs] (imaginary part + ldz), written to the same
+// place of out: out_q = L^-1 sum_i e^{sign 2 pi i (qx x + qy y) / L} in_i, as two passes of L-point sums (4 L
+// multiply-adds per element and pass instead of the 4 N of a product by the dense DFT matrix).  tw: the L
+// factors L^-1/2 e^{2 pi i k / L}.  A CTA keeps vpc vectors twice in shared memory.  Bound by the FP64
+// multiply-adds: pairing matrix of one 20 x 20 walker 9.8 ms as two dense products, 0.5 ms so.
+__global__ void __launch_bounds__(256) soc_dft2_kernel(const double* in, double* out, long ldz, int L, int nvec,
+                                                       long vs, long es, long bs, double sign, const double* tw,
+                                                       int vpc) {
+    extern __shared__ __align__(16) double df_smem[];
+    const int N = L * L, tid = threadIdx.x, nt = blockDim.x, v0 = blockIdx.x * vpc, nv = min(vpc, nvec - v0);
+    double* wr = df_smem;                          // [L] factors
+    double* wi = wr + L;
+    double* buf[2] = {wi + L, wi + L + 2 * (size_t)vpc * N};  // [2 parts][N][vpc]
+    const long o0 = (long)blockIdx.y * bs + (long)v0 * vs;
+    const long im = (long)vpc * N;
+    for (int k = tid; k < L; k += nt) {
+        wr[k] = tw[2 * k];
+        wi[k] = sign * tw[2 * k + 1];
+    }
+    const bool vfast = vs < es;  // neighbouring threads take neighbouring elements of memory
+    for (int e = tid; e < N * nv; e += nt) {
+        const int i = vfast ? e / nv : e % N, v = vfast ? e % nv : e / N;
+        const long o = o0 + (long)v * vs + (long)i * es;
+        buf[0][i * vpc + v] = in[o];
+        buf[0][im + i * vpc + v] = in[o + ldz];
+    }
+    __syncthreads();
+    for (int axis = 0; axis < 2; ++axis) {
+        const double *sr = buf[axis], *si = sr + im;
+        double *dr = buf[axis ^ 1], *di = dr + im;
+        const int st = (axis ? L : 1) * vpc;
+        for (int e = tid; e < N * nv; e += nt) {
+            const int i = e / nv, v = e - i * nv, x = i % L, y = i / L, q = axis ? y : x;
+            const int base = (axis ? x : y * L) * vpc + v;
+            double a0 = 0.0, a1 = 0.0, b0 = 0.0, b1 = 0.0;
+            int k = 0;
+            for (int j = 0; j < L; ++j) {
+                const double r = sr[base + j * st], m = si[base + j * st], c = wr[k], d = wi[k];
+                a0 = fma(r, c, a0);
+                a1 = fma(m, d, a1);
+                b0 = fma(r, d, b0);
+                b1 = fma(m, c, b1);
+                k += q;
+                if (k >= L) k -= L;
+            }
+            dr[i * vpc + v] = a0 - a1;
+            di[i * vpc + v] = b0 + b1;
+        }
+        __syncthreads();
+    }
+    for (int e = tid; e < N * nv; e += nt) {  // two passes: the result is back in buf[0]
+        const int i = vfast ? e / nv : e % N, v = vfast ? e % nv : e / N;
+        const long o = o0 + (long)v * vs + (long)i * es;
+        out[o] = buf[0][i * vpc + v];
+        out[o + ldz] = buf[0][im + i * vpc + v];
+    }
+}
+
 // From At = F2 A F2^+ (row-split, At_{(p s),(q t)} = <c+_{q t} c_{p s}>): nk[k] = At_{ku,ku},
 // nk[N + k] = At_{kd,kd} (complex), and Mk[k][k'] = At_{k'u,ku} At_{-k'd,-kd} - At_{-k'd,ku} At_{k'u,-kd}
 // (<D+_k D_k'> of one walker, D+_k = c+_{k u} c+_{-k d}; -k = (-kx, -ky) mod L).
@@ -1218,11 +1277,9 @@ struct afqmc_soc_ctx {
     bool oz_O = false, oz_G = false;
     void* ozw = nullptr;
     double* ozs = nullptr;
-    // pairing observables (allocated at the first afqmc_soc_measure_pairing): [Re F2 | Im F2] rows,
-    // the realified F2^+ (2 ldz x 2 ldz), FP64 scratch A (2N x 2 ldz), S~ (2 ldz x 2 ldz),
-    // At (2N x 2 ldz), Mk per walker (N x N complex each) and the per-walker outputs
-    double *Frs = nullptr, *Fh = nullptr, *pA = nullptr, *pS = nullptr, *pAt = nullptr, *pMk = nullptr,
-           *pOut = nullptr;
+    // pairing observables (allocated at the first afqmc_soc_measure_pairing): the L DFT factors, FP64
+    // scratch A and At (2N x 2 ldz), Mk per walker (N x N complex each) and the per-walker outputs
+    double *pTw = nullptr, *pA = nullptr, *pAt = nullptr, *pMk = nullptr, *pOut = nullptr;
     // profiling
     struct Ev {
         int ph;
@@ -1979,37 +2036,24 @@ int afqmc_soc_measure_pairing(afqmc_soc_ctx* ctx, double* scalars, double* nk, d
     ctx->last = st;
     const int L = ctx->p.L, N = ctx->N, N2 = ctx->N2, nwk = ctx->nwk;
     const long ldz = ctx->ldz, ld2 = 2 * ldz;
-    if (!ctx->Frs) {
-        // F2 = diag(F, F), F_{q j} = N^{-1/2} e^{-i q.r_j}: its rows for the left product and the
-        // realified right operand of the product by F2^+ (C~ = [[Re C, Im C], [-Im C, Re C]])
-        std::vector<double> frs((size_t)N2 * ld2, 0.0), fh((size_t)ld2 * ld2, 0.0);
-        const double sN = 1.0 / sqrt((double)N);
-        for (int q = 0; q < N; ++q)
-            for (int jj = 0; jj < N; ++jj) {
-                const double ph = -2.0 * M_PI * ((double)(q % L) * (jj % L) + (double)(q / L) * (jj / L)) / L;
-                const double fr = cos(ph) * sN, fi = sin(ph) * sN;
-                for (int sp = 0; sp < 2; ++sp) {
-                    const long r = sp * N + q, c = sp * N + jj;  // F2[r][c] = F[q][jj]
-                    frs[(size_t)r * ld2 + c] = fr;
-                    frs[(size_t)r * ld2 + ldz + c] = fi;
-                    // C = F2^+: C[c][r] = conj(F2[r][c])
-                    fh[(size_t)c * ld2 + r] = fr;
-                    fh[(size_t)c * ld2 + ldz + r] = -fi;
-                    fh[(size_t)(ldz + c) * ld2 + r] = fi;
-                    fh[(size_t)(ldz + c) * ld2 + ldz + r] = fr;
-                }
-            }
-        SCK(soc_alloc(ctx, &ctx->Frs, frs.size() * 8, st));
-        SCK(soc_alloc(ctx, &ctx->Fh, fh.size() * 8, st));
+    if (!ctx->pTw) {
+        std::vector<double> tw(2 * (size_t)L);
+        for (int k = 0; k < L; ++k) {
+            tw[2 * k] = cos(2.0 * M_PI * k / L) / sqrt((double)L);
+            tw[2 * k + 1] = sin(2.0 * M_PI * k / L) / sqrt((double)L);
+        }
         SCK(soc_alloc(ctx, &ctx->pA, (size_t)N2 * ld2 * 8, st));
-        SCK(soc_alloc(ctx, &ctx->pS, (size_t)ld2 * ld2 * 8, st));
         SCK(soc_alloc(ctx, &ctx->pAt, (size_t)N2 * ld2 * 8, st));
         SCK(soc_alloc(ctx, &ctx->pMk, (size_t)nwk * N * N * 16, st));
         SCK(soc_alloc(ctx, &ctx->pOut, (size_t)nwk * (4 + 4 * N) * 8, st));
-        SCK(cudaMemcpyAsync(ctx->Frs, frs.data(), frs.size() * 8, cudaMemcpyHostToDevice, st));
-        SCK(cudaMemcpyAsync(ctx->Fh, fh.data(), fh.size() * 8, cudaMemcpyHostToDevice, st));
-        SCK(cudaStreamSynchronize(st));  // the host tables go out of scope
+        SCK(soc_alloc(ctx, &ctx->pTw, tw.size() * 8, st));
+        SCK(cudaMemcpyAsync(ctx->pTw, tw.data(), tw.size() * 8, cudaMemcpyHostToDevice, st));
+        SCK(cudaStreamSynchronize(st));  // the host table goes out of scope
     }
+    // vectors per CTA of the DFT: two copies in at most 96 KB (two CTAs per SM), at least one
+    const int vpc = std::max(1, std::min(8, (int)(96 * 1024 / (32 * (size_t)N))));
+    const size_t dfs = (2 * (size_t)L + 4 * (size_t)vpc * N) * 8;
+    SCK(ensure_smem_attr((const void*)soc_dft2_kernel, dfs));
     SCK(cudaMemsetAsync(ctx->pOut, 0, (size_t)nwk * (4 + 4 * N) * 8, st));
     const size_t es = ctx->f64 ? 8 : 4;
     for (int w = 0; w < nwk; ++w) {
@@ -2026,22 +2070,16 @@ int afqmc_soc_measure_pairing(afqmc_soc_ctx* ctx, double* scalars, double* nk, d
             ctx->pA, ldz, N, out);
         SCK(cudaGetLastError());
         if (!nk && !Mk) continue;
-        // At = F2 A F2^+: S~ rows [0, 2N) = A (F2^+)~, the realified S~, then [Re F2 | Im F2] S~
-        GemmArgs<double> g1;
-        g1.M = N2; g1.N = (int)ld2; g1.K = (int)ld2;
-        g1.A = ctx->pA; g1.lda = ld2;
-        g1.B = ctx->Fh; g1.ldb = ld2;
-        g1.C = ctx->pS; g1.ldc = ld2;
-        SCK(gemm<double>(st, g1));
+        // At = F2 A F2^+: the DFT e^{+iq.r} along every row's columns, then e^{-iq.r} along the rows, each
+        // spin block on its own
+        const dim3 dg((unsigned)((N2 + vpc - 1) / vpc), 2);
         count_launch();
-        soc_realify_kernel<double><<<dim3((unsigned)((ld2 + 255) / 256), N2, 1), 256, 0, st>>>(ctx->pS, ldz, N2, 0, 1);
+        soc_dft2_kernel<<<dg, 256, dfs, st>>>(ctx->pA, ctx->pAt, ldz, L, N2, ld2, 1, N, 1.0, ctx->pTw, vpc);
         SCK(cudaGetLastError());
-        GemmArgs<double> g2;
-        g2.M = N2; g2.N = (int)ld2; g2.K = (int)ld2;
-        g2.A = ctx->Frs; g2.lda = ld2;
-        g2.B = ctx->pS; g2.ldb = ld2;
-        g2.C = ctx->pAt; g2.ldc = ld2;
-        SCK(gemm<double>(st, g2));
+        count_launch();
+        soc_dft2_kernel<<<dg, 256, dfs, st>>>(ctx->pAt, ctx->pAt, ldz, L, N2, 1, ld2, (long)N * ld2, -1.0, ctx->pTw,
+                                              vpc);
+        SCK(cudaGetLastError());
         count_launch();
         soc_pair_k_kernel<<<(unsigned)std::min<long>(((long)N * N + 255) / 256, 4096), 256, 0, st>>>(
             ctx->pAt, ldz, L, ctx->pMk + (size_t)w * 2 * N * N, nkw);
