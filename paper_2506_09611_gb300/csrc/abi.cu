@@ -1698,8 +1698,8 @@ int afqmc_recompute_G(afqmc_ctx* ctx, double* rel_drift, void* stream) {
             const Fac Lf = (defer && !fwd) ? fac_cur(w) : fac_L(w, j);
             for (int gi = 0; gi < ngr; ++gi) {
                 CK(form_Z(ctx, w, st, R, Lf, grp[gi][0], ng[gi], nullptr));
-                if (f64) CK(finish_G<double>(ctx, w, st, R, grp[gi][0], ng[gi], true));
-                else CK(finish_G<float>(ctx, w, st, R, grp[gi][0], ng[gi], true));
+                if (f64) CK(finish_G<double>(ctx, w, st, R, grp[gi][0], ng[gi], rel_drift != nullptr));
+                else CK(finish_G<float>(ctx, w, st, R, grp[gi][0], ng[gi], rel_drift != nullptr));
             }
             if (defer) {  // the stack entry, off the critical path
                 // Re-orthonormalise only when the next interval would otherwise propagate the basis

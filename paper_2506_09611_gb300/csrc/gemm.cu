@@ -4,7 +4,7 @@
 // flush of the delayed and block force-bias updates (Eqs. FinalDelay,
 // BlkFrcBsTnew2 in G form) and the FP64 recompute (Eq. GrFMatNew).  An FP32
 // update C += alpha A B with a small inner dimension (K <= 64: a window's flush)
-// takes rankm_kernel, written for that shape; everything else the general tile.
+// takes rankm_kernel, written for that shape; other FP32 products the general tile, FP64 ones dgemm_kernel.
 #include "internal.h"
 
 namespace afq {
@@ -85,6 +85,117 @@ __global__ void __launch_bounds__(NT) gemm_kernel(GemmArgs<T> g) {
             C[o] = (g.beta == T(0)) ? v : v + g.beta * C[o];
         }
     }
+}
+
+// The same product in FP64.  This part runs FP64 at 2 multiply-adds a clock and SM (a warp instruction
+// holds its partition's unit for 64 cycles), so a product is bound by the multiply-adds it issues, padding
+// included, and by how evenly they spread over the SMs; shared-memory traffic does not matter.  Hence tiles
+// from 16 x 16 to 64 x 64 (BM / 16 x BN / 16 outputs a thread), picked per shape by dgemm_tile; the next
+// k-slice is fetched into registers under the current one.  The sum runs over k in order.
+template <int BM, int BN>
+__global__ void __launch_bounds__(NT) dgemm_kernel(GemmArgs<double> g) {
+    constexpr int TM = BM / 16, TN = BN / 16;
+    const int z = blockIdx.z;
+    const double* A = g.A + z * g.sA;
+    const double* B = g.B + z * g.sB;
+    double* C = g.C + z * g.sC;
+    const double* rs = g.rs ? g.rs + z * g.srs : nullptr;
+    const double* cs = g.cs ? g.cs + z * g.scs : nullptr;
+    const double* bs = g.bs ? g.bs + z * g.sbs : nullptr;
+    const int K = g.Kdev ? min(g.Kdev[g.kdiv > 0 ? z / g.kdiv : 0], g.K) : g.K;
+    if (K <= 0 && g.beta == 1.0 && g.cs == nullptr && g.rs == nullptr) return;  // C unchanged
+    __shared__ double As[BK][BM + 1];
+    __shared__ double Bs[BK][BN + 1];
+    const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
+    const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+    double acc[TM][TN], pa[TM], pb[TN];
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < TN; ++j) acc[i][j] = 0.0;
+    auto fetch = [&](int k0) {
+#pragma unroll
+        for (int q = 0; q < TM; ++q) {  // k fastest
+            const int e = tid + q * NT, gm = m0 + e / BK, gk = k0 + e % BK;
+            pa[q] = (gm < g.M && gk < K) ? A[(long)gm * g.lda + gk] : 0.0;
+        }
+#pragma unroll
+        for (int q = 0; q < TN; ++q) {  // n fastest
+            const int e = tid + q * NT, gk = k0 + e / BN, gn = n0 + e % BN;
+            pb[q] = (gk < K && gn < g.N) ? B[(long)gk * g.ldb + gn] : 0.0;
+            if (bs && gk < K) pb[q] *= bs[gk];
+        }
+    };
+    fetch(0);
+    for (int k0 = 0; k0 < K; k0 += BK) {
+#pragma unroll
+        for (int q = 0; q < TM; ++q) As[(tid + q * NT) % BK][(tid + q * NT) / BK] = pa[q];
+#pragma unroll
+        for (int q = 0; q < TN; ++q) Bs[(tid + q * NT) / BN][(tid + q * NT) % BN] = pb[q];
+        __syncthreads();
+        if (k0 + BK < K) fetch(k0 + BK);
+        const int kn = min(BK, K - k0);
+        auto step = [&](int kk) {
+            double a[TM], b[TN];
+#pragma unroll
+            for (int i = 0; i < TM; ++i) a[i] = As[kk][ty + 16 * i];
+#pragma unroll
+            for (int j = 0; j < TN; ++j) b[j] = Bs[kk][tx + 16 * j];
+#pragma unroll
+            for (int i = 0; i < TM; ++i)
+#pragma unroll
+                for (int j = 0; j < TN; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+        };
+        if (kn == BK) {
+#pragma unroll
+            for (int kk = 0; kk < BK; ++kk) step(kk);
+        } else {
+            for (int kk = 0; kk < kn; ++kk) step(kk);
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < TM; ++i) {
+        const int gm = m0 + ty + 16 * i;
+        if (gm >= g.M) continue;
+#pragma unroll
+        for (int j = 0; j < TN; ++j) {
+            const int gn = n0 + tx + 16 * j;
+            if (gn >= g.N) continue;
+            double v = acc[i][j];
+            if (g.alpha != 1.0) v *= g.alpha;
+            if (rs) v *= rs[gm];
+            if (cs) v *= cs[gn];
+            const long o = (long)gm * g.ldc + gn;
+            if (g.beta == 1.0) v += C[o];
+            else if (g.beta != 0.0) v = fma(g.beta, C[o], v);
+            C[o] = v;
+        }
+    }
+}
+
+template <int BM, int BN>
+cudaError_t dgemm_launch(cudaStream_t st, const GemmArgs<double>& g) {
+    count_launch();
+    dgemm_kernel<BM, BN><<<dim3((g.N + BN - 1) / BN, (g.M + BM - 1) / BM, g.batch), NT, 0, st>>>(g);
+    return cudaGetLastError();
+}
+
+// The tile whose busiest SM issues the fewest multiply-adds: tiles per SM (rounded up) times the tile's
+// size, plus a fixed cost per tile (its share of latencies, about 32 outputs' worth).
+int dgemm_tile(const GemmArgs<double>& g) {
+    static const int bm[7] = {64, 64, 32, 32, 32, 16, 16}, bn[7] = {64, 32, 64, 32, 16, 32, 16};
+    int best = 0;
+    long cost = 0;
+    for (int t = 0; t < 7; ++t) {
+        const long tiles = (long)((g.M + bm[t] - 1) / bm[t]) * ((g.N + bn[t] - 1) / bn[t]) * g.batch;
+        const long c = (tiles + 151) / 152 * (bm[t] * bn[t] + 32);
+        if (t == 0 || c < cost) {
+            best = t;
+            cost = c;
+        }
+    }
+    return best;
 }
 
 // C += alpha A B for a small inner dimension (K <= RM_KMAX, FP32): the rank-m flush of a window,
@@ -191,10 +302,22 @@ cudaError_t gemm(cudaStream_t st, const GemmArgs<T>& g) {
             return cudaGetLastError();
         }
     }
-    dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM, g.batch);
-    count_launch();
-    gemm_kernel<T><<<grid, NT, 0, st>>>(g);
-    return cudaGetLastError();
+    if constexpr (sizeof(T) == 8) {
+        switch (dgemm_tile(g)) {
+            case 0: return dgemm_launch<64, 64>(st, g);
+            case 1: return dgemm_launch<64, 32>(st, g);
+            case 2: return dgemm_launch<32, 64>(st, g);
+            case 3: return dgemm_launch<32, 32>(st, g);
+            case 4: return dgemm_launch<32, 16>(st, g);
+            case 5: return dgemm_launch<16, 32>(st, g);
+            default: return dgemm_launch<16, 16>(st, g);
+        }
+    } else {
+        dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM, g.batch);
+        count_launch();
+        gemm_kernel<T><<<grid, NT, 0, st>>>(g);
+        return cudaGetLastError();
+    }
 }
 
 template cudaError_t gemm<float>(cudaStream_t, const GemmArgs<float>&);

@@ -2014,8 +2014,8 @@ int afqmc_soc_recompute_G(afqmc_soc_ctx* ctx, double* rel_drift, void* stream) {
         SCK(soc_stab(ctx, st, ctx->Ucur, ctx->fsz()));
         SCK(soc_to_stack(ctx, st, fwd, j));
     }
-    if (ctx->f64) SCK(soc_form_G<double>(ctx, st, j, true));
-    else SCK(soc_form_G<float>(ctx, st, j, true));
+    if (ctx->f64) SCK(soc_form_G<double>(ctx, st, j, rel_drift != nullptr));
+    else SCK(soc_form_G<float>(ctx, st, j, rel_drift != nullptr));
     ctx->need_recompute = false;
     if (rel_drift) {
         SCK(cudaStreamSynchronize(st));
