@@ -7,8 +7,8 @@
 //   * a panel of LU_NB columns is factored by one thread-block cluster per matrix: each CTA
 //     keeps its share of the rows in shared memory and the CTAs agree on every pivot through
 //     distributed shared memory and one cluster barrier per column;
-//   * the pivot rows' trailing part is finished inside the cluster (U12 = L11^{-1} A12);
-//   * the trailing update A22 -= L21 U12 is an FP64 tiled product over the whole GPU.
+//   * the pivot rows' trailing part U12 = L11^{-1} A12 and the trailing update A22 -= L21 U12 of the
+//     unpivoted rows run over the whole GPU.
 // Rows are not swapped: a pivoted row is flagged, keeps its multipliers left of its pivot
 // column and its U entries from there on, and perm[j] names the pivot row of column j.  Both
 // spins go through every launch (two independent matrices).
@@ -28,8 +28,7 @@ constexpr int LU_NB = 32;
 constexpr int LU_NBP = LU_NB + 1;
 
 // One cluster of CS CTAs per matrix (blockIdx.x / CS = matrix).  Factors columns
-// [j0, j0 + nbk) over the rows not yet pivoted and finishes the pivot rows' columns
-// [j0 + nbk, n).
+// [j0, j0 + nbk) over the rows not yet pivoted.
 // Pivot candidates compare |a| through the bit pattern of the double with the sign cleared:
 // for finite non-negative doubles the integer order is the numeric order, and integer compares
 // avoid the long FP64 latency on the pivot search's critical path.  Ties go to the lower row.
@@ -45,205 +44,289 @@ __device__ __forceinline__ void lu_pick(unsigned long long& k, int& r, double& x
     }
 }
 
+// 1 / x for a pivot: a 22-bit reciprocal of x's leading bits, taken in FP32 from the bit pattern, and one
+// step of Halley's iteration (1/x = s (1 + e + e^2 + ...), e = 1 - s x, error e^3 < 2^-63); outside the FP32
+// exponent range the division.  Three dependent FP64 operations where a division takes about 740 cycles.
+__device__ __forceinline__ double lu_rcp(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const int ex = (int)((hi >> 20) & 0x7ffu) - 1023;
+    if (ex < -100 || ex > 100) return 1.0 / x;
+    const float xm = __uint_as_float(0x3f800000u | ((hi & 0xfffffu) << 3) | (lo >> 29));
+    const unsigned rb = __float_as_uint(__fdividef(1.0f, xm));
+    const int re = (int)((rb >> 23) & 0xffu) - 127 - ex + 1023;
+    const double sd = __hiloint2double((int)((hi & 0x80000000u) | ((unsigned)re << 20) | ((rb & 0x7fffffu) >> 3)),
+                                       (int)(rb << 29));
+    const double e = fma(-x, sd, 1.0);
+    return fma(sd, fma(e, e, e), sd);
+}
+
+// The best candidate of a warp in every lane: largest key, ties to the lower row.  Three integer reductions.
+// Returns the lane that holds it.
+__device__ __forceinline__ int lu_warp_best(unsigned long long& k, int& r) {
+    const unsigned hi = (unsigned)(k >> 32), lo = (unsigned)k;
+    const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
+    const bool best = hi == mh && lo == ml;
+    const unsigned mr = __reduce_min_sync(0xffffffffu, best ? (unsigned)r : 0xffffffffu);
+    const int src = __ffs(__ballot_sync(0xffffffffu, best && (unsigned)r == mr)) - 1;
+    k = ((unsigned long long)mh << 32) | ml;
+    r = (int)mr;
+    return src;
+}
+
+// tpr threads per row (a power of two up to 8).  Per column: every warp pushes its candidate into the shared
+// memory of all CTAs, one cluster barrier, warp 0 of every CTA picks the winner and pulls the pivot row from
+// its owner (a pivoted row is never written again) while it takes the reciprocal, one block barrier, and the
+// own rows are updated, the next column first for the next candidates.  Bound by that chain: the first panel
+// of the 1600 x 700 factor took 128 us with one thread per row, the FP64 division and candidates read through
+// distributed shared memory.
 template <int CS>
-__global__ void __launch_bounds__(256) lu_panel_kernel(LuArgs a, int j0, int nbk) {
+__global__ void __launch_bounds__(256) lu_panel_kernel(LuArgs a, int j0, int nbk, int tpr) {
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank();
     const int mat = blockIdx.x / CS;
     double* A = lu_A(a, mat);
     int* perm = a.perm0 + (long)mat * a.pstride;
     int8_t* flag = a.flag0 + (long)mat * a.pstride;
-    const int m = a.m, n = a.n;
+    const int m = a.m;
     const long lda = a.lda;
     const int r0 = (int)((long)m * rank / CS), r1 = (int)((long)m * (rank + 1) / CS), nr = r1 - r0;
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5;
     extern __shared__ __align__(16) double lu_smem[];
     double* Pn = lu_smem;                    // [nr][LU_NBP] own rows of the panel
     int8_t* fl = (int8_t*)(Pn + (size_t)nr * LU_NBP);
-    // each warp's candidate of the step (by step parity): key, row, signed value
-    __shared__ unsigned long long cand_k[2][8];
-    __shared__ int cand_r[2][8];
-    __shared__ double cand_x[2][8];
+    // the candidates of all warps of the cluster (by step parity): key, signed value, row
+    __shared__ unsigned long long cand_k[2][8 * CS];
+    __shared__ double cand_x[2][8 * CS];
+    __shared__ int cand_r[2][8 * CS];
     __shared__ double L11[LU_NB][LU_NBP];    // pivot rows' panel values at their pivot step
-    __shared__ int s_prow[LU_NB];            // pivot row of each step
-    __shared__ int s_bad;
     __shared__ double s_pinv;
+    bool any_bad = false;
     for (int e = tid; e < nr * nbk; e += nt) {
         const int q = e / nbk, c = e - q * nbk;
         Pn[q * LU_NBP + c] = A[(long)(r0 + q) * lda + j0 + c];
     }
     for (int q = tid; q < nr; q += nt) fl[q] = flag[r0 + q];
-    if (tid == 0) s_bad = 0;
-    __syncthreads();
+    cl.sync();  // every CTA of the cluster runs before its shared memory is written from outside
+    const int h = tid & (tpr - 1), rows = nt / tpr, q0 = tid / tpr;
     // candidate of column 0 (later columns: found during the previous step's row update)
     unsigned long long bk = 0;
     int br = INT_MAX;
     double bx = 0.0;
-    for (int q = tid; q < nr; q += nt)
-        if (!fl[q]) {
-            const double x = Pn[q * LU_NBP];
-            lu_pick(bk, br, bx, lu_key(x), r0 + q, x);
-        }
+    if (h == 0)
+        for (int q = q0; q < nr; q += rows)
+            if (!fl[q]) {
+                const double x = Pn[q * LU_NBP];
+                lu_pick(bk, br, bx, lu_key(x), r0 + q, x);
+            }
     for (int jj = 0; jj < nbk; ++jj) {
         const int par = jj & 1;
-        for (int o = 16; o > 0; o >>= 1) {
-            const unsigned long long ok = __shfl_xor_sync(0xffffffffu, bk, o);
-            const int orr = __shfl_xor_sync(0xffffffffu, br, o);
-            const double ox = __shfl_xor_sync(0xffffffffu, bx, o);
-            lu_pick(bk, br, bx, ok, orr, ox);
+        {
+            const int src = lu_warp_best(bk, br);
+            const double x = __shfl_sync(0xffffffffu, bx, src);
+            if (lane < CS) {
+                const int slot = rank * 8 + wid;
+                *cl.map_shared_rank(&cand_k[par][slot], lane) = bk;
+                *cl.map_shared_rank(&cand_x[par][slot], lane) = x;
+                *cl.map_shared_rank(&cand_r[par][slot], lane) = br;
+            }
         }
-        if (lane == 0) {
-            cand_k[par][wid] = (br == INT_MAX) ? 0ULL : bk;
-            cand_r[par][wid] = br;
-            cand_x[par][wid] = bx;
-        }
-        cl.sync();  // every warp's candidate is published
+        cl.sync();  // every warp's candidate has arrived, and every row update of the last step is done
         if (wid == 0) {
-            // the winner over the cluster's 8 x CS warp candidates (4 per lane), then the pivot
-            // row straight from the owner's shared memory (a pivoted row is never written again)
             unsigned long long k = 0;
-            int r = INT_MAX;
-            double x = 0.0;
+            int r = INT_MAX, slot = 0;
 #pragma unroll
             for (int t = 0; t < (8 * CS + 31) / 32; ++t) {
-                const int slot = lane + 32 * t;
-                if (slot < 8 * CS) {
-                    const int cta = slot % CS, w = slot / CS;
-                    const unsigned long long ok = *cl.map_shared_rank(&cand_k[par][w], cta);
-                    const int orr = *cl.map_shared_rank(&cand_r[par][w], cta);
-                    const double ox = *cl.map_shared_rank(&cand_x[par][w], cta);
-                    if (orr != INT_MAX) lu_pick(k, r, x, ok, orr, ox);
+                const int sl = lane + 32 * t;
+                if (sl < 8 * CS) {
+                    const unsigned long long ok = cand_k[par][sl];
+                    const int orr = cand_r[par][sl];
+                    if (ok > k || (ok == k && orr < r)) {
+                        k = ok;
+                        r = orr;
+                        slot = sl;
+                    }
                 }
             }
-            for (int o = 16; o > 0; o >>= 1) {
-                const unsigned long long ok = __shfl_xor_sync(0xffffffffu, k, o);
-                const int orr = __shfl_xor_sync(0xffffffffu, r, o);
-                const double ox = __shfl_xor_sync(0xffffffffu, x, o);
-                lu_pick(k, r, x, ok, orr, ox);
-            }
-            const bool bad = (k == 0ULL) || (k >= 0x7ff0000000000000ULL) || r >= m;
-            const int p = (r >= m) ? 0 : r;
-            if (lane == jj) s_pinv = bad ? 0.0 : 1.0 / x;  // one FP64 division, overlapping the row read
-            int own = (int)(((long)p * CS) / m);
-            while (own > 0 && (int)((long)m * own / CS) > p) --own;
-            while (own < CS - 1 && (int)((long)m * (own + 1) / CS) <= p) ++own;
+            const int src = lu_warp_best(k, r);
+            slot = __shfl_sync(0xffffffffu, slot, src);
+            const bool bad = (k == 0ULL) || (k >= 0x7ff0000000000000ULL) || r >= m || r < 0;
+            const int own = bad ? 0 : slot >> 3, p = bad ? 0 : r;
             const int pr0 = (int)((long)m * own / CS);
             const double* prow = cl.map_shared_rank(Pn, own) + (size_t)(p - pr0) * LU_NBP;
             if (lane < nbk) L11[jj][lane] = prow[lane];
+            const double pinv = bad ? 0.0 : lu_rcp(cand_x[par][slot]);
             if (lane == 0) {
-                if (bad) s_bad = 1;
-                s_prow[jj] = p;
+                s_pinv = pinv;
                 if (p >= r0 && p < r1) fl[p - r0] = 1;
                 if (rank == 0) perm[j0 + jj] = p;
             }
+            any_bad = any_bad || bad;
         }
         __syncthreads();
         const double pinv = s_pinv;
-        // own unpivoted rows: multiplier into column jj, rank-1 step on the later panel columns
-        // (four independent multiply-adds at a time: FP64 latency is long on this part), and the
+        // own unpivoted rows: multiplier into column jj, rank-1 step on the later panel columns, and the
         // candidate for column jj + 1
         bk = 0;
         br = INT_MAX;
         bx = 0.0;
-        for (int q = tid; q < nr; q += nt) {
-            if (fl[q]) continue;
-            double* __restrict__ row = Pn + q * LU_NBP;
-            const double l = row[jj] * pinv;
-            row[jj] = l;
-            int c = jj + 1;
-            for (; c + 3 < nbk; c += 4) {
-                const double u0 = L11[jj][c], u1 = L11[jj][c + 1], u2 = L11[jj][c + 2], u3 = L11[jj][c + 3];
-                const double v0 = row[c], v1 = row[c + 1], v2 = row[c + 2], v3 = row[c + 3];
+        const int hj = jj & (tpr - 1), c0 = jj + 1 + ((h - (jj + 1)) & (tpr - 1));
+        for (int qb = 0; qb < nr; qb += rows) {
+            const int q = qb + q0;
+            const bool act = q < nr && !fl[q];
+            double* __restrict__ row = Pn + (act ? q : 0) * LU_NBP;
+            double l = 0.0;
+            if (act && h == hj) {
+                l = row[jj] * pinv;
+                row[jj] = l;
+            }
+            l = __shfl_sync(0xffffffffu, l, (lane & ~(tpr - 1)) | hj);
+            if (!act) continue;
+            int c = c0;
+            if (c < nbk) {
+                const double x = row[c] - l * L11[jj][c];
+                row[c] = x;
+                if (c == jj + 1) lu_pick(bk, br, bx, lu_key(x), r0 + q, x);
+                c += tpr;
+            }
+            for (; c + 3 * tpr < nbk; c += 4 * tpr) {
+                const double u0 = L11[jj][c], u1 = L11[jj][c + tpr], u2 = L11[jj][c + 2 * tpr], u3 = L11[jj][c + 3 * tpr];
+                const double v0 = row[c], v1 = row[c + tpr], v2 = row[c + 2 * tpr], v3 = row[c + 3 * tpr];
                 row[c] = v0 - l * u0;
-                row[c + 1] = v1 - l * u1;
-                row[c + 2] = v2 - l * u2;
-                row[c + 3] = v3 - l * u3;
+                row[c + tpr] = v1 - l * u1;
+                row[c + 2 * tpr] = v2 - l * u2;
+                row[c + 3 * tpr] = v3 - l * u3;
             }
-            for (; c < nbk; ++c) row[c] -= l * L11[jj][c];
-            if (jj + 1 < nbk) {
-                const double x = row[jj + 1];
-                lu_pick(bk, br, bx, lu_key(x), r0 + q, x);
-            }
+            for (; c < nbk; c += tpr) row[c] -= l * L11[jj][c];
         }
+        __syncwarp();
     }
     cl.sync();  // no CTA leaves while another may still read its shared memory
-    if (s_bad && tid == 0 && rank == 0) set_err(a.err, DEV_NUMERIC);
+    if (any_bad && lane == 0 && rank == 0) set_err(a.err, DEV_NUMERIC);
     for (int e = tid; e < nr * nbk; e += nt) {
         const int q = e / nbk, c = e - q * nbk;
         A[(long)(r0 + q) * lda + j0 + c] = Pn[q * LU_NBP + c];
     }
     for (int q = tid; q < nr; q += nt) flag[r0 + q] = fl[q];
-    // U12 = L11^{-1} A12 on the pivot rows, columns dealt round-robin over the cluster's CTAs
-    // (the FP64 work of a column is sequential, so every SM should get a share)
-    for (int c = j0 + nbk + rank + CS * tid; c < n; c += CS * nt) {
-        double x[LU_NB];
-#pragma unroll
-        for (int k = 0; k < LU_NB; ++k) x[k] = (k < nbk) ? A[(long)s_prow[k] * lda + c] : 0.0;
-        // right-looking: each step's updates are independent of one another
-#pragma unroll
-        for (int kp = 0; kp + 1 < LU_NB; ++kp)
-#pragma unroll
-            for (int k = kp + 1; k < LU_NB; ++k)
-                if (k < nbk) x[k] -= L11[k][kp] * x[kp];
-#pragma unroll
-        for (int k = 1; k < LU_NB; ++k)
-            if (k < nbk) A[(long)s_prow[k] * lda + c] = x[k];
-    }
 }
 
-// A[r][c] -= sum_k A[r][j0 + k] U12[k][c] for the unpivoted rows r and c in [j0 + nbk, n), with
-// U12[k] the pivot row perm[j0 + k].  64 x 64 tiles, 4 x 4 outputs per thread; grid (row tiles,
-// column tiles, matrix).
+// U12 = L11^{-1} A12 on the pivot rows of a panel, columns [j0 + nbk, n): eight lanes per column, lane h
+// holds the entries h, h + 8, ... (the FP64 work of a column is sequential, so a column spreads over lanes
+// and the columns over the whole GPU).  Grid (16-column blocks, matrix).
+constexpr int LU_UC = 16;
+__global__ void __launch_bounds__(8 * LU_UC) lu_u12_kernel(LuArgs a, int j0, int nbk) {
+    const int mat = blockIdx.y, tid = threadIdx.x, lane = tid & 31, h = tid >> 4, cl = tid & 15;
+    double* A = lu_A(a, mat);
+    const int* perm = a.perm0 + (long)mat * a.pstride + j0;
+    const long lda = a.lda;
+    const int c = j0 + nbk + blockIdx.x * LU_UC + cl, cc = min(c, a.n - 1);
+    __shared__ double L11[LU_NB][LU_NBP];
+    __shared__ double xs[LU_NB][LU_UC];  // finished entries
+    (void)lane;
+    for (int e = tid; e < LU_NB * LU_NB; e += 8 * LU_UC) {
+        const int k = e / LU_NB, kp = e % LU_NB;
+        L11[k][kp] = (k < nbk && kp < k) ? A[(long)perm[k] * lda + j0 + kp] : 0.0;
+    }
+    double v[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) v[t] = (h + 8 * t < nbk) ? A[(long)perm[h + 8 * t] * lda + cc] : 0.0;
+    __syncthreads();
+#pragma unroll
+    for (int kp = 0; kp < LU_NB; ++kp) {
+        if (kp < nbk) {
+            if (h == (kp & 7)) xs[kp][cl] = v[kp >> 3];
+            __syncthreads();
+            const double x = xs[kp][cl];
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+                if (8 * t + 7 > kp) v[t] -= L11[h + 8 * t][kp] * x;  // zero at and before kp
+        }
+    }
+    if (c < a.n)
+#pragma unroll
+        for (int t = 0; t < 4; ++t)
+            if (h + 8 * t < nbk && h + 8 * t > 0) A[(long)perm[h + 8 * t] * lda + c] = v[t];
+}
+
+// A[r][c] -= sum_k A[r][j0 + k] U12[k][c] for the unpivoted rows r and c in [j0 + nbk, n), with U12[k] the
+// pivot row perm[j0 + k].  BM x BN tiles, BM / 16 x BN / 16 outputs per thread; grid (tiles of the unpivoted
+// rows, column tiles, matrix).  A block finds its rows by counting the flags, so no multiply-add goes to a
+// pivoted row (they are the bound: 2 a clock and SM).
+template <int BM, int BN>
 __global__ void __launch_bounds__(256) lu_update_kernel(LuArgs a, int j0, int nbk) {
+    constexpr int TM = BM / 16, TN = BN / 16;
     const int mat = blockIdx.z;
     double* A = lu_A(a, mat);
     const int* perm = a.perm0 + (long)mat * a.pstride;
     const int8_t* flag = a.flag0 + (long)mat * a.pstride;
     const long lda = a.lda;
     const int m = a.m, n = a.n;
-    const int r0 = blockIdx.x * 64, c0 = j0 + nbk + blockIdx.y * 64;
-    __shared__ double Ls[64][LU_NBP];
-    __shared__ double Us[LU_NB][64 + 1];
-    __shared__ int8_t fl[64];
-    const int tid = threadIdx.x, nt = blockDim.x;
-    for (int q = tid; q < 64; q += nt) fl[q] = (r0 + q < m) ? flag[r0 + q] : 1;
-    __syncthreads();
-    for (int e = tid; e < 64 * LU_NB; e += nt) {
-        const int q = e / LU_NB, k = e - q * LU_NB;
-        Ls[q][k] = (k < nbk && !fl[q]) ? A[(long)(r0 + q) * lda + j0 + k] : 0.0;
+    const int f0 = blockIdx.x * BM, c0 = j0 + nbk + blockIdx.y * BN;
+    __shared__ double Ls[BM][LU_NBP];
+    __shared__ double Us[LU_NB][BN + 1];
+    __shared__ int rid[BM];
+    __shared__ int wsum[8];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    for (int q = tid; q < BM; q += 256) rid[q] = -1;
+    for (int base = 0, seen = 0; base < m && seen < f0 + BM; base += 256) {
+        const int r = base + tid;
+        const bool open = r < m && !flag[r];
+        const unsigned ball = __ballot_sync(0xffffffffu, open);
+        if (lane == 0) wsum[wid] = __popc(ball);
+        __syncthreads();
+        int before = seen, all = 0;
+        for (int w = 0; w < 8; ++w) {
+            if (w < wid) before += wsum[w];
+            all += wsum[w];
+        }
+        const int pos = before + __popc(ball & ((1u << lane) - 1u)) - f0;
+        if (open && pos >= 0 && pos < BM) rid[pos] = r;
+        seen += all;
+        __syncthreads();
     }
-    for (int e = tid; e < LU_NB * 64; e += nt) {
-        const int k = e >> 6, c = e & 63;
+    for (int e = tid; e < BM * LU_NB; e += 256) {
+        const int q = e / LU_NB, k = e - q * LU_NB;
+        Ls[q][k] = (k < nbk && rid[q] >= 0) ? A[(long)rid[q] * lda + j0 + k] : 0.0;
+    }
+    for (int e = tid; e < LU_NB * BN; e += 256) {
+        const int k = e / BN, c = e % BN;
         Us[k][c] = (k < nbk && c0 + c < n) ? A[(long)perm[j0 + k] * lda + c0 + c] : 0.0;
     }
     __syncthreads();
     const int tx = tid & 15, ty = tid >> 4;
-    double acc[4][4];
+    double acc[TM][TN];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < TM; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
+        for (int j = 0; j < TN; ++j) acc[i][j] = 0.0;
     for (int k = 0; k < nbk; ++k) {
-        double lv[4], uv[4];
+        double lv[TM], uv[TN];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) lv[i] = Ls[ty + 16 * i][k];
+        for (int i = 0; i < TM; ++i) lv[i] = Ls[ty + 16 * i][k];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) uv[j] = Us[k][tx + 16 * j];
+        for (int j = 0; j < TN; ++j) uv[j] = Us[k][tx + 16 * j];
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < TM; ++i)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] += lv[i] * uv[j];
+            for (int j = 0; j < TN; ++j) acc[i][j] += lv[i] * uv[j];
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int q = ty + 16 * i;
-        if (fl[q]) continue;
+    for (int i = 0; i < TM; ++i) {
+        const int r = rid[ty + 16 * i];
+        if (r < 0) continue;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < TN; ++j) {
             const int c = c0 + tx + 16 * j;
-            if (c < n) A[(long)(r0 + q) * lda + c] -= acc[i][j];
+            if (c < n) A[(long)r * lda + c] -= acc[i][j];
         }
     }
+}
+
+template <int BM, int BN>
+static cudaError_t launch_update(cudaStream_t st, const LuArgs& a, int j0, int nbk, int mr, int nc) {
+    count_launch();
+    lu_update_kernel<BM, BN><<<dim3((mr + BM - 1) / BM, (nc + BN - 1) / BN, a.nmat), 256, 0, st>>>(a, j0, nbk);
+    return cudaGetLastError();
 }
 
 // Pivot rows of the factored tall matrix become unit rows: A[perm[j]][c] = (c == j) for c >= j,
@@ -313,8 +396,10 @@ static cudaError_t launch_panel(cudaStream_t st, const LuArgs& a, int j0, int nb
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
+    int tpr = 8;  // threads per row: all 256 threads busy
+    while (tpr > 1 && rpc * tpr > 256) tpr /= 2;
     count_launch();
-    return cudaLaunchKernelEx(&cfg, lu_panel_kernel<CS>, a, j0, nbk);
+    return cudaLaunchKernelEx(&cfg, lu_panel_kernel<CS>, a, j0, nbk, tpr);
 }
 
 // Cluster size: enough CTAs per matrix that a panel step's FP64 work per SM stays small, few
@@ -370,11 +455,22 @@ cudaError_t launch_lu(cudaStream_t st, const LuArgs& a) {
             default: e = launch_panel<16>(st, a, j0, nbk); break;
         }
         if (e != cudaSuccess) return e;
-        const int nc = a.n - j0 - nbk;
+        const int nc = a.n - j0 - nbk, mr = a.m - j0 - nbk;
         if (nc > 0) {
             count_launch();
-            lu_update_kernel<<<dim3((a.m + 63) / 64, (nc + 63) / 64, a.nmat), 256, 0, st>>>(a, j0, nbk);
+            lu_u12_kernel<<<dim3((nc + LU_UC - 1) / LU_UC, a.nmat), 8 * LU_UC, 0, st>>>(a, j0, nbk);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
+            if (mr <= 0) continue;
+            // the tile whose busiest SM issues the fewest multiply-adds (plus a fixed cost per tile)
+            auto cost = [&](int bm, int bn) {
+                const long t = (long)((mr + bm - 1) / bm) * ((nc + bn - 1) / bn) * a.nmat;
+                return (t + 151) / 152 * (bm * bn + 128);
+            };
+            const long c64 = cost(64, 64), c36 = cost(32, 64), c33 = cost(32, 32);
+            if (c64 <= c36 && c64 <= c33) e = launch_update<64, 64>(st, a, j0, nbk, mr, nc);
+            else if (c36 <= c33) e = launch_update<32, 64>(st, a, j0, nbk, mr, nc);
+            else e = launch_update<32, 32>(st, a, j0, nbk, mr, nc);
+            if (e != cudaSuccess) return e;
         }
     }
     return cudaSuccess;
