@@ -128,6 +128,16 @@ __device__ __forceinline__ void named_barrier_sync(int id, int nthreads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 
+// t[k] by a tree of selects: indexing would move the array out of the registers.
+template <typename T, int R>
+__device__ __forceinline__ T reg_pick(T (&t)[R], int k) {
+#pragma unroll
+    for (int w = R / 2; w >= 1; w /= 2)
+#pragma unroll
+        for (int i = 0; i < w; ++i) t[i] = (k & w) ? t[i + w] : t[i];
+    return t[0];
+}
+
 // Field-change factor Delta = exp(c (x' - x)) - 1 for one site and spin (Sec. II.C).
 __device__ __forceinline__ double field_delta(double c, int x, int xp) {
     return exp(c * (double)(xp - x)) - 1.0;

@@ -2,7 +2,10 @@
 // rank-m product (the G form of Eqs. FinalDelay and BlkFrcBsTnew2):
 //     G_s <- G_s - G_s[:, I] W_s (E_I^T - G_s[I, :]),
 //     W_s  = D_s (1 + (1 - G_s[I, I]) D_s)^{-1},   (D_s)_aa = exp(c_s (x'_a - x_a)) - 1.
+#include <cooperative_groups.h>
 #include <math.h>
+
+#include <mutex>
 
 #include "internal.h"
 
@@ -40,115 +43,177 @@ static WindowBufs flips_layout(unsigned char* scratch, int N) {
     return wb;
 }
 
-// One CTA: validate the sites, then W_s for both spins by Gauss-Jordan with partial pivoting
-// on [M | 1] in shared memory, M = 1 + (1 - G_II) D.  The status word wb.m[1] is rewritten by every
-// call: 0, DEV_ARG (a site outside [0, N)) or DEV_NUMERIC (a zero pivot); on either error wb.m[0]
-// (the product's inner dimension) is 0, so G is left unchanged.
-template <typename T>
-__global__ void __launch_bounds__(1024) flips_W_kernel(const T* __restrict__ Gu, const T* __restrict__ Gd, long ld,
-                                                       int N, const int* sites, const double* delta, int m,
-                                                       WindowBufs wb, int NWC) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int tid = threadIdx.x, nt = blockDim.x;
-    const int AP = 2 * m + 1;
-    T* Aug = (T*)smem_raw;
-    T* colk = Aug + (size_t)m * AP;
-    __shared__ int s_piv, s_bad, s_num;
+// W_s = D_s M_s^{-1}, M_s = 1 + (1 - G_II) D_s, one CTA per spin in a cluster of two, by in-place
+// Gauss-Jordan with partial pivoting.  M lives in registers: thread (rg, cg) holds rows rg + 16 i and columns
+// cg + FC j (FC = 16 or 32), up to MP x MP elements.  Step k takes two block barriers: the holders of column
+// k put it into shared memory; every warp finds the pivot among the rows not used yet (two integer
+// reductions per 32 rows) and the holders of the pivot row put it beside; all threads eliminate.  Rows are
+// not swapped: row piv[k] ends as row k of the inverse, with column k the multiplier of equation piv[k].
+// Bound by the latency of the steps (64 of them took 2 x 130 us in shared memory with five barriers each and
+// both spins in turn).
+// The status word wb.m[1] is rewritten by every call: 0, DEV_ARG (a site outside [0, N)) or DEV_NUMERIC (a
+// zero pivot in either spin); on either error wb.m[0] (the product's inner dimension) is 0, so G is left
+// unchanged.
+__device__ __forceinline__ unsigned long long flips_key(double x) {
+    return (unsigned long long)__double_as_longlong(fabs(x));
+}
+__device__ __forceinline__ unsigned long long flips_key(float x) {
+    return (unsigned long long)__float_as_uint(fabsf(x));
+}
+
+template <typename T, int MP>
+struct FlipsTile {
+    static constexpr int FC = MP > 64 ? 32 : 16, TR = MP / 16, TC = MP / FC, THREADS = 16 * FC;
+};
+
+template <typename T, int MP>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(FlipsTile<T, MP>::THREADS)
+    flips_W_kernel(const T* __restrict__ Gu, const T* __restrict__ Gd, long ld, int N, const int* sites,
+                   const double* delta, int m, WindowBufs wb, int NWC) {
+    using F = FlipsTile<T, MP>;
+    constexpr int FC = F::FC, TR = F::TR, TC = F::TC;
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const int s = (int)cl.block_rank(), tid = threadIdx.x, lane = tid & 31, rg = tid / FC, cgi = tid % FC;
+    const T* G = s ? Gd : Gu;
+    __shared__ int sidx[MP];
+    __shared__ int piv[MP];
+    __shared__ T col[2][MP], row[2][MP];  // by step parity
+    __shared__ int s_bad, s_num;
     if (tid == 0) {
         s_bad = 0;
         s_num = 0;
     }
     __syncthreads();
-    for (int a = tid; a < m; a += nt) {
-        int v = sites[a];
+    for (int a = tid; a < m; a += F::THREADS) {
+        const int v = sites[a];
         if (v < 0 || v >= N) s_bad = 1;
-        wb.idx[a] = (v < 0 || v >= N) ? 0 : v;
+        sidx[a] = (v < 0 || v >= N) ? 0 : v;
+        if (s == 0) wb.idx[a] = sidx[a];
     }
     __syncthreads();
-    if (s_bad) {  // nothing is applied: the product below sees m = 0
-        if (tid == 0) {
-            wb.m[0] = 0;
-            wb.m[1] = DEV_ARG;
-        }
-        return;
-    }
-    if (tid == 0) {
-        wb.m[0] = m;
-        wb.m[1] = 0;
-    }
-    const T* G[2] = {Gu, Gd};
-    for (int s = 0; s < 2; ++s) {
-        for (int e = tid; e < m * m; e += nt) {
-            int a = e / m, c = e % m;
-            double A0 = (a == c ? 1.0 : 0.0) - (double)G[s][(long)wb.idx[a] * ld + wb.idx[c]];
-            Aug[a * AP + c] = (T)((a == c ? 1.0 : 0.0) + A0 * delta[s * m + c]);
-            Aug[a * AP + m + c] = (a == c) ? T(1) : T(0);
-        }
-        __syncthreads();
+    if (!s_bad) {
+        T A[TR][TC];
+#pragma unroll
+        for (int i = 0; i < TR; ++i)
+#pragma unroll
+            for (int j = 0; j < TC; ++j) {
+                const int r = rg + 16 * i, c = cgi + FC * j;
+                A[i][j] = T(0);
+                if (r < m && c < m) {
+                    const double a0 = (r == c ? 1.0 : 0.0) - (double)G[(long)sidx[r] * ld + sidx[c]];
+                    A[i][j] = (T)((r == c ? 1.0 : 0.0) + a0 * delta[s * m + c]);
+                }
+            }
+        unsigned used[MP / 32];  // rows taken as pivots (the same in every thread)
+#pragma unroll
+        for (int w = 0; w < MP / 32; ++w) used[w] = 0u;
+        bool singular = false;
         for (int k = 0; k < m; ++k) {
-            if (tid < 32) {
-                T best = T(-1);
-                int br = k;
-                for (int r = k + tid; r < m; r += 32) {
-                    T v = fabs(Aug[r * AP + k]);
-                    if (v > best) { best = v; br = r; }
-                }
-                for (int o = 16; o > 0; o >>= 1) {
-                    T ob = __shfl_down_sync(0xffffffffu, best, o);
-                    int orr = __shfl_down_sync(0xffffffffu, br, o);
-                    if (ob > best || (ob == best && orr < br)) { best = ob; br = orr; }
-                }
-                if (tid == 0) {
-                    s_piv = br;
-                    if (!(best > T(0))) s_num = 1;
+            const int par = k & 1;
+            if (cgi == k % FC) {
+#pragma unroll
+                for (int i = 0; i < TR; ++i) {
+                    T t[TC];
+#pragma unroll
+                    for (int j = 0; j < TC; ++j) t[j] = A[i][j];
+                    col[par][rg + 16 * i] = reg_pick<T, TC>(t, k / FC);
                 }
             }
             __syncthreads();
-            const int pr = s_piv;
-            if (pr != k)
-                for (int c = tid; c < 2 * m; c += nt) {
-                    T t0 = Aug[k * AP + c];
-                    Aug[k * AP + c] = Aug[pr * AP + c];
-                    Aug[pr * AP + c] = t0;
+            // the largest entry of the unused rows, ties to the lower row
+            unsigned long long best = 0;
+            int p = MP;
+#pragma unroll
+            for (int w = 0; w < MP / 32; ++w) {
+                const int r = lane + 32 * w;
+                if (r < m && !((used[w] >> lane) & 1u)) {
+                    const unsigned long long key = flips_key(col[par][r]) + 1;  // above "no row"
+                    if (key > best) {
+                        best = key;
+                        p = r;
+                    }
                 }
-            __syncthreads();
-            const T inv = T(1) / Aug[k * AP + k];
-            for (int r = tid; r < m; r += nt) colk[r] = Aug[r * AP + k];
-            __syncthreads();
-            for (int c = tid; c < 2 * m; c += nt) Aug[k * AP + c] *= inv;
-            __syncthreads();
-            for (int e = tid; e < m * 2 * m; e += nt) {
-                int r = e / (2 * m), c = e % (2 * m);
-                if (r == k) continue;
-                Aug[r * AP + c] -= colk[r] * Aug[k * AP + c];
             }
+            const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(best >> 32));
+            const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(best >> 32) == hi ? (unsigned)best : 0u);
+            const bool mine = best == (((unsigned long long)hi << 32) | lo);
+            p = (int)__reduce_min_sync(0xffffffffu, mine ? (unsigned)p : 0xffffffffu);
+            const T pv = col[par][p];
+            if (!(fabs(pv) > T(0))) singular = true;
+#pragma unroll
+            for (int w = 0; w < MP / 32; ++w)
+                if (w == p >> 5) used[w] |= 1u << (p & 31);
+            if (tid == 0) piv[k] = p;
+            if (rg == (p & 15)) {
+#pragma unroll
+                for (int j = 0; j < TC; ++j) {
+                    T t[TR];
+#pragma unroll
+                    for (int i = 0; i < TR; ++i) t[i] = A[i][j];
+                    row[par][cgi + FC * j] = reg_pick<T, TR>(t, p >> 4);
+                }
+            }
+            const T inv = T(1) / pv;
             __syncthreads();
-        }
-        T* Wm = (T*)wb.Wm + (size_t)s * NWC * NWC;
-        for (int e = tid; e < m * m; e += nt) {
-            int a = e / m, c = e % m;
-            Wm[a * NWC + c] = (T)(delta[s * m + a] * (double)Aug[a * AP + m + c]);
+            // pivot row scaled by 1 / pivot (its column k: 1 / pivot), the others minus their column entry times it
+#pragma unroll
+            for (int j = 0; j < TC; ++j) {
+                const int c = cgi + FC * j;
+                const T rv = c == k ? inv : row[par][c] * inv;
+#pragma unroll
+                for (int i = 0; i < TR; ++i) {
+                    const int r = rg + 16 * i;
+                    const T f = col[par][r];
+                    if (r == p) A[i][j] = rv;
+                    else A[i][j] = c == k ? -f * rv : A[i][j] - f * rv;
+                }
+            }
         }
         __syncthreads();
+        // inverse[k][piv[j]] = A[piv[k]][j]: put M^{-1} D in place through the pivot order
+        T* Wm = (T*)wb.Wm + (size_t)s * NWC * NWC;
+#pragma unroll
+        for (int i = 0; i < TR; ++i) {
+            const int r = rg + 16 * i;
+            int k = -1;
+            if (r < m)
+                for (int q = 0; q < m; ++q)
+                    if (piv[q] == r) k = q;
+#pragma unroll
+            for (int j = 0; j < TC; ++j) {
+                const int c = cgi + FC * j;
+                if (k >= 0 && c < m) Wm[k * NWC + piv[c]] = (T)(delta[s * m + k] * (double)A[i][j]);
+            }
+        }
+        if (singular && tid == 0) s_num = 1;
     }
-    if (tid == 0 && s_num) {  // singular: apply nothing
-        wb.m[0] = 0;
-        wb.m[1] = DEV_NUMERIC;
+    cl.sync();
+    if (s == 0 && tid == 0) {
+        const int num = s_num | *cl.map_shared_rank(&s_num, 1);
+        wb.m[0] = (s_bad || num) ? 0 : m;
+        wb.m[1] = s_bad ? DEV_ARG : num ? DEV_NUMERIC : 0;
     }
+    cl.sync();  // spin down's status is read before its CTA leaves
+}
+
+template <typename T, int MP>
+static cudaError_t launch_flips_W(cudaStream_t st, const T* Gu, const T* Gd, long ld, int N, const int* sites,
+                                  const double* delta, int m, WindowBufs wb) {
+    count_launch();
+    flips_W_kernel<T, MP><<<2, FlipsTile<T, MP>::THREADS, 0, st>>>(Gu, Gd, ld, N, sites, delta, m, wb, window_max<T>());
+    return cudaGetLastError();
 }
 
 template <typename T>
 static cudaError_t apply_flips_impl(cudaStream_t st, int N, long ld, T* Gu, T* Gd, const int* sites,
                                     const double* delta, int m, unsigned char* scratch) {
-    const int NWC = window_max<T>();
     WindowBufs wb = flips_layout<T>(scratch, N);
-    size_t shm = (size_t)m * (2 * (size_t)m + 1) * sizeof(T) + (size_t)m * sizeof(T);
-    const size_t mx = (size_t)NWC * (2 * (size_t)NWC + 1) * sizeof(T) + (size_t)NWC * sizeof(T);
-    cudaError_t e = ensure_smem_attr((const void*)flips_W_kernel<T>, mx);
-    if (e != cudaSuccess) return e;
-    count_launch();
-    flips_W_kernel<T><<<1, 1024, shm, st>>>(Gu, Gd, ld, N, sites, delta, m, wb, NWC);
-    e = cudaGetLastError();
+    cudaError_t e;
+    if (m <= 32) e = launch_flips_W<T, 32>(st, Gu, Gd, ld, N, sites, delta, m, wb);
+    else if (m <= 64) e = launch_flips_W<T, 64>(st, Gu, Gd, ld, N, sites, delta, m, wb);
+    else if constexpr (sizeof(T) == 4) e = launch_flips_W<T, 128>(st, Gu, Gd, ld, N, sites, delta, m, wb);
+    else e = cudaErrorInvalidValue;
     if (e != cudaSuccess) return e;
     SiteParams sp{};
     sp.N = N;
@@ -177,6 +242,43 @@ static int flips_check(int precision, int N, long long ld, void* G_up, void* G_d
     return AFQMC_OK;
 }
 
+// The scratch of afqmc_apply_flips comes from a memory pool of its own per device that keeps up to
+// FLIPS_POOL_KEEP bytes between calls (what a call on the largest common lattices needs): the device's
+// default pool gives everything back at the call's synchronisation, and mapping the memory again cost
+// about 200 us a call.  Allocation stays ordered on the call's stream, so calls on several streams and threads
+// never share a buffer; anything above the bound goes back at the next synchronisation.
+constexpr uint64_t FLIPS_POOL_KEEP = 16u << 20;
+
+static cudaError_t flips_alloc(void** p, size_t bytes, cudaStream_t st) {
+    constexpr int MAXDEV = 64;
+    static std::mutex mu;
+    static cudaMemPool_t pools[MAXDEV] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= MAXDEV) return cudaMallocAsync(p, bytes, st);
+    cudaMemPool_t pool = nullptr;
+    {
+        std::lock_guard<std::mutex> lk(mu);
+        if (!pools[dev]) {
+            cudaMemPoolProps props = {};
+            props.allocType = cudaMemAllocationTypePinned;
+            props.location.type = cudaMemLocationTypeDevice;
+            props.location.id = dev;
+            uint64_t keep = FLIPS_POOL_KEEP;
+            cudaMemPool_t made = nullptr;
+            if ((e = cudaMemPoolCreate(&made, &props)) != cudaSuccess) return e;
+            if ((e = cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) {
+                cudaMemPoolDestroy(made);
+                return e;
+            }
+            pools[dev] = made;
+        }
+        pool = pools[dev];
+    }
+    return cudaMallocFromPoolAsync(p, bytes, pool, st);
+}
+
 }  // namespace afq
 
 using namespace afq;
@@ -189,7 +291,7 @@ extern "C" int afqmc_apply_flips(int precision, int N, long long ld, void* G_up,
     cudaStream_t st = (cudaStream_t)stream;
     const size_t bytes = precision == AFQMC_PREC_FP64 ? flips_scratch_bytes<double>(N) : flips_scratch_bytes<float>(N);
     void* scratch = nullptr;
-    if (cudaMallocAsync(&scratch, bytes, st) != cudaSuccess) return AFQMC_ERR_OOM;
+    if (flips_alloc(&scratch, bytes, st) != cudaSuccess) return AFQMC_ERR_OOM;
     cudaError_t e = precision == AFQMC_PREC_FP64
                         ? apply_flips_impl<double>(st, N, (long)ld, (double*)G_up, (double*)G_dn, sites, delta, m,
                                                    (unsigned char*)scratch)
@@ -234,8 +336,6 @@ constexpr size_t NOALLOC_BYTES = NOALLOC_BYTES_F32 > NOALLOC_BYTES_F64 ? NOALLOC
 static __device__ __align__(256) unsigned char g_flips_scratch[NOALLOC_BYTES];
 
 }  // namespace afq
-
-#include <mutex>
 
 namespace {
 constexpr int NOALLOC_MAXDEV = 64;

@@ -399,16 +399,6 @@ struct FlipConsts {
     T dflip[2][2], sflip[2];
 };
 
-// t[k] by a tree of selects: indexing would move the array out of the registers.
-template <typename T, int R>
-__device__ __forceinline__ T reg_pick(T (&t)[R], int k) {
-#pragma unroll
-    for (int w = R / 2; w >= 1; w /= 2)
-#pragma unroll
-        for (int i = 0; i < w; ++i) t[i] = (k & w) ? t[i + w] : t[i];
-    return t[0];
-}
-
 // x / y for the accept factor.  FP32: the approximate reciprocal of the device and one step of residual
 // correction (q += (x - q y) / y), straight-line code that overlaps the block's update.  FP64: a 22-bit
 // reciprocal of y's leading bits, taken in FP32 from its bit pattern, and one step of Halley's iteration
