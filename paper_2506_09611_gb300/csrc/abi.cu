@@ -2089,16 +2089,15 @@ int afqmc_get_G(afqmc_ctx* ctx, int walker, int spin, double* host_out) {
         if (ctx->p.precision == AFQMC_PREC_FP64) CK(tform_form_G<double>(w, ctx->last));
         else CK(tform_form_G<float>(w, ctx->last));
     }
+    // widened and packed on the device, in this matrix's part of the recompute's scratch (rewritten by every
+    // recompute before it is read), then one copy: the host loop over N^2 elements took 5 ms at 40 x 40
+    const size_t es = esize(ctx), N = (size_t)w->N, z = (size_t)j * 2 + spin;
+    const char* src = (const char*)w->G + z * N * w->ld * es;
+    double* pk = w->Gnew + z * N * w->ld;
+    if (es == 8) CK(launch_to_double<double>(ctx->last, (const double*)src, w->ld, pk, w->N, w->N, w->N));
+    else CK(launch_to_double<float>(ctx->last, (const float*)src, w->ld, pk, w->N, w->N, w->N));
+    CK(cudaMemcpyAsync(host_out, pk, N * N * 8, cudaMemcpyDeviceToHost, ctx->last));
     CK(cudaStreamSynchronize(ctx->last));
-    const size_t es = esize(ctx);
-    std::vector<char> buf((size_t)w->N * w->ld * es);
-    CK(cudaMemcpy(buf.data(), (char*)w->G + ((size_t)j * 2 + spin) * w->N * w->ld * es, buf.size(),
-                  cudaMemcpyDeviceToHost));
-    for (int i = 0; i < w->N; ++i)
-        for (int c = 0; c < w->N; ++c) {
-            size_t o = (size_t)i * w->ld + c;
-            host_out[(size_t)i * w->N + c] = (es == 8) ? ((double*)buf.data())[o] : (double)((float*)buf.data())[o];
-        }
     return read_dev_err(ctx, w);
 }
 

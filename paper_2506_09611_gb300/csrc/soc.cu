@@ -1222,6 +1222,16 @@ __global__ void soc_fields_kernel(uint64_t seed, long count, int8_t* x) {
     if (j < count) x[(long)w * count + j] = philox_uniform(seed, (uint64_t)w, 0x5F1E1DULL, (uint64_t)j) < 0.5 ? 1 : -1;
 }
 
+// out[r][c] = (re, im) in FP64 of a row-split matrix (one block per row).
+template <typename T>
+__global__ void soc_interleave_kernel(const T* G, long ldz, int N2, double* out) {
+    const long r = blockIdx.x;
+    for (int c = threadIdx.x; c < N2; c += blockDim.x) {
+        const double2 v = make_double2((double)G[r * 2 * ldz + c], (double)G[r * 2 * ldz + ldz + c]);
+        *(double2*)(out + 2 * (r * N2 + c)) = v;
+    }
+}
+
 __global__ void soc_iota_kernel(int* g, int n) {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j < n) g[j] = j;
@@ -2134,24 +2144,18 @@ int afqmc_soc_get_G(afqmc_soc_ctx* ctx, int walker, double* out) {
     int rc = soc_sync_walker(ctx, walker);
     if (rc) return rc;
     if (!out) return AFQMC_ERR_ARG;
+    // interleaved on the device, in the walker's part of the recompute's scratch (rewritten by every
+    // recompute before it is read), then one copy
     const int N2 = ctx->N2;
-    const long ld2 = 2 * ctx->ldz;
     const size_t es = ctx->f64 ? 8 : 4;
-    std::vector<unsigned char> h((size_t)N2 * ld2 * es);
-    SCK(cudaMemcpy(h.data(), (char*)ctx->G + (size_t)walker * ctx->gstride() * es, h.size(), cudaMemcpyDeviceToHost));
-    for (int r = 0; r < N2; ++r)
-        for (int c = 0; c < N2; ++c) {
-            double re, im;
-            if (ctx->f64) {
-                re = ((double*)h.data())[(size_t)r * ld2 + c];
-                im = ((double*)h.data())[(size_t)r * ld2 + ctx->ldz + c];
-            } else {
-                re = ((float*)h.data())[(size_t)r * ld2 + c];
-                im = ((float*)h.data())[(size_t)r * ld2 + ctx->ldz + c];
-            }
-            out[((size_t)r * N2 + c) * 2] = re;
-            out[((size_t)r * N2 + c) * 2 + 1] = im;
-        }
+    const void* src = (const char*)ctx->G + (size_t)walker * ctx->gstride() * es;
+    double* pk = ctx->Pb + (size_t)walker * 2 * N2 * N2;
+    count_launch();
+    if (ctx->f64) soc_interleave_kernel<double><<<N2, 256, 0, ctx->last>>>((const double*)src, ctx->ldz, N2, pk);
+    else soc_interleave_kernel<float><<<N2, 256, 0, ctx->last>>>((const float*)src, ctx->ldz, N2, pk);
+    SCK(cudaGetLastError());
+    SCK(cudaMemcpyAsync(out, pk, (size_t)N2 * N2 * 16, cudaMemcpyDeviceToHost, ctx->last));
+    SCK(cudaStreamSynchronize(ctx->last));
     return AFQMC_OK;
 }
 
