@@ -495,13 +495,24 @@ cudaError_t launch_lu_sign(cudaStream_t st, const LuArgs& a, int parity, double*
 // and U[j][j..ns)) and B (ns x N), both matrices of the batch:
 //   forward  y_j = B[perm[j]] - sum_{k<j} L[j][k] y_k,
 //   backward z_j = (y_j - sum_{k>j} U[j][k] z_k) / U[j][j],   Z[j] = z_j.
-// The right-hand sides are independent: each CTA owns SV_COLS columns in shared memory and
-// walks the rows in blocks of 32 (a product with the finished rows, then the 32 x 32 diagonal
-// block column by column).  Grid (column blocks, matrix).
+// The right-hand sides are independent: one warp per column.  The column lives in shared memory; a block of
+// 32 rows is one row per lane: the products with the finished rows (coefficients staged for the whole CTA in
+// 32 x SV_KB tiles, the next one copied asynchronously under the current one), then the 32 x 32 diagonal block
+// by shuffles.  Bound by the FP64 multiply-adds (2 a clock and SM), so what counts is that every partition of
+// the SM has the same work: with the pivot-ordered identity column c costs its forward substitution from row
+// c on, and a CTA takes as many columns from the front as from the back.  (With ten contiguous columns per CTA,
+// ten columns of one row block dealt over eight warps, the inverse of two 700 x 700 matrices took 2.43 ms.)
+// Grid (column blocks, matrix).
 // ---------------------------------------------------------------------------
-constexpr int SV_COLS = 10, SV_YP = SV_COLS + 1, SV_KB = 64;
+constexpr int SV_KB = 64, SV_LP = SV_KB + 1;
 
-__global__ void __launch_bounds__(256) lu_solve_kernel(SolveArgs a) {
+__device__ __forceinline__ void sv_cp_async(double* dst, const double* src, bool in) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    const int sz = in ? 8 : 0;
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(src), "r"(sz) : "memory");
+}
+
+__global__ void __launch_bounds__(320) lu_solve_kernel(SolveArgs a) {
     const int mat = blockIdx.y;
     const double* LU = a.LU0 + (long)mat * a.ostride;
     const int* perm = a.perm0 + (long)mat * a.pstride;
@@ -509,121 +520,139 @@ __global__ void __launch_bounds__(256) lu_solve_kernel(SolveArgs a) {
     double* Z = a.Z0 + (long)mat * a.zstride;
     const int ns = a.ns, N = a.N;
     const long ldl = a.ldl, ldb = a.ldb ? a.ldb : N;
-    const int c0 = blockIdx.x * SV_COLS, nc = min(SV_COLS, N - c0);
-    const int tid = threadIdx.x, nt = blockDim.x;
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, w = tid >> 5, nc = nt >> 5;
+    const bool eye = a.eye != 0;
+    // this warp's column: contiguous, or (identity) half from the front and half from the back
+    const int half = nc / 2;
+    int c = blockIdx.x * nc + w;
+    bool own = c < N;
+    if (eye) {
+        const int f = blockIdx.x * half + (w < half ? w : w - half);
+        c = w < half ? f : N - 1 - f;
+        own = w < half ? f < (N + 1) / 2 : f < N / 2;
+    }
     extern __shared__ __align__(16) double sv_smem[];
-    double* y = sv_smem;                        // [ns][SV_YP]
-    double* Lc = y + (size_t)ns * SV_YP;        // [32][SV_KB + 1]
-    double* rinv = Lc + 32 * (SV_KB + 1);       // [ns]
-    int* sp = (int*)(rinv + ns);                // [ns]
+    double* Lt = sv_smem;                       // [2][32][SV_LP] coefficient tiles
+    double* rinv = Lt + 2 * 32 * SV_LP;         // [ns]
+    double* y = rinv + ns + (size_t)w * ns;     // [ns] the column
+    int* sp = (int*)(rinv + ns + (size_t)nc * ns);  // [ns]
     for (int j = tid; j < ns; j += nt) sp[j] = perm[j];
     __syncthreads();
-    const bool eye = a.eye != 0;
-    for (int e = tid; e < ns * SV_COLS; e += nt) {
-        const int j = e / SV_COLS, c = e - j * SV_COLS;
-        y[j * SV_YP + c] = (c < nc) ? (eye ? (j == c0 + c ? 1.0 : 0.0) : B[(long)sp[j] * ldb + c0 + c]) : 0.0;
-    }
     for (int j = tid; j < ns; j += nt) rinv[j] = 1.0 / LU[(long)sp[j] * ldl + j];
+    if (eye) {
+        for (int j = lane; j < ns; j += 32) y[j] = j == c ? 1.0 : 0.0;
+    } else {  // rows by warps, the CTA's columns by lanes
+        double* y0 = rinv + ns;
+        const int cb = blockIdx.x * nc;
+        for (int j = w; j < ns; j += nc)
+            if (lane < nc) y0[(size_t)lane * ns + j] = cb + lane < N ? B[(long)sp[j] * ldb + cb + lane] : 0.0;
+    }
+    const int nb = (ns + 31) / 32;
+    const int first = eye ? (blockIdx.x * half) / 32 : 0;         // first block any column of the CTA needs
+    const int mine = !own ? nb : (eye ? c / 32 : 0);              // first block this column needs
+    // tile (rows J0.., columns k0 ..): coefficient rows are the pivot rows
+    auto fetch = [&](int buf, int J0, int k0) {
+        for (int r = w; r < 32; r += nc)
+            for (int k = lane; k < SV_KB; k += 32) {
+                const bool in = J0 + r < ns && k0 + k < ns;
+                sv_cp_async(Lt + (buf * 32 + r) * SV_LP + k, in ? LU + (long)sp[J0 + r] * ldl + k0 + k : LU, in);
+            }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    auto arrived = [&] {
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+    };
     __syncthreads();
-    // forward substitution (unit lower L); with the pivot-ordered identity every y_j with j < c0
-    // is zero in this block of columns, so the rows above c0 and their products are skipped
-    const int j_first = eye ? c0 : 0;
-    for (int J0 = (j_first / 32) * 32; J0 < ns; J0 += 32) {
-        const int jb = min(32, ns - J0);
-        for (int k0 = (j_first / SV_KB) * SV_KB; k0 < J0; k0 += SV_KB) {
-            const int kb = min(SV_KB, J0 - k0);
-            for (int e = tid; e < jb * SV_KB; e += nt) {
-                const int r = e / SV_KB, k = e - r * SV_KB;
-                Lc[r * (SV_KB + 1) + k] = (k < kb) ? LU[(long)sp[J0 + r] * ldl + k0 + k] : 0.0;
-            }
-            __syncthreads();
-            for (int e = tid; e < jb * SV_COLS; e += nt) {
-                const int r = e / SV_COLS, c = e - r * SV_COLS;
-                double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;  // independent chains (FP64 latency)
-                int k = 0;
-                for (; k + 3 < kb; k += 4) {
-                    a0 += Lc[r * (SV_KB + 1) + k] * y[(k0 + k) * SV_YP + c];
-                    a1 += Lc[r * (SV_KB + 1) + k + 1] * y[(k0 + k + 1) * SV_YP + c];
-                    a2 += Lc[r * (SV_KB + 1) + k + 2] * y[(k0 + k + 2) * SV_YP + c];
-                    a3 += Lc[r * (SV_KB + 1) + k + 3] * y[(k0 + k + 3) * SV_YP + c];
+    int buf = 0;
+    // forward substitution (unit lower L), then backward (U): block rows jb, coefficient tiles of the finished
+    // columns, then the diagonal block
+    for (int dir = 0; dir < 2; ++dir) {
+        const int b0 = dir ? nb - 1 : first, b1 = dir ? -1 : nb, step = dir ? -1 : 1;
+        for (int jb = b0; jb != b1; jb += step) {
+            const int J0 = jb * 32, row = J0 + lane;
+            // finished columns: [first block, J0) forward, [J0 + 32, ns) backward, in SV_KB steps
+            const int ks = dir ? J0 + 32 : first * 32, ke = dir ? ns : J0;
+            const bool work = own && (dir || jb >= mine);
+            double v = (work && row < ns) ? y[row] : 0.0;
+            fetch(buf, J0, ks < ke ? ks : J0);
+            for (int k0 = ks; k0 < ke; k0 += SV_KB) {
+                arrived();
+                const double* Lc = Lt + (buf * 32 + lane) * SV_LP;
+                buf ^= 1;
+                fetch(buf, J0, k0 + SV_KB < ke ? k0 + SV_KB : J0);  // the next tile, at last the diagonal block
+                const int kb = min(SV_KB, ke - k0);
+                if (work && (dir || k0 + kb > mine * 32)) {
+                    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;  // independent chains (FP64 latency)
+                    int k = 0;
+                    for (; k + 3 < kb; k += 4) {
+                        a0 += Lc[k] * y[k0 + k];
+                        a1 += Lc[k + 1] * y[k0 + k + 1];
+                        a2 += Lc[k + 2] * y[k0 + k + 2];
+                        a3 += Lc[k + 3] * y[k0 + k + 3];
+                    }
+                    for (; k < kb; ++k) a0 += Lc[k] * y[k0 + k];
+                    v -= (a0 + a1) + (a2 + a3);
                 }
-                for (; k < kb; ++k) a0 += Lc[r * (SV_KB + 1) + k] * y[(k0 + k) * SV_YP + c];
-                y[(J0 + r) * SV_YP + c] -= (a0 + a1) + (a2 + a3);
             }
-            __syncthreads();
-        }
-        for (int e = tid; e < jb * 32; e += nt) {
-            const int r = e >> 5, k = e & 31;
-            Lc[r * (SV_KB + 1) + k] = (k < jb) ? LU[(long)sp[J0 + r] * ldl + J0 + k] : 0.0;
-        }
-        __syncthreads();
-        for (int rp = 0; rp + 1 < jb; ++rp) {  // diagonal block, right-looking
-            for (int e = tid; e < (jb - rp - 1) * SV_COLS; e += nt) {
-                const int r = rp + 1 + e / SV_COLS, c = e % SV_COLS;
-                y[(J0 + r) * SV_YP + c] -= Lc[r * (SV_KB + 1) + rp] * y[(J0 + rp) * SV_YP + c];
-            }
-            __syncthreads();
-        }
-    }
-    // backward substitution (U)
-    const int nblk = (ns + 31) / 32;
-    for (int bj = nblk - 1; bj >= 0; --bj) {
-        const int J0 = bj * 32, jb = min(32, ns - J0), J1 = J0 + jb;
-        for (int k0 = J1; k0 < ns; k0 += SV_KB) {
-            const int kb = min(SV_KB, ns - k0);
-            for (int e = tid; e < jb * SV_KB; e += nt) {
-                const int r = e / SV_KB, k = e - r * SV_KB;
-                Lc[r * (SV_KB + 1) + k] = (k < kb) ? LU[(long)sp[J0 + r] * ldl + k0 + k] : 0.0;
-            }
-            __syncthreads();
-            for (int e = tid; e < jb * SV_COLS; e += nt) {
-                const int r = e / SV_COLS, c = e - r * SV_COLS;
-                double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-                int k = 0;
-                for (; k + 3 < kb; k += 4) {
-                    a0 += Lc[r * (SV_KB + 1) + k] * y[(k0 + k) * SV_YP + c];
-                    a1 += Lc[r * (SV_KB + 1) + k + 1] * y[(k0 + k + 1) * SV_YP + c];
-                    a2 += Lc[r * (SV_KB + 1) + k + 2] * y[(k0 + k + 2) * SV_YP + c];
-                    a3 += Lc[r * (SV_KB + 1) + k + 3] * y[(k0 + k + 3) * SV_YP + c];
+            arrived();
+            const double* Ld = Lt + (buf * 32 + lane) * SV_LP;  // row `lane` of the diagonal block
+            const int jn = min(32, ns - J0);
+            if (work) {
+                if (dir == 0) {
+                    for (int k = 0; k + 1 < jn; ++k) {
+                        const double x = __shfl_sync(0xffffffffu, v, k);
+                        if (lane > k && lane < jn) v -= Ld[k] * x;
+                    }
+                } else {
+                    const double ri = lane < jn ? rinv[row] : 0.0;
+                    for (int k = jn - 1; k >= 0; --k) {
+                        if (lane == k) v *= ri;
+                        const double x = __shfl_sync(0xffffffffu, v, k);
+                        if (lane < k) v -= Ld[k] * x;
+                    }
                 }
-                for (; k < kb; ++k) a0 += Lc[r * (SV_KB + 1) + k] * y[(k0 + k) * SV_YP + c];
-                y[(J0 + r) * SV_YP + c] -= (a0 + a1) + (a2 + a3);
+                if (lane < jn) y[row] = v;
             }
-            __syncthreads();
+            buf ^= 1;
         }
-        for (int e = tid; e < jb * 32; e += nt) {
-            const int r = e >> 5, k = e & 31;
-            Lc[r * (SV_KB + 1) + k] = (k < jb) ? LU[(long)sp[J0 + r] * ldl + J0 + k] : 0.0;
-        }
-        __syncthreads();
-        for (int rp = jb - 1; rp >= 1; --rp) {  // diagonal block, right-looking: z_rp = y_rp / U_rp,rp
-            for (int e = tid; e < rp * SV_COLS; e += nt) {
-                const int r = e / SV_COLS, c = e % SV_COLS;
-                y[(J0 + r) * SV_YP + c] -= Lc[r * (SV_KB + 1) + rp] * (y[(J0 + rp) * SV_YP + c] * rinv[J0 + rp]);
-            }
-            __syncthreads();
-        }
-        for (int e = tid; e < jb * SV_COLS; e += nt) {
-            const int r = e / SV_COLS, c = e % SV_COLS;
-            y[(J0 + r) * SV_YP + c] *= rinv[J0 + r];
-        }
-        __syncthreads();
+        __syncwarp();
     }
-    for (int e = tid; e < ns * SV_COLS; e += nt) {
-        const int j = e / SV_COLS, c = e - j * SV_COLS;
-        if (c < nc) Z[(long)j * N + (eye ? sp[c0 + c] : c0 + c)] = y[j * SV_YP + c];
+    __syncthreads();
+    if (eye) {
+        if (own)
+            for (int j = lane; j < ns; j += 32) Z[(long)j * N + sp[c]] = y[j];
+    } else {
+        const double* y0 = rinv + ns;
+        const int cb = blockIdx.x * nc;
+        for (int j = w; j < ns; j += nc)
+            if (lane < nc && cb + lane < N) Z[(long)j * N + cb + lane] = y0[(size_t)lane * ns + j];
     }
 }
 
 cudaError_t launch_lu_solve(cudaStream_t st, const SolveArgs& a) {
-    const size_t shm = ((size_t)a.ns * SV_YP + 32 * (SV_KB + 1) + a.ns) * sizeof(double) + (size_t)a.ns * sizeof(int);
-    if (shm > 220 * 1024) return cudaErrorInvalidValue;
+    auto smem = [&](int nc) {
+        return ((size_t)2 * 32 * SV_LP + (size_t)a.ns * (nc + 1)) * sizeof(double) + (size_t)a.ns * sizeof(int);
+    };
+    // columns (warps) per CTA, an even number (the identity's columns come from both ends): the one whose
+    // busiest SM partition has the fewest columns, the larger on a tie (tiles shared by more columns)
+    int nc = 2;
+    long best = 0;
+    for (int k = 10; k >= 2; k -= 2) {
+        if (smem(k) > 220 * 1024) continue;
+        const long t = (((long)((a.N + k - 1) / k) * a.nmat + 151) / 152) * ((k + 3) / 4);
+        if (best == 0 || t < best) {
+            best = t;
+            nc = k;
+        }
+    }
+    if (smem(nc) > 220 * 1024) return cudaErrorInvalidValue;
     {
         cudaError_t e = ensure_smem_attr((const void*)lu_solve_kernel, 220 * 1024);
         if (e != cudaSuccess) return e;
     }
     count_launch();
-    lu_solve_kernel<<<dim3((a.N + SV_COLS - 1) / SV_COLS, a.nmat), 256, shm, st>>>(a);
+    lu_solve_kernel<<<dim3((a.N + nc - 1) / nc, a.nmat), 32 * nc, smem(nc), st>>>(a);
     return cudaGetLastError();
 }
 
