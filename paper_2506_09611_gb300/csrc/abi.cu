@@ -1223,7 +1223,7 @@ static int sweep_impl(afqmc_ctx* ctx, int gi, int ell, int dir, int mode, int k,
                                w->err, ctx->nsm));
         }
     } else {
-        int nw = (mode == AFQMC_MODE_DELAYED) ? k : (NW / nb) * nb;
+        const int nw = (mode == AFQMC_MODE_DELAYED) ? k : window_fb(nb);
         // Window w's decisions and panels run on st; its rank-m product runs on the group's flush
         // stream sf and overlaps the decisions of window w + 1, whose block (as window w's update will
         // leave it) comes with the panels.  Before window w's panels are formed, st waits for the product
@@ -1375,7 +1375,7 @@ static int tform_windows(afqmc_ctx* ctx, Walker* w, cudaStream_t st, int8_t* xl,
     const long sB = (long)NW * NW, sP = (long)NW * ns, sT = (long)ns * ns;
     {
         PhaseScope ps(ctx, AFQMC_PHASE_CHAIN, st);
-        const int nw = (mode == AFQMC_MODE_BLOCKFB || mode == WIN_MODE_CPB) ? (NW / nb) * nb : k;
+        const int nw = (mode == AFQMC_MODE_BLOCKFB || mode == WIN_MODE_CPB) ? window_fb(nb) : k;
         for (int s0 = 0; s0 < N; s0 += nw) {
             const int n = (N - s0 < nw) ? N - s0 : nw;
             // the window's block of G: 1 - (U_R[J, :] T) U_L[:, J]

@@ -261,7 +261,11 @@ struct Batch {
 };
 
 template <typename T>
-int window_max();      // largest window (sites) the chain kernel holds in shared memory
+int window_max();      // largest window (sites) of the delayed update
+// Sites of a window of the block force-bias update (whole blocks of nb <= 32 sites): at most 64, one register
+// tile, and a rank the flush product takes in its small-rank form.
+constexpr int WIN_FB = 64;
+inline int window_fb(int nb) { return WIN_FB / nb * nb; }
 
 // Separable wrap products (sepwrap.cu, code in sepwrap.cuh): G <- (A (x) A) G (side 0) or
 // G <- G (A (x) A) (side 1) for the batch of N x N matrices of a SepArgs, with its optional row /

@@ -705,6 +705,264 @@ __global__ void __launch_bounds__(WinTile<T, NP>::THREADS) window_reg_kernel(
     }
 }
 
+// One window of the block force-bias update (Sec. III.B) in FP32, blocks of nb <= NBP sites, one block per
+// walker.  Warps 0 and 1 decide (one spin each), eight tile warps hold the window's block in registers as in
+// window_reg_kernel.  Per block of sites S:
+//   the tile threads put the S x S diagonal block of both spins into shared memory;
+//   each deciding warp strips the fields (Eq. BlkFrcBsTnew1) on its spin's block in registers, lane r holding
+//   row r: one rank-1 step per site, the registers rotating by one column a step so that the loop is not
+//   unrolled; warp 0 proposes from the stripped densities (FP64, as the ratio); each warp takes
+//   det(1 + D_F A_FF) as the product of the sequential rank-1 ratios on its block (Eq. BlkFrcBsTnew2);
+//   warp 0 accepts or rejects;
+//   the accepted flips go through the tile one by one, one block barrier each, the deciding warps writing the
+//   rows and columns out for panel_kernel.
+// Bound by the latency of that chain: 16 strip steps and about as many ratio steps of one warp per block.
+// The FP64 update spreads its multiply-adds over 32 warps instead (window_kernel).
+template <int NBP>
+__global__ void __launch_bounds__(320) window_fb_kernel(const float* __restrict__ Gu0, int8_t* xl0,
+                                                        const double* __restrict__ u0,
+                                                        const uint8_t* __restrict__ replay0, SiteParams sp,
+                                                        FlipConsts<float> fc, FlipConsts<float> fstrip, SliceOut so0,
+                                                        int s0, int n, int nb, WindowBufs wb0,
+                                                        const float* __restrict__ blk0, int* err, Batch bt) {
+    constexpr int NP = 64, NW = WinCap<float>::NW, RG = 16, TR = 4, TC = 8;
+    constexpr unsigned FULL = 0xffffffffu;
+    const int tid = threadIdx.x, lane = tid & 31, hw = __shfl_sync(FULL, tid >> 5, 0), wk = blockIdx.x, N = sp.N;
+    const WindowBufs wb = wb_walker<float>(wb0, wk, N);
+    const float* G = Gu0 + (size_t)wk * bt.gstride;
+    const float* src0 = blk0 ? blk0 + (size_t)wk * 2 * NW * NW : G + (size_t)s0 * sp.ld + s0;
+    const float* src1 = blk0 ? src0 + NW * NW : src0 + (size_t)N * sp.ld;
+    const long lds = blk0 ? NW : sp.ld;
+    __shared__ float S1[2][NBP][NBP + 1];           // the current block's S x S of both spins
+    __shared__ float srow[2][2][NP], scol[2][2][NP];  // [flip parity][spin]
+    __shared__ float s_phi[2][NBP];                 // Delta / r of the flips, in order
+    __shared__ float s_diag[2][NBP];                // stripped diagonal
+    __shared__ double s_prod[2], s_E[NP];           // ratio products; e^{lm - lp} of every site
+    __shared__ unsigned s_flip;                     // proposed flips of the block (lane mask)
+    __shared__ int s_acc;
+
+    if (hw >= 2) {  // ---- tile warps ----
+        const int w = hw - 2, s = w >> 2, rg = (w & 3) * 4 + (lane >> 3), cg = lane & 7;
+        const float* srcp = s ? src1 : src0;
+        float g[TR][TC];
+#pragma unroll
+        for (int i = 0; i < TR; ++i)
+#pragma unroll
+            for (int j = 0; j < TC; ++j) {
+                const int r = rg + RG * i, c = cg + 8 * j;
+                g[i][j] = (r < n && c < n) ? srcp[r * lds + c] : 0.f;
+            }
+        int par = 0;
+        for (int p0 = 0; p0 < n; p0 += nb) {
+            const int nbk = min(nb, n - p0);
+#pragma unroll
+            for (int i = 0; i < TR; ++i)
+#pragma unroll
+                for (int j = 0; j < TC; ++j) {
+                    const int r = rg + RG * i - p0, c = cg + 8 * j - p0;
+                    if (r >= 0 && r < nbk && c >= 0 && c < nbk) S1[s][r][c] = g[i][j];
+                }
+            __syncthreads();
+            __syncthreads();
+            if (!s_acc) continue;
+            int q = 0;
+            for (unsigned fl = s_flip; fl; fl &= fl - 1, ++q, par ^= 1) {
+                const int a = p0 + __ffs(fl) - 1;
+                if (rg == (a & (RG - 1))) {
+#pragma unroll
+                    for (int j = 0; j < TC; ++j) {
+                        float t[TR];
+#pragma unroll
+                        for (int i = 0; i < TR; ++i) t[i] = g[i][j];
+                        srow[par][s][cg + 8 * j] = reg_pick<float, TR>(t, a / RG);
+                    }
+                }
+                if (cg == (a & 7)) {
+#pragma unroll
+                    for (int i = 0; i < TR; ++i) {
+                        float t[TC];
+#pragma unroll
+                        for (int j = 0; j < TC; ++j) t[j] = g[i][j];
+                        scol[par][s][rg + RG * i] = reg_pick<float, TC>(t, a >> 3);
+                    }
+                }
+                __syncthreads();
+                const float phi = s_phi[s][q];
+                float rv[TC];
+#pragma unroll
+                for (int j = 0; j < TC; ++j) rv[j] = srow[par][s][cg + 8 * j];
+#pragma unroll
+                for (int i = 0; i < TR; ++i) {
+                    const float wv = phi * scol[par][s][rg + RG * i];
+#pragma unroll
+                    for (int j = 0; j < TC; ++j) g[i][j] = fmaf(wv, rv[j], g[i][j]);
+                }
+            }
+        }
+        return;
+    }
+    // ---- deciding warps: spin hw ----
+    const int s = hw;
+    int8_t* xl = xl0 + (size_t)wk * bt.xstride + s0;
+    const double* u = u0 + (size_t)wk * 2 * N;
+    const uint8_t* rep = replay0 ? replay0 + (size_t)wk * 2 * N : nullptr;
+    const SliceOut so = so_walker(so0, wk, N);
+    auto pair_sync = [&] {
+        __syncwarp();
+        named_barrier_sync(2, 64);
+    };
+    float* Wx = (float*)wb.Wx + (size_t)s * NW * NW;
+    float* Wm = (float*)wb.Wm + (size_t)s * NW * NW;
+    int m = 0, n_prop = 0, n_acc = 0, nneg = 0, par = 0;
+    double maxr = 0.0;
+    bool bad = false;
+    for (int p0 = 0; p0 < n; p0 += nb) {
+        const int nbk = min(nb, n - p0), i = s0 + p0 + lane, blk = (s0 + p0) / nb;
+        const bool in = lane < nbk;
+        const int x = in ? xl[p0 + lane] : 1;
+        const double uq = in ? u[i] : 0.0, ua = u[N + blk];
+        const bool forced = rep && in && rep[i] != 0, force_acc = rep && rep[N + blk] != 0;
+        const unsigned xup = __ballot_sync(FULL, x > 0);
+        __syncthreads();  // S1 is there
+        float g[NBP];
+        // (a) stripped force bias: G <- G - (d/r) G[:, a] (e_a^T - G[a, :]) for every site a of the block,
+        //     d = exp(-c x_a) - 1; g[j] is column (a + j) mod NBP
+#pragma unroll
+        for (int j = 0; j < NBP; ++j) g[j] = (in && j < nbk) ? S1[s][lane][j] : 0.f;
+#pragma unroll 1
+        for (int a = 0; a < NBP; ++a) {
+            const float db = (xup >> a) & 1u ? fstrip.dflip[s][0] : fstrip.dflip[s][1];
+            const float r0 = __shfl_sync(FULL, g[0], a);
+            const float rr = 1.f + db * (1.f - r0);
+            const float f = a < nbk ? accept_quot(db, rr) * g[0] : 0.f;
+            const float first = g[0] - f * (1.f - r0);
+#pragma unroll
+            for (int j = 1; j < NBP; ++j) g[j - 1] = fmaf(f, __shfl_sync(FULL, g[j], a), g[j]);
+            g[NBP - 1] = first;
+        }
+        {
+            float t[NBP];
+#pragma unroll
+            for (int j = 0; j < NBP; ++j) t[j] = g[j];
+            const float dgv = reg_pick<float, NBP>(t, lane & (NBP - 1));
+            if (lane < NBP) s_diag[s][lane] = dgv;
+        }
+        pair_sync();
+        // (b) proposals from lambda(x') = bbar(x') / sum bbar, bbar(x) = s(x) e^{x h}: x' = +1 iff
+        //     u < 1 / (1 + E), E = e^{lm - lp}; a flip to x' carries e^{(x - x') h}
+        double fac = 1.0;
+        if (s == 0) {
+            bool flip = false;
+            if (in) {
+                const double h = sp.c[0] * (1.0 - (double)s_diag[0][lane]) + sp.c[1] * (1.0 - (double)s_diag[1][lane]);
+                const double E = exp((hs_log_scalar(sp, -1) - h) - (hs_log_scalar(sp, +1) + h));
+                const int xp = rep ? (forced ? 1 : -1) : (uq * (1.0 + E) < 1.0 ? 1 : -1);
+                s_E[p0 + lane] = E;
+                so.dec[i] = xp > 0 ? 1 : 0;
+                flip = xp != x;
+                if (flip) {
+                    fac = E * sp.sflip[1];  // e^{-2h}: sflip[1] = s(+1)/s(-1) takes the scalar back out
+                    if (xp < 0) fac = accept_quot(1.0, fac);
+                }
+            }
+            const unsigned fl = __ballot_sync(FULL, flip);
+            if (lane == 0) s_flip = fl;
+        }
+        pair_sync();
+        const unsigned flips = s_flip;
+        // (c) det(1 + D_F A_FF) as the product of the sequential rank-1 ratios
+        double rprod = 1.0;
+        if (flips) {
+            float rl = 1.f;
+            int q = 0;
+#pragma unroll
+            for (int j = 0; j < NBP; ++j) g[j] = (in && j < nbk) ? S1[s][lane][j] : 0.f;
+#pragma unroll 1
+            for (int a = 0; a < NBP; ++a) {
+                float f = 0.f;
+                if ((flips >> a) & 1u) {  // uniform
+                    const float dd = (xup >> a) & 1u ? fc.dflip[s][0] : fc.dflip[s][1];
+                    const float rr = 1.f + dd * (1.f - __shfl_sync(FULL, g[0], a));
+                    const float phi = accept_quot(dd, rr);
+                    if (lane == a) {
+                        rl = rr;
+                        s_phi[s][q] = phi;
+                    }
+                    f = phi * g[0];
+                    ++q;
+                    const float first = g[0];
+#pragma unroll
+                    for (int j = 1; j < NBP; ++j) g[j - 1] = fmaf(f, __shfl_sync(FULL, g[j], a), g[j]);
+                    g[NBP - 1] = first;  // decided columns are not read again
+                } else {
+                    const float first = g[0];
+#pragma unroll
+                    for (int j = 1; j < NBP; ++j) g[j - 1] = g[j];
+                    g[NBP - 1] = first;
+                }
+            }
+            rprod = (double)rl * fac;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) rprod *= __shfl_xor_sync(FULL, rprod, o);
+        }
+        if (lane == 0) s_prod[s] = rprod;
+        pair_sync();
+        ++n_prop;
+        if (s == 0) {
+            const double R = flips ? s_prod[0] * s_prod[1] : 1.0;
+            bool acc = true;
+            if (flips) {
+                acc = rep ? force_acc : ua < fabs(R);
+                if (!isfinite(R)) {
+                    acc = false;
+                    bad = true;
+                }
+                if (acc) {
+                    if (R < 0) ++nneg;
+                    maxr = fmax(maxr, fabs(R));
+                }
+            }
+            if (lane == 0) {
+                so.dec[N + blk] = acc ? 1 : 0;
+                so.ratio[N + blk] = R;
+                s_acc = acc && flips ? 1 : 0;
+            }
+            if (acc) {
+                ++n_acc;
+                if ((flips >> lane) & 1u) xl[p0 + lane] = (int8_t)(-x);
+            }
+        }
+        __syncthreads();
+        if (!s_acc) continue;
+        // (d) the accepted flips, in increasing site order
+        int q = 0;
+        for (unsigned fl = flips; fl; fl &= fl - 1, ++q, ++m, par ^= 1) {
+            const int a = p0 + __ffs(fl) - 1;
+            __syncthreads();
+            const float phi = s_phi[s][q];
+            if (hw == 0 && lane == 0) wb.idx[m] = s0 + a;
+#pragma unroll
+            for (int j = 0; j < NP / 32; ++j) {
+                const int c = lane + 32 * j;
+                Wx[(size_t)m * NW + c] = c == a ? phi : srow[par][s][c];
+                Wm[(size_t)m * NW + c] = c == a ? phi : phi * scol[par][s][c];
+            }
+        }
+    }
+    if (hw != 0) return;
+    for (int q = lane; q < n; q += 32) so.ratio[s0 + q] = 1.0 / (1.0 + s_E[q]);
+    if (lane == 0) {
+        *wb.m = m;
+        if (bad) set_err(err, DEV_NUMERIC);
+        if (so.sign && (nneg & 1)) *so.sign = -*so.sign;
+        so.stats[0] += n_prop;
+        so.stats[1] += n_acc;
+        so.stats[2] += m;
+        so.stats[3] += (m > 0) ? 1 : 0;
+        *so.maxr = fmax(*so.maxr, maxr);
+    }
+}
+
 template <typename T, int MODE>
 __global__ void __launch_bounds__(WIN_THREADS) window_kernel(const T* __restrict__ Gu0, int8_t* xl0, const double* u0,
                                                              const uint8_t* replay0, SiteParams sp, SliceOut so0,
@@ -1113,13 +1371,31 @@ cudaError_t launch_window_chain(cudaStream_t st, int mode, const T* Gu, const T*
             return cudaGetLastError();
         }
     }
-    if (mode != AFQMC_MODE_BLOCKFB) return cudaErrorInvalidValue;
-    cudaError_t e = ensure_smem_attr((const void*)window_kernel<T, AFQMC_MODE_BLOCKFB>, window_smem<T>(WinCap<T>::NW));
-    if (e != cudaSuccess) return e;
-    count_launch();
-    window_kernel<T, AFQMC_MODE_BLOCKFB><<<bt.nwk, WIN_THREADS, window_smem<T>(n), st>>>(
-        Gu, xl, u, replay, sp, so, s0, n, nb, wb, blk, err, bt);
-    return cudaGetLastError();
+    if (mode != AFQMC_MODE_BLOCKFB || n > WIN_FB || nb > NBMAX) return cudaErrorInvalidValue;
+    if constexpr (sizeof(T) == 4) {
+        FlipConsts<float> fc, fs;
+        for (int xi = 0; xi < 2; ++xi) {
+            for (int s = 0; s < 2; ++s) {
+                fc.dflip[s][xi] = (float)sp.dflip[s][xi];
+                fs.dflip[s][xi] = (float)sp.dstrip[s][xi];
+            }
+            fc.sflip[xi] = fs.sflip[xi] = (float)sp.sflip[xi];
+        }
+        count_launch();
+        if (nb <= 16)
+            window_fb_kernel<16><<<bt.nwk, 320, 0, st>>>(Gu, xl, u, replay, sp, fc, fs, so, s0, n, nb, wb, blk, err, bt);
+        else
+            window_fb_kernel<32><<<bt.nwk, 320, 0, st>>>(Gu, xl, u, replay, sp, fc, fs, so, s0, n, nb, wb, blk, err, bt);
+        return cudaGetLastError();
+    } else {
+        cudaError_t e = ensure_smem_attr((const void*)window_kernel<T, AFQMC_MODE_BLOCKFB>,
+                                         window_smem<T>(WinCap<T>::NW));
+        if (e != cudaSuccess) return e;
+        count_launch();
+        window_kernel<T, AFQMC_MODE_BLOCKFB><<<bt.nwk, WIN_THREADS, window_smem<T>(n), st>>>(
+            Gu, xl, u, replay, sp, so, s0, n, nb, wb, blk, err, bt);
+        return cudaGetLastError();
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1375,11 +1651,11 @@ __global__ void __launch_bounds__(PanelCfg<T>::LT) panel_kernel(PanelArgs<T> a) 
         T* out = a.snap + (size_t)z * NW * NW + (size_t)r0 * NW;
         for (int r = warp; r < nr; r += LT / 32)
             for (int c = lane; c < nn; c += 32) {
-                T acc = gb[r * nn + c];
+                T acc = T(0);  // summed on its own: one rounding at G's magnitude, not m
                 const T* wr = bw + r * (n + 1);
 #pragma unroll 8
                 for (int k = 0; k < m; ++k) acc = fma(wr[k], bq[k * nn + c], acc);
-                out[r * NW + c] = acc;
+                out[r * NW + c] = gb[r * nn + c] + acc;
             }
         return;
     }
