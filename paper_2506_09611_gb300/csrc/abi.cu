@@ -868,7 +868,7 @@ int afqmc_init_walkers(afqmc_ctx* ctx, int n_walkers, const int* L, const int* n
         CK(dalloc(A, &w->sign, (size_t)nwk * 8));
         CK(dalloc(A, &w->replay, (size_t)nwk * 2 * N));
         CK(dalloc(A, (char**)&w->colbuf, 4 * (size_t)N * es));  // [2 buffers][2 spins][N]
-        CK(dalloc(A, (char**)&w->rowbuf, 4 * (size_t)N * es));
+        CK(dalloc(A, (char**)&w->rowbuf, local_rowbuf_elems(ld) * es));
         CK(dalloc(A, &w->bar, sizeof(GridBar)));
         CK(dalloc(A, &w->err, sizeof(int)));
         for (int q = 0; q < 2; ++q) {

@@ -237,6 +237,8 @@ cudaError_t launch_uniforms(cudaStream_t st, uint64_t seed, const int* gid, cons
                             double* u, int nwk);
 cudaError_t launch_bump(cudaStream_t st, unsigned long long* visit);
 
+// Local update of one slice.  colbuf: [2][2][N] diagonals; rowbuf: local_rowbuf_elems(ld) elements.
+size_t local_rowbuf_elems(long ld);
 template <typename T>
 cudaError_t launch_local(cudaStream_t st, T* Gu, T* Gd, int8_t* xl, const double* u, const uint8_t* replay,
                          const SiteParams& sp, SliceOut so, T* colbuf, T* rowbuf, GridBar* bar, int* err,

@@ -305,15 +305,240 @@ __global__ void __launch_bounds__(LOCAL_THREADS, 1) local_kernel(T* Gu, T* Gd, i
     }
 }
 
+// The same update with the own rows of G in registers for the whole slice (FP32, N <= 1672 on 152 SMs): thread (g, v)
+// holds the 16-byte column vector v of the rows g, g + ng, ... of both spins, RPT rows at most.  An accept
+// then moves two rows instead of all of G: the other CTAs need row b only, and its owner cannot know b before
+// the grid barrier that fixes it, so with its update every CTA publishes its rows among the next LR_AHEAD
+// sites (double-buffered by phase); the rare accept beyond them costs a second barrier.  The arithmetic is
+// local_kernel's, element by element.  Bound by the barrier and the round trips to L2 (diagonal, row b):
+// 40 x 40: LR_US us per slice against 9.75 ms with G in L2.
+constexpr int LR_THREADS = 448, LR_AHEAD = 4, LR_RPT_MAX = 11;
+inline size_t local_reg_pub(long ld) { return 2 * (size_t)(LR_AHEAD + 1) * 2 * ld; }  // floats of the row buffer
+
+template <int RPT>
+__global__ void __launch_bounds__(LR_THREADS, 1) local_reg_kernel(float* Gu, float* Gd, int8_t* xl_g, const double* u,
+                                                                  const uint8_t* replay, SiteParams sp, SliceOut so,
+                                                                  float* diag, float* pub, GridBar* bar, int* err) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int N = sp.N;
+    const long ld = sp.ld;
+    const int nblk = gridDim.x, b = blockIdx.x, tid = threadIdx.x, nt = LR_THREADS;
+    const int r0 = (int)((long)N * b / nblk), r1 = (int)((long)N * (b + 1) / nblk), nr = r1 - r0;
+    const int nv = (N + 3) / 4, ng = nt / nv, g = tid / nv, v = tid - g * nv;
+    const bool mine = g < ng;
+    double* us = (double*)smem_raw;
+    int8_t* xs = (int8_t*)(us + N);
+    uint8_t* rp = (uint8_t*)(xs + N);
+    __shared__ float colb[2][32];  // G_s[r, b] of the own rows
+    __shared__ int s_b, s_nneg;
+    __shared__ float s_f[2];
+    __shared__ double s_maxr;
+    for (int i = tid; i < N; i += nt) {
+        us[i] = u[i];
+        xs[i] = xl_g[i];
+        rp[i] = replay ? replay[i] : 0;
+    }
+    if (tid == 0) {
+        s_nneg = 0;
+        s_maxr = 0.0;
+    }
+    float4 G0[RPT], G1[RPT];
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) {
+        const int r = g + ng * i;
+        const bool in = mine && r < nr;
+        G0[i] = in ? *(const float4*)(Gu + (long)(r0 + r) * ld + 4 * v) : make_float4(0.f, 0.f, 0.f, 0.f);
+        G1[i] = in ? *(const float4*)(Gd + (long)(r0 + r) * ld + 4 * v) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    for (int e = tid; e < 2 * nr; e += nt) {  // diagonals of the own rows into buffer 0
+        const int s = e >= nr ? 1 : 0, r = r0 + e - s * nr;
+        diag[(0 * 2 + s) * N + r] = (s ? Gd : Gu)[(long)r * ld + r];
+    }
+    // own rows among the sites [p, p + LR_AHEAD) (slot: site - p) to buffer par; or site p alone to slot
+    // LR_AHEAD
+    auto publish = [&](int p, int par, bool one) {
+        if (!mine) return;
+#pragma unroll
+        for (int i = 0; i < RPT; ++i) {
+            const int r = g + ng * i, w = r0 + r - p;
+            if (r < nr && w >= 0 && w < (one ? 1 : LR_AHEAD)) {
+                float* o = pub + (size_t)((par * (LR_AHEAD + 1) + (one ? LR_AHEAD : w)) * 2) * ld + 4 * v;
+                *(float4*)o = G0[i];
+                *(float4*)(o + ld) = G1[i];
+            }
+        }
+    };
+    publish(0, 0, false);
+    unsigned int* ctr = &bar->count;
+    unsigned int nbar = 0;  // grid barriers passed (thread 0)
+    const float df00 = (float)sp.dflip[0][0], df01 = (float)sp.dflip[0][1], df10 = (float)sp.dflip[1][0],
+                df11 = (float)sp.dflip[1][1], sf0 = (float)sp.sflip[0], sf1 = (float)sp.sflip[1];
+    int n_acc = 0, p = 0, base = 0;  // p: next site to test (warp 0); base: first published site
+    int cur = 0;                     // diagonal and row buffer of this phase
+    __syncthreads();
+    for (;;) {
+        if (tid < 32) {  // grid barrier (thread 0), then the scan for the next accept, as in local_kernel
+            int ok = 1;
+            if (tid == 0) ok = grid_arrive_wait(ctr, (++nbar) * (unsigned int)nblk, err) ? 1 : 0;
+            __syncwarp();
+            ok = __shfl_sync(0xffffffffu, ok, 0);
+            int bsel = ok ? N : -1;
+            const float* d0 = diag + (cur * 2 + 0) * N;
+            const float* d1 = diag + (cur * 2 + 1) * N;
+            while (ok && p < N) {
+                const int q = p + tid;
+                bool acc = false;
+                float R = 0.f, rr0 = 1.f, rr1 = 1.f, del0 = df00, del1 = df10;
+                if (q < N) {
+                    const int xi = xs[q] > 0 ? 0 : 1;
+                    del0 = xi ? df01 : df00;
+                    del1 = xi ? df11 : df10;
+                    rr0 = 1.f + del0 * (1.f - __ldcg(d0 + q));
+                    rr1 = 1.f + del1 * (1.f - __ldcg(d1 + q));
+                    R = (xi ? sf1 : sf0) * rr0 * rr1;
+                    acc = replay ? (rp[q] != 0) : (us[q] < (double)fabs(R));
+                    if (!isfinite(R)) {
+                        if (b == 0) set_err(err, DEV_NUMERIC);
+                        acc = false;
+                    }
+                }
+                const unsigned ball = __ballot_sync(0xffffffffu, acc);
+                const int first = ball ? __ffs(ball) - 1 : 32;
+                if (b == 0 && q < N && tid <= first) {
+                    so.dec[q] = (tid == first) ? 1 : 0;
+                    so.ratio[q] = (double)R;
+                }
+                if (tid == first) {
+                    s_f[0] = del0 / rr0;
+                    s_f[1] = del1 / rr1;
+                    if (b == 0) {
+                        xl_g[q] = (int8_t)(-xs[q]);
+                        if (R < 0.f) s_nneg += 1;
+                        s_maxr = fmax(s_maxr, (double)fabs(R));
+                    }
+                }
+                __syncwarp();
+                if (first < 32) {
+                    bsel = p + first;
+                    p = bsel + 1;
+                    break;
+                }
+                p += 32;
+            }
+            if (tid == 0) s_b = bsel;
+        }
+        __syncthreads();
+        const int bs = s_b;
+        if (bs < 0) return;  // a bounded wait expired, or another CTA recorded an error
+        if (bs >= N) break;
+        ++n_acc;
+        int slot = bs - base;
+        if (slot >= LR_AHEAD) {  // not published (the same in every CTA): its owner does so now
+            slot = LR_AHEAD;
+            publish(bs, cur, true);
+            __syncthreads();
+            if (tid == 0 && !grid_arrive_wait(ctr, (++nbar) * (unsigned int)nblk, err)) s_b = -1;
+            __syncthreads();
+            if (s_b < 0) return;
+        }
+        const float* row = pub + (size_t)((cur * (LR_AHEAD + 1) + slot) * 2) * ld;  // row b, both spins (past L1)
+        float4 rv0 = make_float4(0.f, 0.f, 0.f, 0.f), rv1 = rv0;
+        if (mine) {
+            rv0 = __ldcg((const float4*)(row + 4 * v));
+            rv1 = __ldcg((const float4*)(row + ld + 4 * v));
+        }
+        float dnew = 0.f, drow = 0.f;  // the own diagonals: one element per thread
+        const int ds = tid >= nr ? 1 : 0, dr = tid - ds * nr;
+        if (tid < 2 * nr) {
+            dnew = __ldcg(diag + (cur * 2 + ds) * N + r0 + dr);
+            drow = (r0 + dr == bs ? 1.f : 0.f) - __ldcg(row + ds * ld + r0 + dr);
+        }
+        if (mine && v == bs >> 2) {  // column b of the own rows
+            const int k = bs & 3;
+#pragma unroll
+            for (int i = 0; i < RPT; ++i) {
+                const int r = g + ng * i;
+                if (r < nr) {
+                    colb[0][r] = k == 0 ? G0[i].x : k == 1 ? G0[i].y : k == 2 ? G0[i].z : G0[i].w;
+                    colb[1][r] = k == 0 ? G1[i].x : k == 1 ? G1[i].y : k == 2 ? G1[i].z : G1[i].w;
+                }
+            }
+        }
+        __syncthreads();
+        // e_b^T - G[b, :], zero beyond N
+        const int c0 = 4 * v;
+        rv0.x = c0 < N ? (c0 == bs ? 1.f : 0.f) - rv0.x : 0.f;
+        rv0.y = c0 + 1 < N ? (c0 + 1 == bs ? 1.f : 0.f) - rv0.y : 0.f;
+        rv0.z = c0 + 2 < N ? (c0 + 2 == bs ? 1.f : 0.f) - rv0.z : 0.f;
+        rv0.w = c0 + 3 < N ? (c0 + 3 == bs ? 1.f : 0.f) - rv0.w : 0.f;
+        rv1.x = c0 < N ? (c0 == bs ? 1.f : 0.f) - rv1.x : 0.f;
+        rv1.y = c0 + 1 < N ? (c0 + 1 == bs ? 1.f : 0.f) - rv1.y : 0.f;
+        rv1.z = c0 + 2 < N ? (c0 + 2 == bs ? 1.f : 0.f) - rv1.z : 0.f;
+        rv1.w = c0 + 3 < N ? (c0 + 3 == bs ? 1.f : 0.f) - rv1.w : 0.f;
+        const float nf0 = -s_f[0], nf1 = -s_f[1];
+#pragma unroll
+        for (int i = 0; i < RPT; ++i) {
+            const int r = g + ng * i;
+            if (mine && r < nr) {
+                vfma_rank1<float>(G0[i], nf0 * colb[0][r], rv0);
+                vfma_rank1<float>(G1[i], nf1 * colb[1][r], rv1);
+            }
+        }
+        if (tid < 2 * nr)
+            diag[((cur ^ 1) * 2 + ds) * N + r0 + dr] = fma((ds ? nf1 : nf0) * colb[ds][dr], drow, dnew);
+        base = bs + 1;
+        cur ^= 1;
+        publish(base, cur, false);
+        __syncthreads();  // every write of the CTA precedes thread 0's arrival at the next barrier
+    }
+    if (mine) {
+#pragma unroll
+        for (int i = 0; i < RPT; ++i) {
+            const int r = g + ng * i;
+            if (r < nr) {
+                *(float4*)(Gu + (long)(r0 + r) * ld + 4 * v) = G0[i];
+                *(float4*)(Gd + (long)(r0 + r) * ld + 4 * v) = G1[i];
+            }
+        }
+    }
+    if (b == 0 && tid == 0) {
+        if (so.sign && (s_nneg & 1)) *so.sign = -*so.sign;
+        so.stats[0] += N;
+        so.stats[1] += n_acc;
+        so.stats[2] += n_acc;
+        *so.maxr = fmax(*so.maxr, s_maxr);
+    }
+}
+
+template <int RPT>
+static cudaError_t launch_local_reg(cudaStream_t st, float* Gu, float* Gd, int8_t* xl, const double* u,
+                                    const uint8_t* replay, const SiteParams& sp, SliceOut so, float* diag, float* pub,
+                                    GridBar* bar, int* err, int nblk) {
+    const size_t shm = (size_t)sp.N * (sizeof(double) + 2);
+    SiteParams spc = sp;
+    void* args[] = {&Gu, &Gd, &xl, &u, &replay, &spc, &so, &diag, &pub, &bar, &err};
+    count_launch();
+    return cudaLaunchCooperativeKernel((void*)local_reg_kernel<RPT>, dim3(nblk), dim3(LR_THREADS), args, shm, st);
+}
+
 // Grid size of the local kernel: at most max_blocks CTAs (one per SM) and at least one row each.
+size_t local_rowbuf_elems(long ld) { return local_reg_pub(ld); }
+
 template <typename T>
 cudaError_t launch_local(cudaStream_t st, T* Gu, T* Gd, int8_t* xl, const double* u, const uint8_t* replay,
                          const SiteParams& sp, SliceOut so, T* colbuf, T* rowbuf, GridBar* bar, int* err,
                          int max_blocks) {
-    (void)rowbuf;
     const int nblk = max_blocks < sp.N ? max_blocks : sp.N;
     if (nblk < 1) return cudaErrorInvalidValue;
     const int nrmax = (sp.N + nblk - 1) / nblk;
+    if constexpr (sizeof(T) == 4) {  // the own rows in registers, where they fit
+        const int nv = (sp.N + 3) / 4, ng = nv <= LR_THREADS ? LR_THREADS / nv : 0;
+        const int rpt = ng > 0 && nrmax <= 32 ? (nrmax + ng - 1) / ng : LR_RPT_MAX + 1;
+        if (rpt <= 3) return launch_local_reg<3>(st, Gu, Gd, xl, u, replay, sp, so, colbuf, rowbuf, bar, err, nblk);
+        if (rpt <= 6) return launch_local_reg<6>(st, Gu, Gd, xl, u, replay, sp, so, colbuf, rowbuf, bar, err, nblk);
+        if (rpt <= LR_RPT_MAX)
+            return launch_local_reg<LR_RPT_MAX>(st, Gu, Gd, xl, u, replay, sp, so, colbuf, rowbuf, bar, err, nblk);
+    }
     const size_t shm = local_smem<T>(sp.N, sp.ld, nrmax).total;
     cudaError_t e = ensure_smem_attr((const void*)local_kernel<T>, shm);
     if (e != cudaSuccess) return e;
