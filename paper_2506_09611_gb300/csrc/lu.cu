@@ -5,8 +5,8 @@
 // at a small fraction of its FP32 rate and every pivot is a grid-wide dependency, so the
 // factorisation is blocked:
 //   * a panel of LU_NB columns is factored by one thread-block cluster per matrix: each CTA
-//     keeps its share of the rows in shared memory and the CTAs agree on every pivot through
-//     distributed shared memory and one cluster barrier per column;
+//     keeps its share of the rows in shared memory and the CTAs agree on every pivot by sending one
+//     another their best rows through distributed shared memory;
 //   * the pivot rows' trailing part U12 = L11^{-1} A12 and the trailing update A22 -= L21 U12 of the
 //     unpivoted rows run over the whole GPU.
 // Rows are not swapped: a pivoted row is flagged, keeps its multipliers left of its pivot
@@ -74,12 +74,53 @@ __device__ __forceinline__ int lu_warp_best(unsigned long long& k, int& r) {
     return src;
 }
 
-// tpr threads per row (a power of two up to 8).  Per column: every warp pushes its candidate into the shared
-// memory of all CTAs, one cluster barrier, warp 0 of every CTA picks the winner and pulls the pivot row from
-// its owner (a pivoted row is never written again) while it takes the reciprocal, one block barrier, and the
-// own rows are updated, the next column first for the next candidates.  Bound by that chain: the first panel
-// of the 1600 x 700 factor took 128 us with one thread per row, the FP64 division and candidates read through
-// distributed shared memory.
+// ---- asynchronous stores between the CTAs of a cluster, counted by an mbarrier of the receiver ----
+__device__ __forceinline__ unsigned lu_smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ unsigned lu_mapa(unsigned addr, int rank) {
+    unsigned r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void lu_st_async(unsigned dst, double v, unsigned bar) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(dst),
+                 "l"(__double_as_longlong(v)), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void lu_st_async(unsigned dst, int v, unsigned bar) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(dst), "r"(v),
+                 "r"(bar)
+                 : "memory");
+}
+// Wait for phase `parity` of the mbarrier; false after two seconds of %globaltimer.
+__device__ __forceinline__ bool lu_bar_wait(unsigned bar, unsigned parity) {
+    unsigned long long t0 = 0;
+    for (unsigned polls = 0;; ++polls) {
+        unsigned ok;
+        asm volatile(
+            "{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+            "selp.u32 %0, 1, 0, p;\n}\n"
+            : "=r"(ok)
+            : "r"(bar), "r"(parity)
+            : "memory");
+        if (ok) return true;
+        if ((polls & 63u) == 63u) {
+            unsigned long long t;
+            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+            if (t0 == 0) t0 = t;
+            else if (t - t0 > 2000000000ULL) return false;
+        }
+    }
+}
+
+// tpr threads per row (a power of two up to 8).  Per column: every warp's candidate, one block barrier, and
+// warp 0 sends the CTA's best row to all CTAs of the cluster (asynchronous stores counted by the receiver's
+// mbarrier, double-buffered by step parity: no cluster barrier and no memory fence per step); when the CS rows
+// have arrived, every warp picks the winner by itself, takes the reciprocal of the pivot, and updates its
+// rows, the next column first for the next candidates.  A CTA sends its row of step j + 1 after all its warps
+// are done with the rows of step j, so a buffer is free again when the rows of step j + 2 arrive.  Bound by
+// that chain.  First panel of the 1600 x 700 factor: 128 us with one thread per row, the FP64 division and
+// candidates read back through distributed shared memory behind a cluster barrier; 77 us with the
+// candidates pushed before the cluster barrier and the pivot row read after it.
 template <int CS>
 __global__ void __launch_bounds__(256) lu_panel_kernel(LuArgs a, int j0, int nbk, int tpr) {
     cg::cluster_group cl = cg::this_cluster();
@@ -95,19 +136,23 @@ __global__ void __launch_bounds__(256) lu_panel_kernel(LuArgs a, int j0, int nbk
     extern __shared__ __align__(16) double lu_smem[];
     double* Pn = lu_smem;                    // [nr][LU_NBP] own rows of the panel
     int8_t* fl = (int8_t*)(Pn + (size_t)nr * LU_NBP);
-    // the candidates of all warps of the cluster (by step parity): key, signed value, row
-    __shared__ unsigned long long cand_k[2][8 * CS];
-    __shared__ double cand_x[2][8 * CS];
-    __shared__ int cand_r[2][8 * CS];
-    __shared__ double L11[LU_NB][LU_NBP];    // pivot rows' panel values at their pivot step
-    __shared__ double s_pinv;
-    bool any_bad = false;
+    __shared__ __align__(16) double rowb[2][CS][LU_NB];  // every CTA's best row (by step parity)
+    __shared__ int rowi[2][CS];                          // its index in the matrix, INT_MAX: none left
+    __shared__ __align__(8) unsigned long long mbar[2];
+    __shared__ unsigned long long ck[8];
+    __shared__ int cr[8];
+    bool any_bad = false, late = false;
+    if (tid == 0) {
+        for (int q = 0; q < 2; ++q)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(lu_smem_u32(&mbar[q])) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
     for (int e = tid; e < nr * nbk; e += nt) {
         const int q = e / nbk, c = e - q * nbk;
         Pn[q * LU_NBP + c] = A[(long)(r0 + q) * lda + j0 + c];
     }
     for (int q = tid; q < nr; q += nt) fl[q] = flag[r0 + q];
-    cl.sync();  // every CTA of the cluster runs before its shared memory is written from outside
+    cl.sync();  // every CTA of the cluster runs and its mbarriers are set up
     const int h = tid & (tpr - 1), rows = nt / tpr, q0 = tid / tpr;
     // candidate of column 0 (later columns: found during the previous step's row update)
     unsigned long long bk = 0;
@@ -121,50 +166,44 @@ __global__ void __launch_bounds__(256) lu_panel_kernel(LuArgs a, int j0, int nbk
             }
     for (int jj = 0; jj < nbk; ++jj) {
         const int par = jj & 1;
-        {
-            const int src = lu_warp_best(bk, br);
-            const double x = __shfl_sync(0xffffffffu, bx, src);
-            if (lane < CS) {
-                const int slot = rank * 8 + wid;
-                *cl.map_shared_rank(&cand_k[par][slot], lane) = bk;
-                *cl.map_shared_rank(&cand_x[par][slot], lane) = x;
-                *cl.map_shared_rank(&cand_r[par][slot], lane) = br;
-            }
+        const unsigned bar = lu_smem_u32(&mbar[par]);
+        lu_warp_best(bk, br);
+        if (lane == 0) {
+            ck[wid] = bk;
+            cr[wid] = br;
         }
-        cl.sync();  // every warp's candidate has arrived, and every row update of the last step is done
+        __syncthreads();  // the candidates are there, and every row update of the last step is done
         if (wid == 0) {
-            unsigned long long k = 0;
-            int r = INT_MAX, slot = 0;
-#pragma unroll
-            for (int t = 0; t < (8 * CS + 31) / 32; ++t) {
-                const int sl = lane + 32 * t;
-                if (sl < 8 * CS) {
-                    const unsigned long long ok = cand_k[par][sl];
-                    const int orr = cand_r[par][sl];
-                    if (ok > k || (ok == k && orr < r)) {
-                        k = ok;
-                        r = orr;
-                        slot = sl;
-                    }
-                }
+            unsigned long long k = lane < 8 ? ck[lane] : 0ULL;
+            int r = lane < 8 ? cr[lane] : INT_MAX;
+            lu_warp_best(k, r);
+            const double v = (r != INT_MAX && lane < nbk) ? Pn[(r - r0) * LU_NBP + lane] : 0.0;
+            if (lane == 0)
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
+                             "r"(CS * (LU_NB * 8 + 4))
+                             : "memory");
+            const unsigned dv = lu_smem_u32(&rowb[par][rank][lane]), di = lu_smem_u32(&rowi[par][rank]);
+#pragma unroll 4
+            for (int d = 0; d < CS; ++d) {
+                const unsigned rb = lu_mapa(bar, d);
+                lu_st_async(lu_mapa(dv, d), v, rb);
+                if (lane == 0) lu_st_async(lu_mapa(di, d), r, rb);
             }
-            const int src = lu_warp_best(k, r);
-            slot = __shfl_sync(0xffffffffu, slot, src);
-            const bool bad = (k == 0ULL) || (k >= 0x7ff0000000000000ULL) || r >= m || r < 0;
-            const int own = bad ? 0 : slot >> 3, p = bad ? 0 : r;
-            const int pr0 = (int)((long)m * own / CS);
-            const double* prow = cl.map_shared_rank(Pn, own) + (size_t)(p - pr0) * LU_NBP;
-            if (lane < nbk) L11[jj][lane] = prow[lane];
-            const double pinv = bad ? 0.0 : lu_rcp(cand_x[par][slot]);
-            if (lane == 0) {
-                s_pinv = pinv;
-                if (p >= r0 && p < r1) fl[p - r0] = 1;
-                if (rank == 0) perm[j0 + jj] = p;
-            }
-            any_bad = any_bad || bad;
         }
-        __syncthreads();
-        const double pinv = s_pinv;
+        if (!late && !lu_bar_wait(bar, (unsigned)(jj >> 1) & 1u)) late = true;
+        // the winner over the cluster's CTAs
+        int r = lane < CS ? rowi[par][lane] : INT_MAX;
+        unsigned long long k = (lane < CS && r != INT_MAX) ? lu_key(rowb[par][lane < CS ? lane : 0][jj]) : 0ULL;
+        const int win = lu_warp_best(k, r) & (CS - 1);
+        const double* urow = rowb[par][win];
+        const bool bad = late || (k == 0ULL) || (k >= 0x7ff0000000000000ULL) || r >= m || r < 0;
+        const int p = bad ? 0 : r;
+        const double pinv = bad ? 0.0 : lu_rcp(urow[jj]);
+        any_bad = any_bad || bad;
+        if (tid == 0) {
+            if (p >= r0 && p < r1) fl[p - r0] = 1;
+            if (rank == 0) perm[j0 + jj] = p;
+        }
         // own unpivoted rows: multiplier into column jj, rank-1 step on the later panel columns, and the
         // candidate for column jj + 1
         bk = 0;
@@ -173,7 +212,7 @@ __global__ void __launch_bounds__(256) lu_panel_kernel(LuArgs a, int j0, int nbk
         const int hj = jj & (tpr - 1), c0 = jj + 1 + ((h - (jj + 1)) & (tpr - 1));
         for (int qb = 0; qb < nr; qb += rows) {
             const int q = qb + q0;
-            const bool act = q < nr && !fl[q];
+            const bool act = q < nr && r0 + q != p && !fl[q];
             double* __restrict__ row = Pn + (act ? q : 0) * LU_NBP;
             double l = 0.0;
             if (act && h == hj) {
@@ -184,25 +223,26 @@ __global__ void __launch_bounds__(256) lu_panel_kernel(LuArgs a, int j0, int nbk
             if (!act) continue;
             int c = c0;
             if (c < nbk) {
-                const double x = row[c] - l * L11[jj][c];
+                const double x = row[c] - l * urow[c];
                 row[c] = x;
                 if (c == jj + 1) lu_pick(bk, br, bx, lu_key(x), r0 + q, x);
                 c += tpr;
             }
             for (; c + 3 * tpr < nbk; c += 4 * tpr) {
-                const double u0 = L11[jj][c], u1 = L11[jj][c + tpr], u2 = L11[jj][c + 2 * tpr], u3 = L11[jj][c + 3 * tpr];
+                const double u0 = urow[c], u1 = urow[c + tpr], u2 = urow[c + 2 * tpr], u3 = urow[c + 3 * tpr];
                 const double v0 = row[c], v1 = row[c + tpr], v2 = row[c + 2 * tpr], v3 = row[c + 3 * tpr];
                 row[c] = v0 - l * u0;
                 row[c + tpr] = v1 - l * u1;
                 row[c + 2 * tpr] = v2 - l * u2;
                 row[c + 3 * tpr] = v3 - l * u3;
             }
-            for (; c < nbk; c += tpr) row[c] -= l * L11[jj][c];
+            for (; c < nbk; c += tpr) row[c] -= l * urow[c];
         }
         __syncwarp();
     }
-    cl.sync();  // no CTA leaves while another may still read its shared memory
-    if (any_bad && lane == 0 && rank == 0) set_err(a.err, DEV_NUMERIC);
+    cl.sync();  // no CTA leaves while a store to another may still be in flight
+    if (late && lane == 0) set_err(a.err, DEV_TIMEOUT);
+    if (tid == 0 && rank == 0 && any_bad) set_err(a.err, DEV_NUMERIC);
     for (int e = tid; e < nr * nbk; e += nt) {
         const int q = e / nbk, c = e - q * nbk;
         A[(long)(r0 + q) * lda + j0 + c] = Pn[q * LU_NBP + c];
