@@ -1726,11 +1726,18 @@ __host__ __device__ inline int panel_tri(int m) {
     return PL_B * PL_B * (nb * (nb + 1) / 2);
 }
 
+// Pitch of the column lines: whole 16-byte vectors, an odd number of them.
+template <typename T>
+__host__ __device__ inline int panel_pitch(int n) {
+    constexpr int VW = 16 / sizeof(T);
+    return ((n + VW - 1) / VW | 1) * VW;
+}
+
 template <typename T>
 static size_t panel_smem(int n, int nn) {
     constexpr size_t LN = PanelCfg<T>::LT / 4, RB = PanelCfg<T>::RB;
-    const size_t lines = (size_t)panel_tri(n) + LN * (n + 1);
-    const size_t block = nn > 0 ? 2 * (size_t)panel_tri(n) + RB * (n + 1) + (size_t)n * nn + RB * nn : 0;
+    const size_t lines = (size_t)panel_tri(n) + LN * panel_pitch<T>(n);
+    const size_t block = nn > 0 ? 2 * (size_t)panel_tri(n) + RB * panel_pitch<T>(n) + (size_t)n * nn + RB * nn : 0;
     return (lines > block ? lines : block) * sizeof(T) + 3 * WinCap<T>::NW * sizeof(int);
 }
 
@@ -1741,6 +1748,20 @@ __device__ __forceinline__ void cp_async_elem(T* dst, const T* src, bool in) {
     const int sz = in ? (int)sizeof(T) : 0;
     if (sizeof(T) == 4) asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(sz) : "memory");
     else asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(src), "r"(sz) : "memory");
+}
+// ... and of 16 bytes (both addresses aligned).
+__device__ __forceinline__ void cp_async_16(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+// count elements from src to dst, lanes of a warp; vec: in 16-byte vectors (aligned, padded to whole vectors).
+template <typename T>
+__device__ __forceinline__ void cp_async_row(T* dst, const T* src, int count, bool vec, int lane) {
+    constexpr int VW = 16 / sizeof(T);
+    if (vec)
+        for (int c = lane * VW; c < count; c += 32 * VW) cp_async_16(dst + c, src + c);
+    else
+        for (int c = lane; c < count; c += 32) cp_async_elem(dst + c, src + c, true);
 }
 __device__ __forceinline__ void cp_async_wait_all() {
     asm volatile("cp.async.commit_group;" ::: "memory");
@@ -1800,18 +1821,18 @@ __device__ __forceinline__ void panel_line(T* line, const int* off, int step, co
             Ep += PL_B * w - PL_B;
         }
         const int w = ep - kb;
+        // FP32 straight-line: entries from m on are zero, as are their coefficients (FP64 leaves them out)
 #pragma unroll
         for (int j = 0; j < PL_B; ++j) {
-            if (kb + j < m) {
-                T x = __shfl_sync(FULL, v[j & 3], (lane & ~3) | (j >> 2));
-                if (col) x *= Eb[j * w + j];
-                if (own && h == 0) line[off[kb + j] * step] = x;
-                T d[4];
+            if (sizeof(T) == 8 && kb + j >= m) break;
+            T x = __shfl_sync(FULL, v[j & 3], (lane & ~3) | (j >> 2));
+            if (col) x *= Eb[j * w + j];
+            if (own && h == 0 && kb + j < m) line[off[kb + j] * step] = x;
+            T d[4];
 #pragma unroll
-                for (int t = 0; t < 4; t += VW) *(V*)(d + t) = *(const V*)(Eb + j * w + 4 * h + t);
+            for (int t = 0; t < 4; t += VW) *(V*)(d + t) = *(const V*)(Eb + j * w + 4 * h + t);
 #pragma unroll
-                for (int t = 0; t < 4; ++t) v[t] = fma(x, d[t], v[t]);  // entries up to j are not read again
-            }
+            for (int t = 0; t < 4; ++t) v[t] = fma(x, d[t], v[t]);  // entries up to j are not read again
         }
         __syncwarp();
         Eb += PL_B * w;
@@ -1826,11 +1847,12 @@ __device__ __forceinline__ void panel_line(T* line, const int* off, int step, co
 template <typename T, bool TF>
 __global__ void __launch_bounds__(PanelCfg<T>::LT) panel_kernel(PanelArgs<T> a) {
     constexpr int NW = WinCap<T>::NW, LT = PanelCfg<T>::LT, LN = LT / 4, RB = PanelCfg<T>::RB;
-    const int wk = blockIdx.z, s = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int wk = blockIdx.z, s = blockIdx.y, tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     const int N = a.N, n = a.n, nl = (N + LN - 1) / LN, z = 2 * wk + s, bx = blockIdx.x;
     const WindowBufs wb = wb_walker<T>(a.wb, wk, N);
     const T* G = TF ? nullptr : a.G + (size_t)wk * a.gw + (size_t)s * a.gs;
-    const int m = *wb.m;
+    const int m = __shfl_sync(0xffffffffu, *wb.m, 0), PC = panel_pitch<T>(n);
     extern __shared__ __align__(16) unsigned char pl_smem[];
     T* E = (T*)pl_smem;
     const T* W0 = (const T*)wb.Wx + (size_t)s * NW * NW;
@@ -1838,8 +1860,8 @@ __global__ void __launch_bounds__(PanelCfg<T>::LT) panel_kernel(PanelArgs<T> a) 
     const int tri = panel_tri(m);
     if (bx >= 2 * nl) {  // rows r0 .. r0 + RB - 1 of the next window's block
         T* E1 = E + tri;
-        T* bw = E1 + tri;                    // w lines [RB][n + 1]
-        T* bq = bw + RB * (n + 1);           // q lines [m][nn]
+        T* bw = E1 + tri;                    // w lines [RB][PC], accept k at its position in the window
+        T* bq = bw + RB * PC;                // q lines [m][nn]
         T* gb = bq + (size_t)n * a.nn;       // G[J rows][J] [RB][nn]
         int* gidx = (int*)(gb + RB * a.nn);  // accepts: global index, position in the window, own index
         int *pos = gidx + NW, *idn = pos + NW;
@@ -1851,13 +1873,14 @@ __global__ void __launch_bounds__(PanelCfg<T>::LT) panel_kernel(PanelArgs<T> a) 
         }
         __syncthreads();
         const T* rows = G + (long)(a.sn + r0) * a.ld;
+        constexpr int VW = 16 / sizeof(T);
+        const bool vc = a.s0 % VW == 0, vn = a.sn % VW == 0 && nn % VW == 0;
         for (int r = warp; r < nr; r += LT / 32) {
-            for (int c = lane; c < nn; c += 32) cp_async_elem(gb + r * nn + c, rows + r * a.ld + a.sn + c, true);
-            for (int k = lane; k < m; k += 32) cp_async_elem(bw + r * (n + 1) + k, rows + r * a.ld + gidx[k], true);
+            cp_async_row<T>(gb + r * nn, rows + r * a.ld + a.sn, nn, vn, lane);
+            cp_async_row<T>(bw + r * PC, rows + r * a.ld + a.s0, n, vc, lane);
         }
         for (int k = warp; k < m; k += LT / 32)
-            for (int c = lane; c < nn; c += 32)
-                cp_async_elem(bq + k * nn + c, G + (long)gidx[k] * a.ld + a.sn + c, true);
+            cp_async_row<T>(bq + k * nn, G + (long)gidx[k] * a.ld + a.sn, nn, vn, lane);
         panel_load_tri<T>(E, W0, pos, m, tid, LT);
         panel_load_tri<T>(E1, W1, pos, m, tid, LT);
         cp_async_wait_all();
@@ -1869,26 +1892,33 @@ __global__ void __launch_bounds__(PanelCfg<T>::LT) panel_kernel(PanelArgs<T> a) 
             const bool col = wv < RW;
             const int l0 = (col ? wv : wv - RW) * 8, l = l0 + (lane >> 2), lim = col ? nr : nn, lc = min(l, lim - 1);
             if (l0 < lim)
-                panel_line<T>(col ? bw + lc * (n + 1) : bq + lc, idn, col ? 1 : nn, col ? E : E1, m, col, false, nullptr,
-                              0, l < lim, lane);
+                panel_line<T>(col ? bw + lc * PC : bq + lc, col ? pos : idn, col ? 1 : nn, col ? E : E1, m, col, false,
+                              nullptr, 0, l < lim, lane);
         }
         __syncthreads();
         T* out = a.snap + (size_t)z * NW * NW + (size_t)r0 * NW;
+        // sums of their own, then added: one rounding at G's magnitude, not m
         for (int r = warp; r < nr; r += LT / 32)
-            for (int c = lane; c < nn; c += 32) {
-                T acc = T(0);  // summed on its own: one rounding at G's magnitude, not m
-                const T* wr = bw + r * (n + 1);
+            for (int c = lane; c < nn; c += 64) {
+                const int c1 = c + 32 < nn ? c + 32 : c;
+                T acc = T(0), acc1 = T(0);
+                const T* wr = bw + r * PC;
 #pragma unroll 8
-                for (int k = 0; k < m; ++k) acc = fma(wr[k], bq[k * nn + c], acc);
+                for (int k = 0; k < m; ++k) {
+                    const T w = wr[pos[k]];
+                    acc = fma(w, bq[k * nn + c], acc);
+                    acc1 = fma(w, bq[k * nn + c1], acc1);
+                }
                 out[r * NW + c] = gb[r * nn + c] + acc;
+                if (c1 != c) out[r * NW + c1] = gb[r * nn + c1] + acc1;
             }
         return;
     }
     if (m == 0) return;
     const bool col = bx < nl;  // column lines: one per row of G
     const int i0 = (col ? bx : bx - nl) * LN, cnt = min(LN, N - i0);
-    T* buf = E + tri;  // column lines [LN][n + 1], row lines [m][LN]
-    int* gidx = (int*)(buf + (size_t)LN * (n + 1));
+    T* buf = E + tri;  // column lines [LN][PC] (T form: accept k at k, else at its position), row lines [m][LN]
+    int* gidx = (int*)(buf + (size_t)LN * PC);
     int *pos = gidx + NW, *idn = pos + NW;
     for (int k = tid; k < m; k += LT) {
         gidx[k] = TF ? -1 : wb.idx[k];
@@ -1896,30 +1926,29 @@ __global__ void __launch_bounds__(PanelCfg<T>::LT) panel_kernel(PanelArgs<T> a) 
         idn[k] = k;
     }
     __syncthreads();
+    constexpr int VW = 16 / sizeof(T);
     if (col) {
         for (int r = warp; r < cnt; r += LT / 32)
-            for (int k = lane; k < m; k += 32)
-                cp_async_elem(buf + r * (n + 1) + k,
-                              TF ? a.V + ((size_t)z * N + i0 + r) * NW + k : G + (long)(i0 + r) * a.ld + gidx[k], true);
+            cp_async_row<T>(buf + r * PC, TF ? a.V + ((size_t)z * N + i0 + r) * NW : G + (long)(i0 + r) * a.ld + a.s0,
+                            TF ? m : n, TF || a.s0 % VW == 0, lane);
     } else {
         for (int k = warp; k < m; k += LT / 32)
-            for (int c = lane; c < cnt; c += 32)
-                cp_async_elem(buf + k * LN + c,
-                              TF ? a.R + ((size_t)z * NW + k) * a.ldy + i0 + c : G + (long)gidx[k] * a.ld + i0 + c, true);
+            cp_async_row<T>(buf + k * LN, TF ? a.R + ((size_t)z * NW + k) * a.ldy + i0 : G + (long)gidx[k] * a.ld + i0,
+                            cnt, !TF, lane);
     }
     panel_load_tri<T>(E, col ? W0 : W1, pos, m, tid, LT);
     cp_async_wait_all();
     __syncthreads();
     if (warp * 8 < cnt) {
         const int l = tid >> 2, lc = min(l, cnt - 1);
-        panel_line<T>(col ? buf + lc * (n + 1) : buf + lc, idn, col ? 1 : LN, E, m, col, TF && !col, gidx, i0 + lc,
-                      l < cnt, lane);
+        panel_line<T>(col ? buf + lc * PC : buf + lc, col && !TF ? pos : idn, col ? 1 : LN, E, m, col, TF && !col, gidx,
+                      i0 + lc, l < cnt, lane);
     }
     __syncthreads();
     if (col) {
         T* out = a.X + ((size_t)z * N + i0) * NW;
         for (int r = warp; r < cnt; r += LT / 32)
-            for (int k = lane; k < m; k += 32) out[r * NW + k] = buf[r * (n + 1) + k];
+            for (int k = lane; k < m; k += 32) out[r * NW + k] = buf[r * PC + (TF ? k : pos[k])];
     } else {
         for (int k = warp; k < m; k += LT / 32)
             for (int c = lane; c < cnt; c += 32) a.Y[((size_t)z * NW + k) * a.ldy + i0 + c] = buf[k * LN + c];
