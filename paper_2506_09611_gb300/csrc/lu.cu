@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(256) lu_panel_kernel(LuArgs a, int j0, int nbk
         const int win = lu_warp_best(k, r) & (CS - 1);
         const double* urow = rowb[par][win];
         const bool bad = late || (k == 0ULL) || (k >= 0x7ff0000000000000ULL) || r >= m || r < 0;
-        const int p = bad ? 0 : r;
+        const int p = (late || r >= m || r < 0) ? 0 : r;  // with a zero pivot too: perm stays a permutation
         const double pinv = bad ? 0.0 : lu_rcp(urow[jj]);
         any_bad = any_bad || bad;
         if (tid == 0) {
