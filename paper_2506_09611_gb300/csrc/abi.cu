@@ -121,7 +121,6 @@ struct Walker {
     double* Gnew = nullptr;  // [nwk][2][N][ld]: the recomputed G
     int* perm2 = nullptr;    // [nwk][2][maxr]: pivot rows
     int8_t* flag2 = nullptr; // [nwk][2][maxr]: pivoted-row flags
-    int* visited = nullptr;  // [nwk][maxr]: permutation-parity scratch
     double* acc2 = nullptr;  // [nwk][2]
     // the recompute's two FP64 products on the tensor cores (digit splitting, ozaki.cu)
     bool oz_Z = false, oz_G = false;  // U_L U_R, and U_R Z
@@ -448,7 +447,7 @@ static cudaError_t stab_rows(afqmc_ctx* ctx, Walker* w, cudaStream_t st, const F
         PhaseScope ps(ctx, AFQMC_PHASE_ELIM, st);
         if ((e = launch_lu(st, a)) != cudaSuccess) return e;
     }
-    if (sign && (e = launch_lu_sign(st, a, 0, sign, w->visited)) != cudaSuccess) return e;
+    if (sign && (e = launch_lu_sign(st, a, 0, sign)) != cudaSuccess) return e;
     return launch_lu_unit_rows(st, a);
 }
 
@@ -500,7 +499,7 @@ static cudaError_t form_O(afqmc_ctx* ctx, Walker* w, cudaStream_t st, const Fac&
         PhaseScope ps(ctx, AFQMC_PHASE_LU_O, st);
         if ((e = launch_lu(st, a)) != cudaSuccess) return e;
     }
-    if (sign && (e = launch_lu_sign(st, a, 1, sign, w->visited)) != cudaSuccess) return e;
+    if (sign && (e = launch_lu_sign(st, a, 1, sign)) != cudaSuccess) return e;
     return cudaSuccess;
 }
 
@@ -909,7 +908,6 @@ int afqmc_init_walkers(afqmc_ctx* ctx, int n_walkers, const int* L, const int* n
         CK(dalloc(A, &w->Gnew, (size_t)nwk * 2 * N * ld * 8));
         CK(dalloc(A, (char**)&w->perm2, (size_t)nwk * 2 * maxr * sizeof(int)));
         CK(dalloc(A, (char**)&w->flag2, (size_t)nwk * 2 * maxr));
-        CK(dalloc(A, (char**)&w->visited, (size_t)nwk * maxr * sizeof(int)));
         CK(dalloc(A, &w->acc2, (size_t)nwk * 2 * 8));
         if (ctx->form == AFQMC_FORM_T) {
             const size_t fsb = (size_t)nwk * 2 * N * nsm * es, pan = (size_t)nwk * 2 * NW * nsm * es;
@@ -1775,7 +1773,7 @@ static int cp_refresh(afqmc_ctx* ctx, Walker* w, cudaStream_t st, int set_ref) {
     count_launch();
     cp_begin_kernel<<<(nwk + 127) / 128, 128, 0, st>>>(w->cpl, w->cpsg, nwk);  // (re)sets the sign product
     CK(cudaGetLastError());
-    CK(launch_lu_sign(st, a, 1, w->cpsg, w->visited));
+    CK(launch_lu_sign(st, a, 1, w->cpsg));
     count_launch();
     cp_logdet_kernel<<<nb2, 256, 0, st>>>(w->Ob, os, w->perm2, w->rows_max(), ns, w->cpla);
     CK(cudaGetLastError());

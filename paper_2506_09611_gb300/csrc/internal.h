@@ -160,8 +160,8 @@ cudaError_t launch_lu(cudaStream_t st, const LuArgs& a);
 // After launch_lu: pivot rows become unit rows, so A = P L spans the factored columns.
 cudaError_t launch_lu_unit_rows(cudaStream_t st, const LuArgs& a);
 // After launch_lu: sign_out[j] *= sign(prod of pivots) (times the row permutation's parity when
-// parity != 0) over the ng matrices of walker j; visited: nmat * m ints of scratch.
-cudaError_t launch_lu_sign(cudaStream_t st, const LuArgs& a, int parity, double* sign_out, int* visited);
+// parity != 0) over the ng matrices of walker j.
+cudaError_t launch_lu_sign(cudaStream_t st, const LuArgs& a, int parity, double* sign_out);
 // Z = O^{-1} B for the O factored by launch_lu (ns x ns, leading dimension ldl, matrix b at
 // LU0 + b ostride with pivots perm0 + b pstride), B (ns x N) at B0 + j wstride + q sstride
 // (b = j ng + q), row stride ldb (0: N), and Z (ns x N) at Z0 + b zstride.
