@@ -4,13 +4,12 @@
 //             rank-1 update G <- G - (d/r) G_{:,i} (e_i^T - G_{i,:}) applied to
 //             the whole of G on every accepted flip (Eqs. DetRatiolocal,
 //             UpdateLTRlocal restated for G).
-//   delayed : a window of n consecutive sites is decided by ONE CTA on the
-//   blockfb   n x n diagonal block of G held in shared memory; the accepted
-//             flips I are then applied to the full G as one rank-|I| product
-//                 G <- G - G[:, I] W (E_I^T - G[I, :]),  W = D_I (1 + A0_II D_I)^{-1}
-//             which equals the buffered sum of the paper's delayed vectors
-//             (Eqs. DelayTMat00, DelayRgenk, FinalDelay) and the block
-//             force-bias upgrade (Eq. BlkFrcBsTnew2).
+//   delayed : a window of consecutive sites is decided by ONE CTA on its diagonal block of G, held in
+//   blockfb   registers (FP64 block force bias: in shared memory); the accepted flips I are then applied
+//             to the full G as one rank-|I| product G <- G + X Y, the buffered sum of the paper's delayed
+//             vectors (Eqs. DelayTMat00, DelayRgenk, FinalDelay) and the block force-bias upgrade
+//             (Eq. BlkFrcBsTnew2): the columns of X and rows of Y follow from G[:, I] and G[I, :] by a
+//             recursion over the accepts.
 #include <math.h>
 
 #include "internal.h"
@@ -311,7 +310,7 @@ __global__ void __launch_bounds__(LOCAL_THREADS, 1) local_kernel(T* Gu, T* Gd, i
 // the grid barrier that fixes it, so with its update every CTA publishes its rows among the next LR_AHEAD
 // sites (double-buffered by phase); the rare accept beyond them costs a second barrier.  The arithmetic is
 // local_kernel's, element by element.  Bound by the barrier and the round trips to L2 (diagonal, row b):
-// 40 x 40: LR_US us per slice against 9.75 ms with G in L2.
+// 40 x 40, a pass of four slices and two recomputes: 62 ms with G in L2 (9.75 ms of it a slice), 43 ms so.
 constexpr int LR_THREADS = 448, LR_AHEAD = 4, LR_RPT_MAX = 11;
 inline size_t local_reg_pub(long ld) { return 2 * (size_t)(LR_AHEAD + 1) * 2 * ld; }  // floats of the row buffer
 
@@ -555,7 +554,7 @@ template <typename T> struct WinCap;
 template <> struct WinCap<float> { static constexpr int NW = 128; };
 template <> struct WinCap<double> { static constexpr int NW = 64; };
 constexpr int NBMAX = 32;
-constexpr int WIN_THREADS = 1024;  // 32 warps: the tail's W solve assigns 16 warps to each spin
+constexpr int WIN_THREADS = 1024;
 
 template <typename T>
 int window_max() { return WinCap<T>::NW; }
@@ -835,8 +834,8 @@ __global__ void __launch_bounds__(WinTile<T, NP>::THREADS) window_reg_kernel(
                 r0 = T(1) + e0 * b0[j];
                 r1 = T(1) + e1 * b1[j];
                 R = sf * r0 * r1;
-                const unsigned yes = __ballot_sync(FULL, ul[j] < fabs(R) && isfinite(R));
-                ball = (forced ? repm[j] : yes) & open;
+                const bool want = forced ? ((repm[j] >> lane) & 1u) != 0 : ul[j] < fabs(R);
+                ball = __ballot_sync(FULL, want && isfinite(R)) & open;  // never on a ratio that is not finite
             }
             // sites before the first accept are rejected; it and they are decided now
             const unsigned bit = ball & (0u - ball), done = ball ? open & (bit | (bit - 1u)) : open;
