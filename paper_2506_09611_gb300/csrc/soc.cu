@@ -83,7 +83,7 @@ __host__ __device__ __forceinline__ cx<T> cinv(cx<T> a) {
 
 // 2 x 2 complex block, row-major
 template <typename T>
-struct c22 {
+struct alignas(16) c22 {
     cx<T> a[2][2];
 };
 
@@ -214,6 +214,7 @@ struct SocWinArgs {
 };
 
 constexpr int SOC_PIPE_N = 32;  // windows of up to 32 sites run pipelined (the correction's staging buffer)
+constexpr int SOC_GJ_BUF = 16 * 16;
 
 template <typename T>
 __device__ __forceinline__ cx<T> g_at(const T* G, long ldz, int r, int c) {
@@ -291,6 +292,92 @@ __device__ bool gj_inverse_2x2(cx<T>* M, int m2, int ldm, cx<T>* colF, cx<T>* de
     return true;
 }
 
+// The same inverse with M in registers, m2 <= 32: thread (I, J) of the first 256 holds the 2 x 2 block (I, J).  Per
+// step the holders of pivot row and column put them into shared memory (double-buffered by step parity), and
+// after one barrier every thread takes the pivot's inverse, its columns of the scaled pivot row and its
+// block's update, with the operations of the shared-memory form one by one.  Bound by that latency chain (16
+// steps of one barrier instead of three for a 32 x 32 matrix).  Block force bias n_b = 16 at 24 x 24, with the
+// window's block of G in shared memory and one lane per proposal: the pass 59.0 -> 52.1 ms.  A tile of 64 x 64
+// (two blocks a thread) saved another 0.5 % of the pairing pass but rounds differently.  buf: 256 complex.
+template <typename T>
+__device__ bool gj_inverse_reg(cx<T>* M, int m2, int ldm, cx<T>* buf, cx<T>* det) {
+    constexpr int NB = 16, TH = NB * NB;
+    const int tid = threadIdx.x, nb = m2 / 2, J = tid % NB, I = tid / NB;
+    __shared__ int s_ok;
+    __syncthreads();
+    if (tid < TH) {
+        c22<T> B;
+        c22<T>* rowB = (c22<T>*)buf;   // [2][NB]
+        c22<T>* colB = rowB + 2 * NB;  // [2][NB]
+        auto publish = [&](int t, int par) {
+            if (I == t) rowB[par * NB + J] = B;
+            if (J == t) colB[par * NB + I] = B;
+        };
+#pragma unroll
+        for (int p = 0; p < 2; ++p)
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+                B.a[p][q] = (I < nb && J < nb) ? M[(2 * I + p) * ldm + 2 * J + q] : cmk((T)0, (T)0);
+        publish(0, 0);
+        cx<T> dacc = cmk((T)1, (T)0);
+        bool ok = true;
+        for (int t = 0; t < nb; ++t) {
+            const int par = t & 1;
+            named_barrier_sync(1, TH);
+            const c22<T> pb = rowB[par * NB + t], rw = rowB[par * NB + J], f = colB[par * NB + I];
+            const cx<T> a = pb.a[0][0], b = pb.a[0][1], c = pb.a[1][0], d = pb.a[1][1];
+            const cx<T> dt = csub(cmul(a, d), cmul(b, c));
+            const T mag = dt.r * dt.r + dt.i * dt.i;
+            if (!(mag > (T)0) || !isfinite(mag)) {  // uniform: every thread read the same block
+                ok = false;
+                break;
+            }
+            const cx<T> di = cinv(dt);
+            c22<T> P;
+            P.a[0][0] = cmul(d, di);
+            P.a[0][1] = cmul(cmk(-b.r, -b.i), di);
+            P.a[1][0] = cmul(cmk(-c.r, -c.i), di);
+            P.a[1][1] = cmul(a, di);
+            dacc = cmul(dacc, dt);
+            const bool pc = J == t;  // the pivot's own column: as if M were zero there and the row the inverse
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                cx<T> n0 = cmul(P.a[0][0], rw.a[0][q]), n1 = cmul(P.a[1][0], rw.a[0][q]);
+                cfma(n0, P.a[0][1], rw.a[1][q]);
+                cfma(n1, P.a[1][1], rw.a[1][q]);
+                n0 = pc ? P.a[0][q] : n0;
+                n1 = pc ? P.a[1][q] : n1;
+#pragma unroll
+                for (int p = 0; p < 2; ++p) {
+                    cx<T> w = pc ? cmk((T)0, (T)0) : B.a[p][q];
+                    cfma(w, cmk(-f.a[p][0].r, -f.a[p][0].i), n0);
+                    cfma(w, cmk(-f.a[p][1].r, -f.a[p][1].i), n1);
+                    B.a[p][q] = I != t ? w : p ? n1 : n0;
+                }
+            }
+            publish(t + 1, par ^ 1);
+        }
+        if (I < nb && J < nb)
+#pragma unroll
+            for (int p = 0; p < 2; ++p)
+#pragma unroll
+                for (int q = 0; q < 2; ++q) M[(2 * I + p) * ldm + 2 * J + q] = B.a[p][q];
+        if (tid == 0) {
+            s_ok = ok ? 1 : 0;
+            if (det) *det = dacc;
+        }
+    }
+    __syncthreads();
+    return s_ok != 0;
+}
+
+// The register form up to 32 x 32, the shared-memory form beyond.
+template <typename T>
+__device__ bool gj_inverse(cx<T>* M, int m2, int ldm, cx<T>* colF, cx<T>* buf, cx<T>* det) {
+    if (m2 <= 32) return gj_inverse_reg<T>(M, m2, ldm, buf, det);
+    return gj_inverse_2x2<T>(M, m2, ldm, colF, det);
+}
+
 // W = Delta_F Minv (2m x 2m complex, leading dimension ldw).  Delta_F is block diagonal: the
 // 2 x 2 block dl[t] of flipped site t.
 template <typename T>
@@ -353,14 +440,17 @@ __global__ void __launch_bounds__(512) soc_window_kernel(SocWinArgs a) {
 
     cx<T>* Mw = (cx<T>*)soc_smem;               // (2 kmax)^2: the window block / the LU matrix
     cx<T>* aux = Mw + 4 * a.kmax * a.kmax;      // 8 kmax: column / row snapshots, GJ scratch
-    cx<T>* Ys = aux + 8 * a.kmax;               // (2 SOC_PIPE_N)^2: staging of the correction
-    cx<T>* Gw = (cx<T>*)a.Gw0 + (long)z * 4 * a.kmax * a.kmax;  // n2 x n2: the block of the current G
+    cx<T>* gjb = aux + 8 * a.kmax;              // SOC_GJ_BUF: pivot rows and columns of gj_inverse_reg
+    cx<T>* Ys = gjb + SOC_GJ_BUF;               // (2 SOC_PIPE_N)^2: staging of the correction
+    // n2 x n2: the block of the current G, in shared memory where it fits
+    cx<T>* Gw = n <= SOC_PIPE_N ? Ys + 4 * SOC_PIPE_N * SOC_PIPE_N
+                                : (cx<T>*)a.Gw0 + (long)z * 4 * a.kmax * a.kmax;
     __shared__ cx<T> s_dl[64][2][2];            // flip deltas of the flipped sites
     __shared__ int s_site[64];
     __shared__ T s_uT[64];
     __shared__ int s_x[64], s_rep[64];
     __shared__ int s_m, s_acc;
-    __shared__ T s_logq;
+    __shared__ T s_logq, s_lq[64];
     __shared__ c22<T> s_w2;
     __shared__ cx<T> s_det;
     auto orb = [&](int q) { return (q & 1) ? N + s0 + (q >> 1) : s0 + (q >> 1); };
@@ -370,6 +460,9 @@ __global__ void __launch_bounds__(512) soc_window_kernel(SocWinArgs a) {
         s_x[t] = x[s0 + t];
         s_rep[t] = rep ? (int)rep[s0 + t] : -1;
     }
+    // the block's acceptance (mode 1), read ahead of its use
+    const T uacc = a.mode ? (T)u[N + a.blk] : (T)0;
+    const int racc = a.mode && rep ? (int)rep[N + a.blk] : -1;
     // ---- the window's block of the current G, into Gw ----
     {
         const int m2p = a.corr ? a.pKdev[z] : 0;
@@ -556,7 +649,7 @@ __global__ void __launch_bounds__(512) soc_window_kernel(SocWinArgs a) {
             }
             Mw[e] = v;
         }
-        if (!gj_inverse_2x2<T>(Mw, m2, m2, aux, nullptr)) {
+        if (!gj_inverse<T>(Mw, m2, m2, aux, gjb, nullptr)) {
             if (tid == 0) {
                 set_err(a.err, DEV_NUMERIC);
                 a.Kdev[z] = 0;
@@ -581,7 +674,7 @@ __global__ void __launch_bounds__(512) soc_window_kernel(SocWinArgs a) {
             }
             Mw[e] = v;
         }
-        if (!gj_inverse_2x2<T>(Mw, n2, n2, aux, nullptr)) {
+        if (!gj_inverse<T>(Mw, n2, n2, aux, gjb, nullptr)) {
             if (tid == 0) {
                 set_err(a.err, DEV_NUMERIC);
                 a.Kdev[z] = 0;
@@ -608,42 +701,52 @@ __global__ void __launch_bounds__(512) soc_window_kernel(SocWinArgs a) {
             }
         }
         __syncthreads();
-        if (tid == 0) {
+        if (warp == 0) {
             // obar_t = the stripped expectation of the field's generator, Abar = (1 + Delta_s) Minv A,
             // 1 + Delta_s = A(-gamma x): spin-y Abar[dn t, up t] - Abar[up t, dn t], spin-z
             // i (Abar[up t, up t] - Abar[dn t, dn t]); the proposal weight of x' is exp(x' h),
-            // h = gamma Re(obar) (bulk precision)
-            T logq = 0;
+            // h = gamma Re(obar) (bulk precision).  One lane per site.
             int m = 0;
-            for (int t = 0; t < n; ++t) {
-                const int i = s0 + t, xi = s_x[t];
-                const T c = (T)(a.k.c1m1 + 1.0), s = (T)(-xi * a.k.s1);  // spin-y A(-gamma x) = [[c, s], [-s, c]]
-                const cx<T> MA00 = aux[4 * t], MA01 = aux[4 * t + 1], MA10 = aux[4 * t + 2], MA11 = aux[4 * t + 3];
-                T h;
-                if (a.k.hs == AFQMC_SOC_HS_SZ) {  // spin-z A(-gamma x) = diag(c + i s, c - i s)
-                    const cx<T> uu = cmul(cmk(c, s), MA00), dd = cmul(cmk(c, -s), MA11);
-                    h = -(T)a.k.gamma * (uu.i - dd.i);
-                } else {
-                    const cx<T> dn_up = cadd(cscale(MA00, -s), cscale(MA10, c));
-                    const cx<T> up_dn = cadd(cscale(MA01, c), cscale(MA11, s));
-                    h = (T)a.k.gamma * (dn_up.r - up_dn.r);
+            for (int tb = 0; tb < n; tb += 32) {
+                const int t = tb + lane, i = s0 + t;
+                T h = 0;
+                int xi = 0, xp = 0;
+                if (t < n) {
+                    xi = s_x[t];
+                    const T c = (T)(a.k.c1m1 + 1.0), s = (T)(-xi * a.k.s1);  // spin-y A(-gamma x) = [[c, s], [-s, c]]
+                    const cx<T> MA00 = aux[4 * t], MA01 = aux[4 * t + 1], MA10 = aux[4 * t + 2], MA11 = aux[4 * t + 3];
+                    if (a.k.hs == AFQMC_SOC_HS_SZ) {  // spin-z A(-gamma x) = diag(c + i s, c - i s)
+                        const cx<T> uu = cmul(cmk(c, s), MA00), dd = cmul(cmk(c, -s), MA11);
+                        h = -(T)a.k.gamma * (uu.i - dd.i);
+                    } else {
+                        const cx<T> dn_up = cadd(cscale(MA00, -s), cscale(MA10, c));
+                        const cx<T> up_dn = cadd(cscale(MA01, c), cscale(MA11, s));
+                        h = (T)a.k.gamma * (dn_up.r - up_dn.r);
+                    }
+                    const T lp = (T)1 / ((T)1 + exp((T)-2 * h));
+                    lam[i] = (double)lp;
+                    xp = s_rep[t] >= 0 ? (s_rep[t] ? 1 : -1) : (s_uT[t] < lp ? 1 : -1);
+                    dec[i] = (uint8_t)(xp > 0);
                 }
-                const T lp = (T)1 / ((T)1 + exp((T)-2 * h));
-                lam[i] = (double)lp;
-                const int xp = s_rep[t] >= 0 ? (s_rep[t] ? 1 : -1) : (s_uT[t] < lp ? 1 : -1);
-                dec[i] = (uint8_t)(xp > 0);
+                const unsigned flips = __ballot_sync(0xffffffffu, xp != xi);
                 if (xp != xi) {
+                    const int k = m + __popc(flips & ((1u << lane) - 1u));
                     cx<T> dl[2][2];
                     site_delta<T>(a.k.hs, a.k.c2m1, a.k.s2, xi, dl);
                     for (int p = 0; p < 2; ++p)
-                        for (int q = 0; q < 2; ++q) s_dl[m][p][q] = dl[p][q];
-                    s_site[m] = i;
-                    logq += (T)(xi - xp) * h;
-                    ++m;
+                        for (int q = 0; q < 2; ++q) s_dl[k][p][q] = dl[p][q];
+                    s_site[k] = i;
+                    s_lq[k] = (T)(xi - xp) * h;
                 }
+                m += __popc(flips);
             }
-            s_m = m;
-            s_logq = logq;
+            __syncwarp();
+            if (lane == 0) {
+                T logq = 0;
+                for (int k = 0; k < m; ++k) logq += s_lq[k];
+                s_m = m;
+                s_logq = logq;
+            }
         }
         __syncthreads();
         const int m = s_m;
@@ -670,7 +773,7 @@ __global__ void __launch_bounds__(512) soc_window_kernel(SocWinArgs a) {
             }
             Mw[e] = v;
         }
-        const bool ok = gj_inverse_2x2<T>(Mw, m2, m2, aux, &s_det);
+        const bool ok = gj_inverse<T>(Mw, m2, m2, aux, gjb, &s_det);
         if (tid == 0) {
             const cx<T> dt = ok ? s_det : cmk((T)0, (T)0);
             const T f = exp(s_logq);
@@ -679,22 +782,17 @@ __global__ void __launch_bounds__(512) soc_window_kernel(SocWinArgs a) {
             ratio[2 * (N + a.blk)] = (double)Rr;
             ratio[2 * (N + a.blk) + 1] = (double)Ri;
             if (!isfinite(absR)) set_err(a.err, DEV_NUMERIC);
-            const int racc = rep ? (int)rep[N + a.blk] : -1;
-            const int acc = racc >= 0 ? (racc != 0) : ((T)u[N + a.blk] < absR);
+            const int acc = racc >= 0 ? (racc != 0) : (uacc < absR);
             dec[N + a.blk] = (uint8_t)acc;
             s_acc = acc && ok && absR > (T)0 && isfinite(absR);
-            if (s_acc) {
-                for (int t = 0; t < m; ++t) {
-                    sites[t] = s_site[t];
-                    x[s_site[t]] = (int8_t)(-x[s_site[t]]);
-                }
-                a.Kdev[z] = m2;
-            } else {
-                a.Kdev[z] = 0;
-            }
+            a.Kdev[z] = s_acc ? m2 : 0;
         }
         __syncthreads();
         if (!s_acc) return;
+        for (int t = tid; t < m; t += nt) {
+            sites[t] = s_site[t];
+            x[s_site[t]] = (int8_t)(-s_x[s_site[t] - s0]);
+        }
     }
     write_W<T>(Mw, m2, m2, s_dl, W, ldw);
     if (tid == 0) a.Kdev[z] = m2;
@@ -1571,7 +1669,7 @@ cudaError_t soc_wrap(afqmc_soc_ctx* ctx, cudaStream_t st, const int8_t* xl, int 
 
 template <typename T>
 size_t window_smem(int kmax) {
-    return (size_t)(4 * kmax * kmax + 8 * kmax + 4 * SOC_PIPE_N * SOC_PIPE_N) * sizeof(cx<T>);
+    return (size_t)(4 * kmax * kmax + 8 * kmax + SOC_GJ_BUF + 8 * SOC_PIPE_N * SOC_PIPE_N) * sizeof(cx<T>);
 }
 
 // ---- one window: chain, then X' = G[:, F] W and the out-of-place flush ----
