@@ -27,6 +27,11 @@ __device__ __forceinline__ double* lu_A(const LuArgs& a, int b) {
 constexpr int LU_NB = 32;
 constexpr int LU_NBP = LU_NB + 1;
 
+// A pivoted row's flag: its panel's number from 1 (a trailing update that runs beside the next panel tells
+// the rows of that panel, which it still updates, from the earlier ones).
+constexpr int LU_PANELS_MAX = 254;
+__device__ __forceinline__ int8_t lu_flag(int j0) { return (int8_t)min(j0 / LU_NB + 1, LU_PANELS_MAX + 1); }
+
 // One cluster of CS CTAs per matrix (blockIdx.x / CS = matrix).  Factors columns
 // [j0, j0 + nbk) over the rows not yet pivoted.
 // Pivot candidates compare |a| through the bit pattern of the double with the sign cleared:
@@ -122,7 +127,7 @@ __device__ __forceinline__ bool lu_bar_wait(unsigned bar, unsigned parity) {
 // candidates read back through distributed shared memory behind a cluster barrier; 77 us with the
 // candidates pushed before the cluster barrier and the pivot row read after it.
 template <int CS>
-__global__ void __launch_bounds__(256) lu_panel_kernel(LuArgs a, int j0, int nbk, int tpr) {
+__device__ __forceinline__ void lu_panel(const LuArgs& a, int j0, int nbk, int tpr) {
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank();
     const int mat = blockIdx.x / CS;
@@ -201,7 +206,7 @@ __global__ void __launch_bounds__(256) lu_panel_kernel(LuArgs a, int j0, int nbk
         const double pinv = bad ? 0.0 : lu_rcp(urow[jj]);
         any_bad = any_bad || bad;
         if (tid == 0) {
-            if (p >= r0 && p < r1) fl[p - r0] = 1;
+            if (p >= r0 && p < r1) fl[p - r0] = lu_flag(j0);
             if (rank == 0) perm[j0 + jj] = p;
         }
         // own unpivoted rows: multiplier into column jj, rank-1 step on the later panel columns, and the
@@ -250,6 +255,11 @@ __global__ void __launch_bounds__(256) lu_panel_kernel(LuArgs a, int j0, int nbk
     for (int q = tid; q < nr; q += nt) flag[r0 + q] = fl[q];
 }
 
+template <int CS>
+__global__ void __launch_bounds__(256) lu_panel_kernel(LuArgs a, int j0, int nbk, int tpr) {
+    lu_panel<CS>(a, j0, nbk, tpr);
+}
+
 // U12 = L11^{-1} A12 on the pivot rows of a panel, columns [j0 + nbk, n): eight lanes per column, lane h
 // holds the entries h, h + 8, ... (the FP64 work of a column is sequential, so a column spreads over lanes
 // and the columns over the whole GPU).  Grid (16-column blocks, matrix).
@@ -288,20 +298,19 @@ __global__ void __launch_bounds__(8 * LU_UC) lu_u12_kernel(LuArgs a, int j0, int
             if (h + 8 * t < nbk && h + 8 * t > 0) A[(long)perm[h + 8 * t] * lda + c] = v[t];
 }
 
-// A[r][c] -= sum_k A[r][j0 + k] U12[k][c] for the unpivoted rows r and c in [j0 + nbk, n), with U12[k] the
-// pivot row perm[j0 + k].  BM x BN tiles, BM / 16 x BN / 16 outputs per thread; grid (tiles of the unpivoted
-// rows, column tiles, matrix).  A block finds its rows by counting the flags, so no multiply-add goes to a
+// A[r][c] -= sum_k A[r][j0 + k] U12[k][c] for the rows r that were unpivoted after the panel at j0 and c in
+// [ca, cb), with U12[k] the pivot row perm[j0 + k]: tile (bx, by) of BM of these rows x BN columns, BM / 16 x
+// BN / 16 outputs per thread.  A block finds its rows by counting the flags, so no multiply-add goes to a
 // pivoted row (they are the bound: 2 a clock and SM).
 template <int BM, int BN>
-__global__ void __launch_bounds__(256) lu_update_kernel(LuArgs a, int j0, int nbk) {
+__device__ __forceinline__ void lu_update(const LuArgs& a, int j0, int nbk, int ca, int cb, int bx, int by, int mat) {
     constexpr int TM = BM / 16, TN = BN / 16;
-    const int mat = blockIdx.z;
     double* A = lu_A(a, mat);
     const int* perm = a.perm0 + (long)mat * a.pstride;
     const int8_t* flag = a.flag0 + (long)mat * a.pstride;
     const long lda = a.lda;
-    const int m = a.m, n = a.n;
-    const int f0 = blockIdx.x * BM, c0 = j0 + nbk + blockIdx.y * BN;
+    const int m = a.m, n = cb, closed = (uint8_t)lu_flag(j0);
+    const int f0 = bx * BM, c0 = ca + by * BN;
     __shared__ double Ls[BM][LU_NBP];
     __shared__ double Us[LU_NB][BN + 1];
     __shared__ int rid[BM];
@@ -310,7 +319,8 @@ __global__ void __launch_bounds__(256) lu_update_kernel(LuArgs a, int j0, int nb
     for (int q = tid; q < BM; q += 256) rid[q] = -1;
     for (int base = 0, seen = 0; base < m && seen < f0 + BM; base += 256) {
         const int r = base + tid;
-        const bool open = r < m && !flag[r];
+        const int f = r < m ? (int)(uint8_t)flag[r] : closed;
+        const bool open = f == 0 || f > closed;
         const unsigned ball = __ballot_sync(0xffffffffu, open);
         if (lane == 0) wsum[wid] = __popc(ball);
         __syncthreads();
@@ -362,10 +372,32 @@ __global__ void __launch_bounds__(256) lu_update_kernel(LuArgs a, int j0, int nb
     }
 }
 
+// Grid (tiles of the unpivoted rows, column tiles, matrix).
 template <int BM, int BN>
-static cudaError_t launch_update(cudaStream_t st, const LuArgs& a, int j0, int nbk, int mr, int nc) {
+__global__ void __launch_bounds__(256) lu_update_kernel(LuArgs a, int j0, int nbk, int ca, int cb) {
+    lu_update<BM, BN>(a, j0, nbk, ca, cb, blockIdx.x, blockIdx.y, blockIdx.z);
+}
+
+// The panel at j0 on the first CS nmat blocks and, on the others, the trailing update of the panel before it
+// on the columns right of this one (their tiles: nx x ny per matrix).  The two touch different columns, and
+// no block waits for one outside its cluster.  Against the update in a launch of its own: the 24 x 24 spin-coupled
+// pass 52.1 -> 50.0 ms, 40 x 40 62.8 -> 61.7 ms, eight 20 x 20 pairing walkers 204.9 -> 202.6 ms.
+template <int CS, int BM, int BN>
+__global__ void __launch_bounds__(256) lu_step_kernel(LuArgs a, int j0, int nbk, int tpr, int nx, int ny) {
+    const int b = (int)blockIdx.x - CS * a.nmat;
+    if (b < 0) {
+        lu_panel<CS>(a, j0, nbk, tpr);
+    } else if (b < nx * ny * a.nmat) {
+        const int t = b % (nx * ny);
+        lu_update<BM, BN>(a, j0 - LU_NB, LU_NB, j0 + nbk, a.n, t % nx, t / nx, b / (nx * ny));
+    }
+}
+
+template <int BM, int BN>
+static cudaError_t launch_update(cudaStream_t st, const LuArgs& a, int j0, int nbk, int mr, int ca, int cb) {
     count_launch();
-    lu_update_kernel<BM, BN><<<dim3((mr + BM - 1) / BM, (nc + BN - 1) / BN, a.nmat), 256, 0, st>>>(a, j0, nbk);
+    lu_update_kernel<BM, BN><<<dim3((mr + BM - 1) / BM, (cb - ca + BN - 1) / BN, a.nmat), 256, 0, st>>>(a, j0, nbk, ca,
+                                                                                                      cb);
     return cudaGetLastError();
 }
 
@@ -423,10 +455,18 @@ __global__ void __launch_bounds__(LS_THREADS) lu_sign_kernel(LuArgs a, int parit
     if ((__syncthreads_count(odd) & 1) && tid == 0) sign_out[wk] = -sign_out[wk];
 }
 
+// Dynamic shared memory of a panel's CTA, and the most of it beside the trailing update's static tiles.
+static size_t lu_panel_smem(int m, int cs) {
+    const size_t rpc = (m + cs - 1) / cs;
+    return rpc * LU_NBP * sizeof(double) + rpc + 16;
+}
+constexpr size_t LU_STEP_SMEM = 144 * 1024;
+
+// mr > 0: with the update of the mr rows unpivoted after the panel before, on the columns right of this one.
 template <int CS>
-static cudaError_t launch_panel(cudaStream_t st, const LuArgs& a, int j0, int nbk) {
+static cudaError_t launch_panel(cudaStream_t st, const LuArgs& a, int j0, int nbk, int mr) {
     const int rpc = (a.m + CS - 1) / CS;
-    const size_t shm = (size_t)rpc * LU_NBP * sizeof(double) + (size_t)rpc + 16;
+    const size_t shm = lu_panel_smem(a.m, CS);
     {
         cudaError_t e = ensure_smem_attr((const void*)lu_panel_kernel<CS>, 227 * 1024 - 16 * 1024);
         if (e != cudaSuccess) return e;
@@ -450,7 +490,18 @@ static cudaError_t launch_panel(cudaStream_t st, const LuArgs& a, int j0, int nb
     int tpr = 8;  // threads per row: all 256 threads busy
     while (tpr > 1 && rpc * tpr > 256) tpr /= 2;
     count_launch();
-    return cudaLaunchKernelEx(&cfg, lu_panel_kernel<CS>, a, j0, nbk, tpr);
+    if (mr == 0) return cudaLaunchKernelEx(&cfg, lu_panel_kernel<CS>, a, j0, nbk, tpr);
+    // with the previous panel's update: the tile whose busiest SM issues the fewest multiply-adds
+    const int nc = a.n - j0 - nbk;
+    auto tiles = [&](int b) { return (long)((mr + b - 1) / b) * ((nc + b - 1) / b) * a.nmat; };
+    const bool big = (tiles(64) + 151) / 152 * (64 * 64 + 128) <= (tiles(32) + 151) / 152 * (32 * 32 + 128);
+    const int b = big ? 64 : 32, nx = (mr + b - 1) / b, ny = (nc + b - 1) / b;
+    auto kern = big ? lu_step_kernel<CS, 64, 64> : lu_step_kernel<CS, 32, 32>;
+    cudaError_t e = ensure_smem_attr((const void*)kern, LU_STEP_SMEM);
+    if (e == cudaSuccess && CS > 8) e = ensure_func_attr((const void*)kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    cfg.gridDim = dim3((unsigned)(CS * a.nmat + (tiles(b) + CS - 1) / CS * CS));
+    return cudaLaunchKernelEx(&cfg, kern, a, j0, nbk, tpr, nx, ny);
 }
 
 // Cluster size: enough CTAs per matrix that a panel step's FP64 work per SM stays small, few
@@ -496,33 +547,43 @@ cudaError_t launch_lu(cudaStream_t st, const LuArgs& a) {
     if ((a.m + cs - 1) / cs * (LU_NBP * sizeof(double) + 1) > 200 * 1024) return cudaErrorInvalidValue;
     cudaError_t e;
     if ((e = cudaMemsetAsync(a.flag0, 0, (size_t)(a.nmat - 1) * a.pstride + a.m, st)) != cudaSuccess) return e;
+    // Look-ahead: a panel's update goes to the next panel's columns first (a launch of its own), the rest of it
+    // beside the next panel, whose chain leaves most of the FP64 units idle; only where that rest is more than
+    // two 32 x 32 tiles an SM (below, the extra launch costs what it hides: four 441 x 138 factors 32.3 ms a
+    // pass without, 32.4 with it).
+    const bool ahead = a.n <= LU_PANELS_MAX * LU_NB && lu_panel_smem(a.m, cs) <= LU_STEP_SMEM;
+    int mr_open = 0;  // rows of the update that goes with the next panel, 0: none
     for (int j0 = 0; j0 < a.n; j0 += LU_NB) {
         const int nbk = (a.n - j0 < LU_NB) ? a.n - j0 : LU_NB;
         switch (cs) {
-            case 1: e = launch_panel<1>(st, a, j0, nbk); break;
-            case 2: e = launch_panel<2>(st, a, j0, nbk); break;
-            case 4: e = launch_panel<4>(st, a, j0, nbk); break;
-            case 8: e = launch_panel<8>(st, a, j0, nbk); break;
-            default: e = launch_panel<16>(st, a, j0, nbk); break;
+            case 1: e = launch_panel<1>(st, a, j0, nbk, mr_open); break;
+            case 2: e = launch_panel<2>(st, a, j0, nbk, mr_open); break;
+            case 4: e = launch_panel<4>(st, a, j0, nbk, mr_open); break;
+            case 8: e = launch_panel<8>(st, a, j0, nbk, mr_open); break;
+            default: e = launch_panel<16>(st, a, j0, nbk, mr_open); break;
         }
         if (e != cudaSuccess) return e;
-        const int nc = a.n - j0 - nbk, mr = a.m - j0 - nbk;
-        if (nc > 0) {
-            count_launch();
-            lu_u12_kernel<<<dim3((nc + LU_UC - 1) / LU_UC, a.nmat), 8 * LU_UC, 0, st>>>(a, j0, nbk);
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
-            if (mr <= 0) continue;
-            // the tile whose busiest SM issues the fewest multiply-adds (plus a fixed cost per tile)
-            auto cost = [&](int bm, int bn) {
-                const long t = (long)((mr + bm - 1) / bm) * ((nc + bn - 1) / bn) * a.nmat;
-                return (t + 151) / 152 * (bm * bn + 128);
-            };
-            const long c64 = cost(64, 64), c36 = cost(32, 64), c33 = cost(32, 32);
-            if (c64 <= c36 && c64 <= c33) e = launch_update<64, 64>(st, a, j0, nbk, mr, nc);
-            else if (c36 <= c33) e = launch_update<32, 64>(st, a, j0, nbk, mr, nc);
-            else e = launch_update<32, 32>(st, a, j0, nbk, mr, nc);
-            if (e != cudaSuccess) return e;
+        const int ca = j0 + nbk, nc = a.n - ca, mr = a.m - ca;
+        if (nc <= 0) break;
+        count_launch();
+        lu_u12_kernel<<<dim3((nc + LU_UC - 1) / LU_UC, a.nmat), 8 * LU_UC, 0, st>>>(a, j0, nbk);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        mr_open = 0;
+        if (mr <= 0) continue;
+        if (ahead && (long)((mr + 31) / 32) * ((nc - 1) / 32) * a.nmat > 304) {
+            if ((e = launch_update<32, 16>(st, a, j0, nbk, mr, ca, ca + LU_NB)) != cudaSuccess) return e;
+            mr_open = mr;
+            continue;
         }
+        // the tile whose busiest SM issues the fewest multiply-adds (plus a fixed cost per tile)
+        auto cost = [&](int bm, int bn) {
+            const long t = (long)((mr + bm - 1) / bm) * ((nc + bn - 1) / bn) * a.nmat;
+            return (t + 151) / 152 * (bm * bn + 128);
+        };
+        const long c64 = cost(64, 64), c33 = cost(32, 32);
+        if (c64 <= c33) e = launch_update<64, 64>(st, a, j0, nbk, mr, ca, a.n);
+        else e = launch_update<32, 32>(st, a, j0, nbk, mr, ca, a.n);
+        if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
