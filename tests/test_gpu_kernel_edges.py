@@ -9,6 +9,7 @@ import pytest
 
 import oracle
 from paper_2506_09611_gb300 import inputs
+from tests import test_gpu_soc as gsoc
 from tests.test_gpu_parity import FP32_TOL, FP64_TOL, _replay, _run_sweep, make, rel
 
 pytestmark = pytest.mark.gpu
@@ -82,10 +83,10 @@ def test_local_update_sparse_accepts_fp32(L, ns):
     _replay_sweep(L, ns, "local", slices=1, keep=0.15)
 
 
-@pytest.mark.parametrize("L,ns", [(9, 1), (9, 31), (9, 32), (9, 33), (9, 64), (9, 65), (17, 100), (27, 203)])
+@pytest.mark.parametrize("L,ns", [(9, 1), (9, 31), (9, 32), (9, 33), (9, 64), (9, 65), (17, 100), (27, 203), (33, 401)])
 def test_factorisation_and_solve(L, ns):
     """G(0) and a recompute: LU panels and solves with whole and partial 32-blocks, one to several CTAs per
-    matrix."""
+    matrix, and (33 x 33) trailing updates beside the next panel until they are too small."""
     ctx, w, P, X = make(L, ns, 2, stab=1)
     with ctx:
         for s in range(2):
@@ -163,3 +164,12 @@ def test_pairing_dft_sizes(L, ns):
         mk, mkp = [(-(q // L) % L) * L + (-(q % L)) % L for q in (k, kp)]
         ref = At[kp, k] * At[N + mkp, N + mk] - At[N + mkp, k] * At[kp, N + mk]
         assert abs(got["Mk"][0][k, kp] - ref) < 1e-11
+
+
+@pytest.mark.parametrize("mode,k,nb", [("blockfb", 1, 15), ("blockfb", 1, 16), ("blockfb", 1, 17), ("blockfb", 1, 32),
+                                       ("delayed", 16, 1), ("delayed", 32, 1)])
+def test_soc_window_inverse(mode, k, nb):
+    """Window matrices up to and beyond the 32 x 32 register tile, with a ragged last window (36 sites)."""
+    ctx, w = gsoc.make(6, 36, 2, 1, seed=23)
+    with ctx:
+        gsoc._free_run(ctx, w, mode, k, nb, 23, 4, 1, FP64_TOL)
