@@ -339,7 +339,7 @@ def main():
     kernels = kernel_rooflines(prof, args.gemm, pk, pk_src, args.steps)
     roof = dict(kernels[0]) if kernels else None
     l2_gbs = optional_leg("l2_copy", lambda: l2_copy_bandwidth(torch))
-    kernels += local_and_chain_rooflines(cmp_prof, pk, pk_src, l2_gbs if isinstance(l2_gbs, float) else None)
+    kernels += local_and_chain_rooflines(cmp_prof, l2_gbs if isinstance(l2_gbs, float) else None)
 
 
     # ---------------- end to end through the C ABI with host buffers ----------------
@@ -441,7 +441,7 @@ def main():
         dist.destroy_process_group()
 
 
-def compare_modes(afqmc, ctx, stream, k, nb, n_slices, stab=STAB, elem_bytes=4):
+def compare_modes(afqmc, ctx, stream, k, nb, n_slices, stab=STAB):
     """Local, block force-bias and delayed updates on the same walker: each mode sweeps slices
     1..n_slices forward under the library's phase profiler (its recomputes included), then the walker
     walks back to slice 0 with the delayed update so that the next mode starts from the same place.
@@ -475,45 +475,35 @@ def compare_modes(afqmc, ctx, stream, k, nb, n_slices, stab=STAB, elem_bytes=4):
                      "acceptance": acc / max(props, 1), "slices": len(sample),
                      "k" if mode == "delayed" else ("nb" if mode == "blockfb" else "kind"):
                          (k if mode == "delayed" else (nb if mode == "blockfb" else "rank-1 update per accept"))}
-        raw[mode] = {"prof": p, "proposals": props, "accepts": acc, "flipped": flips, "slices": len(sample),
-                     "elem_bytes": elem_bytes}
+        raw[mode] = {"prof": p, "proposals": props, "accepts": acc, "flipped": flips, "slices": len(sample)}
     return cmp, raw
 
 
-def local_and_chain_rooflines(raw, pk, pk_src, l2_gbs):
-    """The local update's rank-1 read-modify-write and the delayed window chain, from the comparison
-    sample's intervals.
-    * local_kernel: each accepted flip reads and writes both spins' G once: 2 x 2 x N^2 x s bytes
-      (s = element size); achieved = those bytes x accepts / the kernel's time (one launch per slice).
-      G of both spins (20.5 MB in FP32) stays in the 129 MB L2, so the fraction is given against the
-      measured HBM copy bandwidth and against an L2-resident copy measured in this run.
-    * window chain (window kernel + next-window block, one CTA per walker): latency-bound; reported as
-      time per proposed site and per accept."""
+def local_and_chain_rooflines(raw, l2_gbs):
+    """The local update and the delayed window chain, from the comparison sample's intervals.
+    * local update (FP32): G of both spins stays in registers for a slice, so an accept is bound by the
+      grid barrier and the round trips to L2; reported as time per accept.
+    * window chain (window and panel kernels): latency-bound; reported as time per proposed site and per
+      accept."""
     out = []
     lo = raw["local"]
     ph = lo["prof"]["local"]
     if ph["intervals"] and lo["accepts"]:
-        per_acc = 2 * 2 * N * N * lo["elem_bytes"]
-        ach = per_acc * lo["accepts"] / (ph["ms"] / 1e3) / 1e9
-        out.append({"kernel": "local_kernel (rank-1 update per accepted flip, both spins, one cooperative launch "
-                              "per slice)", "bound": "hbm", "achieved": ach, "peak": pk["hbm_gbs"], "unit": "GB/s",
-                    "frac": ach / pk["hbm_gbs"], "l2_copy_gbs": l2_gbs,
-                    "frac_of_l2_copy": (ach / l2_gbs) if l2_gbs else None,
-                    "traffic": None, "launches": ph["intervals"], "ms_per_launch": ph["ms"] / ph["intervals"],
-                    "us_per_accept": ph["ms"] * 1e3 / lo["accepts"], "work_per_accept": per_acc,
-                    "accepts_per_launch": lo["accepts"] / ph["intervals"],
-                    "peak_source": "measured HBM copy (of %s); G is L2-resident: l2_copy_gbs is a copy of an "
-                                   "80 MB working set (src + dst) timed in this run" % pk_src})
+        out.append({"kernel": "local_reg_kernel (rank-1 update per accepted flip, both spins, one cooperative launch "
+                              "per slice)", "bound": "latency", "launches": ph["intervals"],
+                    "ms_per_launch": ph["ms"] / ph["intervals"], "us_per_accept": ph["ms"] * 1e3 / lo["accepts"],
+                    "accepts_per_launch": lo["accepts"] / ph["intervals"], "l2_copy_gbs": l2_gbs,
+                    "note": "the rows of G stay in registers for the slice; an accept costs one grid barrier and "
+                            "two round trips to L2"})
     de = raw["delayed"]
     ch = de["prof"]["chain"]
     if ch["intervals"] and de["accepts"]:
-        out.append({"kernel": "window chain (window_kernel + next_block_kernel, delayed, one CTA)",
+        out.append({"kernel": "window chain (window_reg_kernel + panel_kernel, delayed)",
                     "bound": "latency", "ns_per_site": ch["ms"] * 1e6 / de["proposals"],
                     "ns_per_accept": ch["ms"] * 1e6 / de["accepts"], "ms_per_slice": ch["ms"] / de["slices"],
                     "acceptance": de["accepts"] / max(de["proposals"], 1),
-                    "note": "the serial Metropolis chain of the delayed update; the bound it is compared "
-                            "with is stated in the design notes (one 1024-thread block barrier plus one "
-                            "warp scan per accept)"})
+                    "note": "the serial Metropolis chain of the delayed update; per accept two "
+                            "barriers of ten warps and the deciding warp's dependent path"})
     return out
 
 
@@ -676,7 +666,7 @@ def fp64_bulk_leg(afqmc, torch, stream, args, seed):
                     afqmc.afqmc_recompute_G(c.h, None, stream)
 
         ms = tune.time_on_stream(torch, stream, sweep)
-        cmp, _ = compare_modes(afqmc, c, stream, k64, args.nb, 4, elem_bytes=8)
+        cmp, _ = compare_modes(afqmc, c, stream, k64, args.nb, 4)
         return {"value": N * M * 2 / (ms / 1e3), "unit": UNIT, "ms_per_step": ms, "k": k64,
                 "compare_sample": cmp,
                 "speedup_update_only_vs_local": {m: cmp[m]["update_only"] / cmp["local"]["update_only"]
@@ -755,7 +745,7 @@ OZ_PAIRS = 45
 # DRAM bytes per launch (read + write) from one ncu capture of the current kernel on this
 # workload; None where the phase spans several kernels or no capture of the current kernel exists.
 NCU_TRAFFIC = {"elim": None, "lu_o": None,
-               "solve": 25.807104e6 + 0.080896e6,      # lu_solve_kernel, 700 x 700, 1600 right-hand sides
+               "solve": None,
                "wrap_gemm": 30.749184e6 + 0.02432e6,   # tc_gemm_kernel<160, split3>, 1600^3, both spins
                "flush_gemm": 22.055936e6 + 0.0,        # rankm_kernel, 1600 x 1600 x m, both spins (writes stay in L2)
                # sep_line_circ_kernel<float, 40>: the four passes of one wrap (cold cache: 20.53 MB read per
