@@ -156,6 +156,11 @@ int afqmc_get_info(afqmc_ctx* ctx, int walker, int* N, int* n_up, int* n_dn, int
  * out[j] = u(seed, walker, visit, j) for j < count (device generator, copied to the host). */
 int afqmc_debug_uniforms(uint64_t seed, uint64_t walker, uint64_t visit, int count, double* host_out);
 
+/* Validation hook for the kernels' own division: for j < count (host arrays, FP64 but quotf) quot[j] = x[j] / y[j]
+ * and rcp[j] = 1 / y[j] as the FP64 accept factors and LU pivots take them, quotf[j] = x[j] / y[j] (both rounded
+ * to FP32 first) as the FP32 accept factors do. */
+int afqmc_debug_quotients(int count, const double* x, const double* y, double* quot, double* rcp, float* quotf);
+
 /* Validation hook for the bounded device waits: one thread waits on a device flag that nothing
  * sets, for limit_ns nanoseconds of %globaltimer (1000 <= limit_ns <= 2e9), then records the device
  * timeout code and returns.  Every bounded wait of the library (grid barriers, mbarrier waits)

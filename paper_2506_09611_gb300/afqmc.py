@@ -25,8 +25,9 @@ GEMMS = {"tc3": 0, "simt": 1, "tf32": 2}
 
 EXPORTS = ["afqmc_create", "afqmc_destroy", "afqmc_init_walkers", "afqmc_sweep_slice", "afqmc_recompute_G",
            "afqmc_measure_energy", "afqmc_get_G", "afqmc_set_G", "afqmc_get_fields", "afqmc_get_decisions",
-           "afqmc_get_ratios", "afqmc_get_info", "afqmc_debug_uniforms", "afqmc_set_profiling", "afqmc_set_graphs",
-           "afqmc_get_profile", "afqmc_launch_count", "afqmc_apply_flips", "afqmc_apply_flips_noalloc",
+           "afqmc_get_ratios", "afqmc_get_info", "afqmc_debug_uniforms", "afqmc_debug_quotients",
+           "afqmc_set_profiling", "afqmc_set_graphs", "afqmc_get_profile", "afqmc_launch_count",
+           "afqmc_apply_flips", "afqmc_apply_flips_noalloc",
            "afqmc_debug_gemm", "afqmc_debug_dgemm", "afqmc_debug_ozaki_plan", "afqmc_debug_wait_timeout",
            "afqmc_set_wrap", "afqmc_set_wrap_tile", "afqmc_set_form", "afqmc_strerror", "afqmc_cp_init",
            "afqmc_cp_step", "afqmc_cp_comb", "afqmc_cp_reorth", "afqmc_cp_energy", "afqmc_cp_get_walker"]
@@ -79,6 +80,7 @@ def load(path: str = LIB_PATH):
     lib.afqmc_get_ratios.argtypes = [vp, ctypes.c_int, dp]
     lib.afqmc_get_info.argtypes = [vp, ctypes.c_int, ip, ip, ip, ip, ip]
     lib.afqmc_debug_uniforms.argtypes = [ctypes.c_uint64, ctypes.c_uint64, ctypes.c_uint64, ctypes.c_int, dp]
+    lib.afqmc_debug_quotients.argtypes = [ctypes.c_int, dp, dp, dp, dp, ctypes.POINTER(ctypes.c_float)]
     lib.afqmc_debug_wait_timeout.argtypes = [ctypes.c_longlong, vp]
     lib.afqmc_set_profiling.argtypes = [vp, ctypes.c_int]
     lib.afqmc_set_graphs.argtypes = [vp, ctypes.c_int]
@@ -222,6 +224,16 @@ def afqmc_debug_uniforms(seed, walker, visit, count):
     out = np.zeros(count)
     _ck("afqmc_debug_uniforms", load().afqmc_debug_uniforms(seed, walker, visit, count, _ptr(out, ctypes.c_double)))
     return out
+
+
+def afqmc_debug_quotients(x, y):
+    """x / y and 1 / y as the FP64 kernels take them, and x / y as the FP32 kernels do."""
+    x, y = np.ascontiguousarray(x, np.float64), np.ascontiguousarray(y, np.float64)
+    q, r, qf = np.empty(x.size), np.empty(x.size), np.empty(x.size, np.float32)
+    _ck("afqmc_debug_quotients", load().afqmc_debug_quotients(
+        x.size, _ptr(x, ctypes.c_double), _ptr(y, ctypes.c_double), _ptr(q, ctypes.c_double),
+        _ptr(r, ctypes.c_double), _ptr(qf, ctypes.c_float)))
+    return q, r, qf
 
 
 def afqmc_debug_wait_timeout(limit_ns, stream=None):

@@ -251,6 +251,14 @@ __global__ void debug_wait_kernel(const unsigned int* flag, unsigned long long l
     }
 }
 
+__global__ void debug_quotients_kernel(int count, const double* x, const double* y, double* q, double* r, float* qf) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= count) return;
+    q[j] = fast_quot(x[j], y[j]);
+    r[j] = fast_rcp(y[j]);
+    qf[j] = fast_quot((float)x[j], (float)y[j]);
+}
+
 __global__ void debug_uniforms_kernel(uint64_t seed, uint64_t walker, uint64_t visit, int count, double* out) {
     int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j < count) out[j] = philox_uniform(seed, walker, visit, (uint64_t)j);
@@ -2344,6 +2352,26 @@ int afqmc_debug_wait_timeout(long long limit_ns, void* stream) {
     if (e != cudaSuccess) return AFQMC_ERR_CUDA;
     if (h == DEV_TIMEOUT) return AFQMC_ERR_TIMEOUT;
     return h ? AFQMC_ERR_CUDA : AFQMC_OK;
+}
+
+int afqmc_debug_quotients(int count, const double* x, const double* y, double* quot, double* rcp, float* quotf) {
+    if (count < 0 || (count > 0 && (!x || !y || !quot || !rcp || !quotf))) return AFQMC_ERR_ARG;
+    if (count == 0) return AFQMC_OK;
+    const size_t n = (size_t)count;
+    double* d = nullptr;  // x, y, quot, rcp, then quotf
+    if (cudaMalloc(&d, n * 36) != cudaSuccess) return AFQMC_ERR_OOM;
+    cudaError_t e = cudaMemcpy(d, x, n * 8, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(d + n, y, n * 8, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) {
+        count_launch();
+        debug_quotients_kernel<<<(count + 255) / 256, 256>>>(count, d, d + n, d + 2 * n, d + 3 * n, (float*)(d + 4 * n));
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaMemcpy(quot, d + 2 * n, n * 8, cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess) e = cudaMemcpy(rcp, d + 3 * n, n * 8, cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess) e = cudaMemcpy(quotf, d + 4 * n, n * 4, cudaMemcpyDeviceToHost);
+    cudaFree(d);
+    return e == cudaSuccess ? AFQMC_OK : AFQMC_ERR_CUDA;
 }
 
 int afqmc_debug_uniforms(uint64_t seed, uint64_t walker, uint64_t visit, int count, double* host_out) {

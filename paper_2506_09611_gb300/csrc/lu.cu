@@ -49,22 +49,6 @@ __device__ __forceinline__ void lu_pick(unsigned long long& k, int& r, double& x
     }
 }
 
-// 1 / x for a pivot: a 22-bit reciprocal of x's leading bits, taken in FP32 from the bit pattern, and one
-// step of Halley's iteration (1/x = s (1 + e + e^2 + ...), e = 1 - s x, error e^3 < 2^-63); outside the FP32
-// exponent range the division.  Three dependent FP64 operations where a division takes about 740 cycles.
-__device__ __forceinline__ double lu_rcp(double x) {
-    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-    const int ex = (int)((hi >> 20) & 0x7ffu) - 1023;
-    if (ex < -100 || ex > 100) return 1.0 / x;
-    const float xm = __uint_as_float(0x3f800000u | ((hi & 0xfffffu) << 3) | (lo >> 29));
-    const unsigned rb = __float_as_uint(__fdividef(1.0f, xm));
-    const int re = (int)((rb >> 23) & 0xffu) - 127 - ex + 1023;
-    const double sd = __hiloint2double((int)((hi & 0x80000000u) | ((unsigned)re << 20) | ((rb & 0x7fffffu) >> 3)),
-                                       (int)(rb << 29));
-    const double e = fma(-x, sd, 1.0);
-    return fma(sd, fma(e, e, e), sd);
-}
-
 // The best candidate of a warp in every lane: largest key, ties to the lower row.  Three integer reductions.
 // Returns the lane that holds it.
 __device__ __forceinline__ int lu_warp_best(unsigned long long& k, int& r) {
@@ -203,7 +187,7 @@ __device__ __forceinline__ void lu_panel(const LuArgs& a, int j0, int nbk, int t
         const double* urow = rowb[par][win];
         const bool bad = late || (k == 0ULL) || (k >= 0x7ff0000000000000ULL) || r >= m || r < 0;
         const int p = (late || r >= m || r < 0) ? 0 : r;  // with a zero pivot too: perm stays a permutation
-        const double pinv = bad ? 0.0 : lu_rcp(urow[jj]);
+        const double pinv = bad ? 0.0 : fast_rcp(urow[jj]);
         any_bad = any_bad || bad;
         if (tid == 0) {
             if (p >= r0 && p < r1) fl[p - r0] = lu_flag(j0);

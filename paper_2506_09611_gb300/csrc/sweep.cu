@@ -623,29 +623,6 @@ struct FlipConsts {
     T dflip[2][2], sflip[2];
 };
 
-// x / y for the accept factor.  FP32: the approximate reciprocal of the device and one step of residual
-// correction (q += (x - q y) / y), straight-line code that overlaps the block's update.  FP64: a 22-bit
-// reciprocal of y's leading bits, taken in FP32 from its bit pattern, and one step of Halley's iteration
-// (1/y = s (1 + e + e^2 + ...), e = 1 - s y, error e^3 < 2^-63): four dependent FP64 operations, where each
-// costs about 100 cycles and a full division about 740.  Outside the FP32 exponent range: the division.
-__device__ __forceinline__ float accept_quot(float x, float y) {
-    const float rc = __fdividef(1.0f, y), q = x * rc;
-    return fmaf(fmaf(-q, y, x), rc, q);
-}
-__device__ __forceinline__ double accept_quot(double x, double y) {
-    const unsigned hi = (unsigned)__double2hiint(y), lo = (unsigned)__double2loint(y);
-    const int ex = (int)((hi >> 20) & 0x7ffu) - 1023;
-    if (ex < -100 || ex > 100) return x / y;
-    // y = +-1.m 2^ex: the float 1.m (23 bits), its reciprocal in (0.5, 1], back with exponent -ex
-    const float ym = __uint_as_float(0x3f800000u | ((hi & 0xfffffu) << 3) | (lo >> 29));
-    const unsigned rb = __float_as_uint(__fdividef(1.0f, ym));
-    const int re = (int)((rb >> 23) & 0xffu) - 127 - ex + 1023;
-    const double sd = __hiloint2double((int)((hi & 0x80000000u) | ((unsigned)re << 20) | ((rb & 0x7fffffu) >> 3)),
-                                       (int)(rb << 29));
-    const double e = fma(-y, sd, 1.0);
-    return x * fma(sd, fma(e, e, e), sd);
-}
-
 // Warps and register tile of window_reg_kernel for windows of up to NP sites.  Warp 0 decides, TW tile warps
 // hold the block (RG row groups x 8 column groups of threads per spin, a thread rows rg + RG i and columns
 // cg + 8 j), one warp exports the accepts.  Up to 64 sites warps 4, 8, ... exit at once, so the deciding
@@ -846,7 +823,7 @@ __global__ void __launch_bounds__(WinTile<T, NP>::THREADS) window_reg_kernel(
             const int first = __ffs(ball) - 1, par = m & 1;
             T f0, f1;
             if (sizeof(T) == 4) {  // every lane's factors, under the ballot's latency
-                const T q0 = -accept_quot(e0, r0), q1 = -accept_quot(e1, r1);
+                const T q0 = -fast_quot(e0, r0), q1 = -fast_quot(e1, r1);
                 if (lane == first) {
                     s_a[par] = 32 * j + first;
                     s_f[par][0] = q0;
@@ -860,7 +837,7 @@ __global__ void __launch_bounds__(WinTile<T, NP>::THREADS) window_reg_kernel(
                 block_sync();
                 const T n0 = __shfl_sync(FULL, e0, first), n1 = __shfl_sync(FULL, e1, first);
                 const T d0 = __shfl_sync(FULL, r0, first), d1 = __shfl_sync(FULL, r1, first);
-                const T fq = -accept_quot((lane & 1) ? n1 : n0, (lane & 1) ? d1 : d0);
+                const T fq = -fast_quot((lane & 1) ? n1 : n0, (lane & 1) ? d1 : d0);
                 if (lane < 2) s_f[par][lane] = fq;
                 f0 = __shfl_sync(FULL, fq, 0);
                 f1 = __shfl_sync(FULL, fq, 1);
@@ -1058,7 +1035,7 @@ __global__ void __launch_bounds__(320) window_fb_kernel(const float* __restrict_
             const float db = (xup >> a) & 1u ? fstrip.dflip[s][0] : fstrip.dflip[s][1];
             const float r0 = __shfl_sync(FULL, g[0], a);
             const float rr = 1.f + db * (1.f - r0);
-            const float f = a < nbk ? accept_quot(db, rr) * g[0] : 0.f;
+            const float f = a < nbk ? fast_quot(db, rr) * g[0] : 0.f;
             const float first = g[0] - f * (1.f - r0);
 #pragma unroll
             for (int j = 1; j < NBP; ++j) g[j - 1] = fmaf(f, __shfl_sync(FULL, g[j], a), g[j]);
@@ -1086,7 +1063,7 @@ __global__ void __launch_bounds__(320) window_fb_kernel(const float* __restrict_
                 flip = xp != x;
                 if (flip) {
                     fac = E * sp.sflip[1];  // e^{-2h}: sflip[1] = s(+1)/s(-1) takes the scalar back out
-                    if (xp < 0) fac = accept_quot(1.0, fac);
+                    if (xp < 0) fac = fast_quot(1.0, fac);
                 }
             }
             const unsigned fl = __ballot_sync(FULL, flip);
@@ -1107,7 +1084,7 @@ __global__ void __launch_bounds__(320) window_fb_kernel(const float* __restrict_
                 if ((flips >> a) & 1u) {  // uniform
                     const float dd = (xup >> a) & 1u ? fc.dflip[s][0] : fc.dflip[s][1];
                     const float rr = 1.f + dd * (1.f - __shfl_sync(FULL, g[0], a));
-                    const float phi = accept_quot(dd, rr);
+                    const float phi = fast_quot(dd, rr);
                     if (lane == a) {
                         rl = rr;
                         s_phi[s][q] = phi;
