@@ -15,7 +15,10 @@
 #include <cooperative_groups.h>
 #include <limits.h>
 
+#include <algorithm>
+
 #include "internal.h"
+#include "lu_cluster.h"
 
 namespace afq {
 namespace cg = cooperative_groups;
@@ -439,12 +442,12 @@ __global__ void __launch_bounds__(LS_THREADS) lu_sign_kernel(LuArgs a, int parit
     if ((__syncthreads_count(odd) & 1) && tid == 0) sign_out[wk] = -sign_out[wk];
 }
 
-// Dynamic shared memory of a panel's CTA, and the most of it beside the trailing update's static tiles.
+// Dynamic shared memory of a panel's CTA, the most of it, and the most beside the trailing update's static tiles.
 static size_t lu_panel_smem(int m, int cs) {
     const size_t rpc = (m + cs - 1) / cs;
     return rpc * LU_NBP * sizeof(double) + rpc + 16;
 }
-constexpr size_t LU_STEP_SMEM = 144 * 1024;
+constexpr size_t LU_PANEL_SMEM = 227 * 1024 - 16 * 1024, LU_STEP_SMEM = 144 * 1024;
 
 // mr > 0: with the update of the mr rows unpivoted after the panel before, on the columns right of this one.
 template <int CS>
@@ -452,7 +455,7 @@ static cudaError_t launch_panel(cudaStream_t st, const LuArgs& a, int j0, int nb
     const int rpc = (a.m + CS - 1) / CS;
     const size_t shm = lu_panel_smem(a.m, CS);
     {
-        cudaError_t e = ensure_smem_attr((const void*)lu_panel_kernel<CS>, 227 * 1024 - 16 * 1024);
+        cudaError_t e = ensure_smem_attr((const void*)lu_panel_kernel<CS>, LU_PANEL_SMEM);
         if (e != cudaSuccess) return e;
         if (CS > 8) {
             e = ensure_func_attr((const void*)lu_panel_kernel<CS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -488,17 +491,12 @@ static cudaError_t launch_panel(cudaStream_t st, const LuArgs& a, int j0, int nb
     return cudaLaunchKernelEx(&cfg, kern, a, j0, nbk, tpr, nx, ny);
 }
 
-// Cluster size: enough CTAs per matrix that a panel step's FP64 work per SM stays small, few
-// enough that all nmat clusters of a batch are resident together (about two CTAs per SM).
-// Rows per CTA stay at or below 512 (shared memory); 16-CTA clusters are used only if two of
-// them fit on the device at once (else 8).
-static int lu_big_cluster(const LuArgs& a) {
-    static int big = 0;
-    if (big) return big;
+// Resident 16-CTA clusters of a kernel with shm bytes of dynamic shared memory, -1 if that cannot be told.
+static int lu_resident16(const void* fn, size_t attr_bytes, size_t shm) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(32);
     cfg.blockDim = dim3(256);
-    cfg.dynamicSmemBytes = (size_t)((a.m + 15) / 16) * LU_NBP * sizeof(double) + (a.m + 15) / 16 + 16;
+    cfg.dynamicSmemBytes = shm;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = 16;
@@ -507,21 +505,34 @@ static int lu_big_cluster(const LuArgs& a) {
     cfg.attrs = at;
     cfg.numAttrs = 1;
     int ncl = 0;
-    ensure_func_attr((const void*)lu_panel_kernel<16>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    ensure_smem_attr((const void*)lu_panel_kernel<16>, 227 * 1024 - 16 * 1024);
-    if (cudaOccupancyMaxActiveClusters(&ncl, (void*)lu_panel_kernel<16>, &cfg) == cudaSuccess && ncl >= 2) big = 16;
-    else big = 8;
+    if (ensure_func_attr(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+        ensure_smem_attr(fn, attr_bytes) == cudaSuccess &&
+        cudaOccupancyMaxActiveClusters(&ncl, fn, &cfg) == cudaSuccess)
+        return ncl;
     cudaGetLastError();
-    return big;
+    return -1;
 }
 
+// Cluster size: enough CTAs per matrix that a panel step's FP64 work per SM stays small, few
+// enough that all nmat clusters of a batch are resident together (about two CTAs per SM).
+// Rows per CTA stay at or below 512 (shared memory); 16-CTA clusters are used only if two of
+// them fit on the device at once (else 8), of the panel kernel and of the step kernel with its update tiles.
 static int lu_cluster_size(const LuArgs& a) {
+    static BigClusterCache big;
     int nsm = 152, dev = 0;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     int cs = 1;
     while (cs < 16 && (a.m + cs - 1) / cs > 64 && cs * a.nmat <= nsm) cs *= 2;  // spread rows
     while (cs < 16 && (a.m + cs - 1) / cs > 512) cs *= 2;                              // shared memory
-    if (cs == 16) cs = lu_big_cluster(a);
+    if (cs == 16) {
+        const size_t shm = lu_panel_smem(a.m, 16);
+        const bool fits = big.fits(dev, shm, [&] {
+            const int panel = lu_resident16((const void*)lu_panel_kernel<16>, LU_PANEL_SMEM, shm);
+            if (shm > LU_STEP_SMEM) return panel;  // no look-ahead
+            return std::min(panel, lu_resident16((const void*)lu_step_kernel<16, 64, 64>, LU_STEP_SMEM, shm));
+        });
+        if (!fits) cs = 8;
+    }
     return cs;
 }
 
