@@ -789,6 +789,19 @@ def fp64_gemm_tflops(torch, n=4096, reps=3):
     return tf
 
 
+def lu_flop(m, n):
+    """Floating-point operations of the LU of one real m x n matrix (m >= n) to leading order: the sum over the
+    pivots j of 2 (m - j) (n - j)."""
+    return m * n ** 2 - n ** 3 / 3.0
+
+
+def soc_recompute_flop(Ns, n_e):
+    """Floating-point operations per walker of the spin-coupled recompute's FP64 launches: the realified factor is
+    one 4 Ns x 2 n_e matrix, the realified U_L U_R one 2 n_e x 2 n_e matrix, the solve has 2 Ns columns."""
+    return {"elim": lu_flop(4 * Ns, 2 * n_e), "lu_o": lu_flop(2 * n_e, 2 * n_e),
+            "solve": 2.0 * (2 * n_e) ** 2 * 2 * Ns}
+
+
 def kernel_rooflines(prof, gemm, pk, pk_src, steps, wrap="separable", wrap_tile=0):
     """Per-kernel rooflines from the nested per-launch intervals of the timed region:
     achieved = algorithmic work of the launches / their summed CUDA-event durations.
@@ -811,9 +824,9 @@ def kernel_rooflines(prof, gemm, pk, pk_src, steps, wrap="separable", wrap_tile=
               2 * 2.0 * NS ** 2 * N))
     for name, label, flop in (
             ("elim", "lu_panel_kernel + lu_update_kernel (FP64 LU of the propagated N x ns factor, both spins)",
-             2 * (N * NS ** 2 - NS ** 3 / 3.0)),
+             2 * lu_flop(N, NS)),
             ("lu_o", "lu_panel_kernel + lu_update_kernel (FP64 LU of U_L U_R, ns x ns, both spins)",
-             2 * (2.0 / 3.0) * NS ** 3),
+             2 * lu_flop(NS, NS)),
             solve):
         ph = prof.get(name, {"ms": 0.0, "intervals": 0})
         if ph["intervals"] > 0:
@@ -1068,10 +1081,11 @@ def soc_leg(torch, stream, args, seed):
                       "ms_per_launch": dg["ms"] / dg["intervals"], "work_per_launch": OZ_PAIRS * flop64,
                       "fp64_equivalent_tflops": ach64, "fp64_equivalent_vs_fp64_peak": ach64 / fp64,
                       "peak_source": "measured bf16 burst (of %s)" % pk_src})
+    soc_work = soc_recompute_flop(Ns, n_e)
     for name, label, flop in (
-            ("elim", "FP64 LU of the realified 4N x 2N_e factor", 2 * (2 * N2 * nv ** 2 - nv ** 3 / 3.0)),
-            ("lu_o", "FP64 LU of the realified U_L U_R (2N_e x 2N_e)", (2.0 / 3.0) * nv ** 3),
-            ("solve", "FP64 solve with 2N right-hand sides", 2.0 * nv ** 2 * N2)):
+            ("elim", "FP64 LU of the realified 4N x 2N_e factor", soc_work["elim"]),
+            ("lu_o", "FP64 LU of the realified U_L U_R (2N_e x 2N_e)", soc_work["lu_o"]),
+            ("solve", "FP64 solve with 2N right-hand sides", soc_work["solve"])):
         ph = prof[name]
         if ph["intervals"]:
             ach = flop * ph["intervals"] / (ph["ms"] / 1e3) / 1e12
