@@ -43,12 +43,10 @@ __device__ __forceinline__ int8_t lu_flag(int j0) { return (int8_t)min(j0 / LU_N
 __device__ __forceinline__ unsigned long long lu_key(double x) {
     return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffULL;
 }
-__device__ __forceinline__ void lu_pick(unsigned long long& k, int& r, double& x, unsigned long long ok, int orr,
-                                        double ox) {
+__device__ __forceinline__ void lu_pick(unsigned long long& k, int& r, unsigned long long ok, int orr) {
     if (ok > k || (ok == k && orr < r)) {
         k = ok;
         r = orr;
-        x = ox;
     }
 }
 
@@ -149,13 +147,9 @@ __device__ __forceinline__ void lu_panel(const LuArgs& a, int j0, int nbk, int t
     // candidate of column 0 (later columns: found during the previous step's row update)
     unsigned long long bk = 0;
     int br = INT_MAX;
-    double bx = 0.0;
     if (h == 0)
         for (int q = q0; q < nr; q += rows)
-            if (!fl[q]) {
-                const double x = Pn[q * LU_NBP];
-                lu_pick(bk, br, bx, lu_key(x), r0 + q, x);
-            }
+            if (!fl[q]) lu_pick(bk, br, lu_key(Pn[q * LU_NBP]), r0 + q);
     for (int jj = 0; jj < nbk; ++jj) {
         const int par = jj & 1;
         const unsigned bar = lu_smem_u32(&mbar[par]);
@@ -200,7 +194,6 @@ __device__ __forceinline__ void lu_panel(const LuArgs& a, int j0, int nbk, int t
         // candidate for column jj + 1
         bk = 0;
         br = INT_MAX;
-        bx = 0.0;
         const int hj = jj & (tpr - 1), c0 = jj + 1 + ((h - (jj + 1)) & (tpr - 1));
         for (int qb = 0; qb < nr; qb += rows) {
             const int q = qb + q0;
@@ -217,7 +210,7 @@ __device__ __forceinline__ void lu_panel(const LuArgs& a, int j0, int nbk, int t
             if (c < nbk) {
                 const double x = row[c] - l * urow[c];
                 row[c] = x;
-                if (c == jj + 1) lu_pick(bk, br, bx, lu_key(x), r0 + q, x);
+                if (c == jj + 1) lu_pick(bk, br, lu_key(x), r0 + q);
                 c += tpr;
             }
             for (; c + 3 * tpr < nbk; c += 4 * tpr) {
@@ -252,14 +245,13 @@ __global__ void __launch_bounds__(256) lu_panel_kernel(LuArgs a, int j0, int nbk
 // and the columns over the whole GPU).  Grid (16-column blocks, matrix).
 constexpr int LU_UC = 16;
 __global__ void __launch_bounds__(8 * LU_UC) lu_u12_kernel(LuArgs a, int j0, int nbk) {
-    const int mat = blockIdx.y, tid = threadIdx.x, lane = tid & 31, h = tid >> 4, cl = tid & 15;
+    const int mat = blockIdx.y, tid = threadIdx.x, h = tid >> 4, cl = tid & 15;
     double* A = lu_A(a, mat);
     const int* perm = a.perm0 + (long)mat * a.pstride + j0;
     const long lda = a.lda;
     const int c = j0 + nbk + blockIdx.x * LU_UC + cl, cc = min(c, a.n - 1);
     __shared__ double L11[LU_NB][LU_NBP];
     __shared__ double xs[LU_NB][LU_UC];  // finished entries
-    (void)lane;
     for (int e = tid; e < LU_NB * LU_NB; e += 8 * LU_UC) {
         const int k = e / LU_NB, kp = e % LU_NB;
         L11[k][kp] = (k < nbk && kp < k) ? A[(long)perm[k] * lda + j0 + kp] : 0.0;

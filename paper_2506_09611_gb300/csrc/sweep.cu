@@ -520,9 +520,9 @@ static cudaError_t launch_local_reg(cudaStream_t st, float* Gu, float* Gd, int8_
     return cudaLaunchCooperativeKernel((void*)local_reg_kernel<RPT>, dim3(nblk), dim3(LR_THREADS), args, shm, st);
 }
 
-// Grid size of the local kernel: at most max_blocks CTAs (one per SM) and at least one row each.
 size_t local_rowbuf_elems(long ld) { return local_reg_pub(ld); }
 
+// Grid size: at most max_blocks CTAs (one per SM) and at least one row each.
 template <typename T>
 cudaError_t launch_local(cudaStream_t st, T* Gu, T* Gd, int8_t* xl, const double* u, const uint8_t* replay,
                          const SiteParams& sp, SliceOut so, T* colbuf, T* rowbuf, GridBar* bar, int* err,
@@ -573,13 +573,12 @@ __device__ __forceinline__ WindowBufs wb_walker(WindowBufs wb, int j, int N) {
     return wb;
 }
 
-template <typename T>
 static size_t window_smem(int n) {
     size_t P = (size_t)n + 1;
-    size_t g = 2 * (size_t)n * P * sizeof(T);  // Gs[2][n][n+1]
-    size_t s1 = 2 * (size_t)NBMAX * (NBMAX + 1) * sizeof(T);
-    size_t vec = 4 * (size_t)n * sizeof(T) + 2 * (size_t)NBMAX * sizeof(T);  // staging vectors
-    size_t misc = (size_t)n * (sizeof(int) + 1) + 8 * (size_t)NBMAX * sizeof(double) + 256;
+    size_t g = 2 * (size_t)n * P * sizeof(double);  // Gs[2][n][n+1]
+    size_t s1 = 2 * (size_t)NBMAX * (NBMAX + 1) * sizeof(double);
+    size_t vec = 2 * (size_t)n * sizeof(double) + 2 * (size_t)NBMAX * sizeof(double);  // staging vectors
+    size_t misc = (size_t)n * (sizeof(int) + 1) + 2 * (size_t)NBMAX * sizeof(double) + 256;
     return g + s1 + vec + misc;
 }
 
@@ -1164,11 +1163,14 @@ __global__ void __launch_bounds__(320) window_fb_kernel(const float* __restrict_
     }
 }
 
-template <typename T, int MODE>
-__global__ void __launch_bounds__(WIN_THREADS) window_kernel(const T* __restrict__ Gu0, int8_t* xl0, const double* u0,
-                                                             const uint8_t* replay0, SiteParams sp, SliceOut so0,
-                                                             int s0, int n, int nb, WindowBufs wb0, const T* blk0,
-                                                             int* err, Batch bt) {
+// One window of the block force-bias update in FP64 (AFQMC_MODE_BLOCKFB) or of the constrained path's
+// (WIN_MODE_CPB), one block per walker, the window's block of G in shared memory.
+template <int MODE>
+__global__ void __launch_bounds__(WIN_THREADS) window_kernel(const double* __restrict__ Gu0, int8_t* xl0,
+                                                             const double* u0, const uint8_t* replay0, SiteParams sp,
+                                                             SliceOut so0, int s0, int n, int nb, WindowBufs wb0,
+                                                             const double* blk0, int* err, Batch bt) {
+    using T = double;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int P = n + 1;
     const int tid = threadIdx.x, nt = blockDim.x;
@@ -1188,13 +1190,12 @@ __global__ void __launch_bounds__(WIN_THREADS) window_kernel(const T* __restrict
     size_t off = 2 * (size_t)n * P * sizeof(T);
     T* S1 = (T*)(smem_raw + off);  // [2][NBMAX][NBMAX+1]
     off += 2 * (size_t)NBMAX * (NBMAX + 1) * sizeof(T);
-    T* stc = (T*)(smem_raw + off);  // staging: col[2][n], row[2][n]
-    off += 4 * (size_t)n * sizeof(T);
-    T* stb = (T*)(smem_raw + off);  // small staging [2][NBMAX]
+    T* strow = (T*)(smem_raw + off);  // staging: rows [2][n]
+    off += 2 * (size_t)n * sizeof(T);
+    T* stb = (T*)(smem_raw + off);  // columns [2][NBMAX]
     off += 2 * (size_t)NBMAX * sizeof(T);
-    off = (off + 7) & ~(size_t)7;
-    double* fb = (double*)(smem_raw + off);  // block-FB scalars [8][NBMAX]
-    off += 8 * (size_t)NBMAX * sizeof(double);
+    double* fb = (double*)(smem_raw + off);  // scalars [2][NBMAX]
+    off += 2 * (size_t)NBMAX * sizeof(double);
     int* idx = (int*)(smem_raw + off);  // accepted positions [n]
     off += (size_t)n * sizeof(int);
     int8_t* xw = (int8_t*)(smem_raw + off);  // window fields [n]
@@ -1228,15 +1229,11 @@ __global__ void __launch_bounds__(WIN_THREADS) window_kernel(const T* __restrict
             }
     }
     for (int p = tid; p < n; p += nt) xw[p] = xl_g[s0 + p];
-    __shared__ double c_dflip[2][2], c_dstrip[2][2], c_sflip[2];
-    __shared__ T c_dflipT[2][2], c_sflipT[2];  // the same in T for the scan's critical path
+    __shared__ double c_dflip[2][2], c_dstrip[2][2];
     if (tid < 4) {
         c_dflip[tid >> 1][tid & 1] = sp.dflip[tid >> 1][tid & 1];
         c_dstrip[tid >> 1][tid & 1] = sp.dstrip[tid >> 1][tid & 1];
     }
-    if (tid < 2) c_sflip[tid] = sp.sflip[tid];
-    if (tid < 4) c_dflipT[tid >> 1][tid & 1] = (T)sp.dflip[tid >> 1][tid & 1];
-    if (tid < 2) c_sflipT[tid] = (T)sp.sflip[tid];
     if (tid == 0) s_m = 0;
     __syncthreads();
 
@@ -1248,7 +1245,7 @@ __global__ void __launch_bounds__(WIN_THREADS) window_kernel(const T* __restrict
     __syncthreads();
     int n_prop = 0, n_acc = 0, n_flip = 0;
 
-    __shared__ int8_t s_xch[WinCap<float>::NW];  // constrained path: the field chosen at each site
+    __shared__ int8_t s_xch[NWC];                // constrained path: the field chosen at each site
     __shared__ double s_cpl[2];                  // constrained path: sum ln N_i, sum ln |r_up r_dn|
     __shared__ int s_dead;
     if (MODE == WIN_MODE_CPB && tid == 0) {
@@ -1267,7 +1264,6 @@ __global__ void __launch_bounds__(WIN_THREADS) window_kernel(const T* __restrict
         // walker; the fields are then applied as accepts of the delayed update.
         __shared__ T s_phi2[2][NBMAX];
         __shared__ double s_rs2[2];
-        T* strow = stc + 2 * n;  // [2][n]
         for (int p0 = 0; p0 < n && !s_dead; p0 += nb) {
             const int nbk = min(nb, n - p0);
             if (tid < nbk) {
@@ -1301,7 +1297,7 @@ __global__ void __launch_bounds__(WIN_THREADS) window_kernel(const T* __restrict
                 }
                 if (tid < 2) {
                     const int xi = s_xch[mb + q] > 0 ? 0 : 1;
-                    const T dd = c_dflipT[tid][xi];
+                    const T dd = c_dflip[tid][xi];
                     const T rr = T(1) + dd * (T(1) - S1[(tid * NBMAX + q) * (NBMAX + 1) + q]);
                     s_rs2[tid] *= (double)rr;
                     s_phi2[tid][q] = dd / rr;
@@ -1353,7 +1349,6 @@ __global__ void __launch_bounds__(WIN_THREADS) window_kernel(const T* __restrict
         __shared__ double s_rs[2];
         __shared__ int s_accb;
         __shared__ T s_phi[2][NBMAX];
-        T* strow = stc + 2 * n;  // [2][n]
         for (int p0 = 0; p0 < n; p0 += nb) {
             const int nbk = min(nb, n - p0);
             const int blk = (s0 + p0) / nb;
@@ -1373,7 +1368,7 @@ __global__ void __launch_bounds__(WIN_THREADS) window_kernel(const T* __restrict
                 }
                 if (tid < 2) {
                     const int xi = xw[p0 + a] > 0 ? 0 : 1;
-                    const T db = (T)c_dstrip[tid][xi];
+                    const T db = c_dstrip[tid][xi];
                     const T rr = T(1) + db * (T(1) - S1[(tid * NBMAX + a) * (NBMAX + 1) + a]);
                     s_fs[tid] = db / rr;
                 }
@@ -1446,11 +1441,10 @@ __global__ void __launch_bounds__(WIN_THREADS) window_kernel(const T* __restrict
                 }
                 if (tid < 2) {
                     const int xi = xw[p0 + a] > 0 ? 0 : 1;
-                    const T dd = (T)c_dflip[tid][xi];
+                    const T dd = c_dflip[tid][xi];
                     const T rr = T(1) + dd * (T(1) - S1[(tid * NBMAX + a) * (NBMAX + 1) + a]);
                     s_rs[tid] *= (double)rr;
                     s_phi[tid][q] = dd / rr;
-                    fb[(4 + tid) * NBMAX + q] = (double)dd;
                 }
                 __syncthreads();
                 for (int e = tid; e < 2 * nbk * nbk; e += nt) {
@@ -1563,11 +1557,10 @@ cudaError_t launch_window_chain(cudaStream_t st, int mode, const T* Gu, const T*
             return launch_window_reg<T, WIN_MODE_CP, 64>(st, Gu, xl, u, replay, sp, so, s0, n, wb, blk, err, bt);
         }
         if (mode == WIN_MODE_CPB) {
-            cudaError_t e = ensure_smem_attr((const void*)window_kernel<T, WIN_MODE_CPB>,
-                                             window_smem<T>(WinCap<T>::NW));
+            cudaError_t e = ensure_smem_attr((const void*)window_kernel<WIN_MODE_CPB>, window_smem(WinCap<T>::NW));
             if (e != cudaSuccess) return e;
             count_launch();
-            window_kernel<T, WIN_MODE_CPB><<<bt.nwk, WIN_THREADS, window_smem<T>(n), st>>>(
+            window_kernel<WIN_MODE_CPB><<<bt.nwk, WIN_THREADS, window_smem(n), st>>>(
                 Gu, xl, u, replay, sp, so, s0, n, nb, wb, blk, err, bt);
             return cudaGetLastError();
         }
@@ -1589,11 +1582,10 @@ cudaError_t launch_window_chain(cudaStream_t st, int mode, const T* Gu, const T*
             window_fb_kernel<32><<<bt.nwk, 320, 0, st>>>(Gu, xl, u, replay, sp, fc, fs, so, s0, n, nb, wb, blk, err, bt);
         return cudaGetLastError();
     } else {
-        cudaError_t e = ensure_smem_attr((const void*)window_kernel<T, AFQMC_MODE_BLOCKFB>,
-                                         window_smem<T>(WinCap<T>::NW));
+        cudaError_t e = ensure_smem_attr((const void*)window_kernel<AFQMC_MODE_BLOCKFB>, window_smem(WinCap<T>::NW));
         if (e != cudaSuccess) return e;
         count_launch();
-        window_kernel<T, AFQMC_MODE_BLOCKFB><<<bt.nwk, WIN_THREADS, window_smem<T>(n), st>>>(
+        window_kernel<AFQMC_MODE_BLOCKFB><<<bt.nwk, WIN_THREADS, window_smem(n), st>>>(
             Gu, xl, u, replay, sp, so, s0, n, nb, wb, blk, err, bt);
         return cudaGetLastError();
     }
