@@ -179,9 +179,10 @@ int afqmc_debug_wait_timeout(long long limit_ns, void* stream);
  *   delta       2*m doubles, delta[s*m + a] = exp(c_s (x'_a - x_a)) - 1 (spin s = 0 up, 1 down).
  *   m           0 <= m <= 128 (FP32) or 64 (FP64); 0 is a no-op.
  * Work is enqueued on `stream`; device scratch comes from a memory pool of the library's own (it keeps at
- * most 16 MB per device between calls), allocated and freed in that stream's order.  The call then copies the device's status word back and waits for the stream, so it returns
- * after the update.  Returns AFQMC_ERR_ARG for bad sizes or null pointers (checked before any device
- * work) and for a site outside [0, N) (found on the device; G is left unchanged), and
+ * most 32 MB per device between calls), allocated and freed in that stream's order.  The call then copies
+ * the device's status word back and waits for the stream, so it returns after the update.  Returns
+ * AFQMC_ERR_ARG for bad sizes or null pointers (checked before any device work) and for a site outside
+ * [0, N) (found on the device; G is left unchanged), and
  * AFQMC_ERR_NUMERIC when 1 + (1 - G_II) D has a zero pivot for either spin (G is left unchanged). */
 int afqmc_apply_flips(int precision, int N, long long ld, void* G_up, void* G_dn, const int* sites,
                       const double* delta, int m, void* stream);

@@ -243,11 +243,13 @@ static int flips_check(int precision, int N, long long ld, void* G_up, void* G_d
 }
 
 // The scratch of afqmc_apply_flips comes from a memory pool of its own per device that keeps up to
-// FLIPS_POOL_KEEP bytes between calls (what a call on the largest common lattices needs): the device's
-// default pool gives everything back at the call's synchronisation, and mapping the memory again cost
-// about 200 us a call.  Allocation stays ordered on the call's stream, so calls on several streams and threads
-// never share a buffer; anything above the bound goes back at the next synchronisation.
-constexpr uint64_t FLIPS_POOL_KEEP = 16u << 20;
+// FLIPS_POOL_KEEP bytes between calls: the device's default pool gives everything back at the first
+// synchronisation after a call, and mapping the memory again costs about 200 us a call.  A pool grows by blocks
+// of 32 MB (cudaMemPoolAttrReservedMemCurrent) and gives back whole ones, so one block is the least bound that keeps
+// anything (with 16 MB a call between synchronisations took 258 us, with 32 MB 61 us: 8 x 8, FP64, 4 changes); it
+// holds the scratch of any lattice up to 64 x 64.  Allocation stays ordered on the call's stream, so calls on several
+// streams and threads never share a buffer; anything above the bound goes back at the next synchronisation.
+constexpr uint64_t FLIPS_POOL_KEEP = 32u << 20;
 
 static cudaError_t flips_alloc(void** p, size_t bytes, cudaStream_t st) {
     constexpr int MAXDEV = 64;
