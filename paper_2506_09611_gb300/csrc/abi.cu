@@ -128,7 +128,7 @@ struct Walker {
     double* ozs = nullptr;            // row / column scales
     // T form (afqmc_set_form): U_R [nwk][2][N x nsm], U_L [nwk][2][nsm x N], T [nwk][2][nsm x nsm] in
     // the bulk precision; the window gathers U_L[:, I] (nsm x NW) and U_R[I, :] (NW x nsm), the
-    // products V = T U_L[:, I], Y = U_R[I, :] T and Y' = W Y, the rows U_R[J, :] T of the next
+    // products V = T U_L[:, I] and Y = U_R[I, :] T, Y after the accepts' recursion, U_R[J, :] T of the next
     // window (NW x nsm); an FP64 identity (nsm x nsm): T = 1 after every recompute
     void *TUR = nullptr, *TUL = nullptr, *TT = nullptr;
     void *ULI = nullptr, *URI = nullptr, *Vt = nullptr, *Yt = nullptr, *Ypt = nullptr, *Pt = nullptr;
@@ -1279,9 +1279,9 @@ static int sweep_impl(afqmc_ctx* ctx, int gi, int ell, int dir, int mode, int k,
 //   wrap   U_R <- D E U_R, U_L <- U_L E^{-1} D^{-1} (forward; backward the inverse moves after the
 //          update) by the separable passes on the N x Nsigma and Nsigma x N factors; T is unchanged;
 //   per window of sites J: the block 1 - U_R[J, :] T U_L[:, J] of G, the window kernel (the same
-//          decisions, ratios and update matrix W as the G form), then the window's update
-//          T <- T - V W Y with V = T U_L[:, I], Y = U_R[I, :] T (the G form's W by the push-through
-//          identity, Eq. BlkFrcBsTnew2) and the rows I of U_R scaled by the field change
+//          decisions and ratios as the G form), then the window's update T <- T - V W Y with
+//          V = T U_L[:, I], Y = U_R[I, :] T (the G form's W by the push-through identity, Eq.
+//          BlkFrcBsTnew2, as a recursion over the accepts) and the rows I of U_R scaled by the field change
 //          (Eq. UpdateLTRMat).
 // ---- constrained-path AFQMC helpers (Sec. IV.D) ----
 // la[z] = ln |det O_z| of the O = U_L U_R factored by launch_lu (U entries at the pivot rows).
@@ -2095,10 +2095,21 @@ int afqmc_get_G(afqmc_ctx* ctx, int walker, int spin, double* host_out) {
         if (ctx->p.precision == AFQMC_PREC_FP64) CK(tform_form_G<double>(w, ctx->last));
         else CK(tform_form_G<float>(w, ctx->last));
     }
-    // widened and packed on the device, in this matrix's part of the recompute's scratch (rewritten by every
-    // recompute before it is read), then one copy: the host loop over N^2 elements took 5 ms at 40 x 40
     const size_t es = esize(ctx), N = (size_t)w->N, z = (size_t)j * 2 + spin;
     const char* src = (const char*)w->G + z * N * w->ld * es;
+    if (N * w->ld * es <= GET_G_HOST_BYTES) {
+        std::vector<char> buf(N * w->ld * es);
+        CK(cudaStreamSynchronize(ctx->last));
+        CK(cudaMemcpy(buf.data(), src, buf.size(), cudaMemcpyDeviceToHost));
+        for (size_t i = 0; i < N; ++i)
+            for (size_t c = 0; c < N; ++c) {
+                const size_t o = i * w->ld + c;
+                host_out[i * N + c] = es == 8 ? ((const double*)buf.data())[o] : (double)((const float*)buf.data())[o];
+            }
+        return read_dev_err(ctx, w);
+    }
+    // widened and packed on the device, in this matrix's part of the recompute's scratch (rewritten by every
+    // recompute before it is read), then one copy
     double* pk = w->Gnew + z * N * w->ld;
     if (es == 8) CK(launch_to_double<double>(ctx->last, (const double*)src, w->ld, pk, w->N, w->N, w->N));
     else CK(launch_to_double<float>(ctx->last, (const float*)src, w->ld, pk, w->N, w->N, w->N));

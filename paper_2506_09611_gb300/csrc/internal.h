@@ -19,6 +19,10 @@ inline cudaError_t ensure_smem_attr(const void* fn, size_t bytes) {
     return ensure_func_attr(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
+// Largest G that the accessors copy as it is and widen and pack on the host: a launch costs more than the loop
+// there (8 x 8 FP32: 36 us against 44, the same at 100 KB), less beyond (40 x 40 FP32: 1.3 ms against 0.5).
+constexpr size_t GET_G_HOST_BYTES = 100 * 1024;
+
 // Row-major batched GEMM with diagonal scalings (all pointers device):
 //   C[z] = alpha * diag(rs[z]) * A[z] * diag(bs[z]) * B[z] * diag(cs[z]) + beta * C[z]
 // A is M x K (lda), B is K x N (ldb), C is M x N (ldc).  Null scale pointers

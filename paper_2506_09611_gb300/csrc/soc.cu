@@ -2242,11 +2242,22 @@ int afqmc_soc_get_G(afqmc_soc_ctx* ctx, int walker, double* out) {
     int rc = soc_sync_walker(ctx, walker);
     if (rc) return rc;
     if (!out) return AFQMC_ERR_ARG;
+    const int N2 = ctx->N2;
+    const size_t es = ctx->f64 ? 8 : 4, bytes = (size_t)N2 * 2 * ctx->ldz * es;
+    const void* src = (const char*)ctx->G + (size_t)walker * ctx->gstride() * es;
+    if (bytes <= GET_G_HOST_BYTES) {
+        std::vector<char> h(bytes);
+        SCK(cudaMemcpy(h.data(), src, bytes, cudaMemcpyDeviceToHost));
+        auto at = [&](size_t o) { return ctx->f64 ? ((const double*)h.data())[o] : (double)((const float*)h.data())[o]; };
+        for (size_t r = 0; r < (size_t)N2; ++r)
+            for (size_t c = 0; c < (size_t)N2; ++c) {
+                out[(r * N2 + c) * 2] = at(r * 2 * ctx->ldz + c);
+                out[(r * N2 + c) * 2 + 1] = at(r * 2 * ctx->ldz + ctx->ldz + c);
+            }
+        return AFQMC_OK;
+    }
     // interleaved on the device, in the walker's part of the recompute's scratch (rewritten by every
     // recompute before it is read), then one copy
-    const int N2 = ctx->N2;
-    const size_t es = ctx->f64 ? 8 : 4;
-    const void* src = (const char*)ctx->G + (size_t)walker * ctx->gstride() * es;
     double* pk = ctx->Pb + (size_t)walker * 2 * N2 * N2;
     count_launch();
     if (ctx->f64) soc_interleave_kernel<double><<<N2, 256, 0, ctx->last>>>((const double*)src, ctx->ldz, N2, pk);
