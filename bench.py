@@ -913,7 +913,7 @@ def kernel_rooflines(prof, gemm, pk, pk_src, steps, wrap="separable", wrap_tile=
     if fg["intervals"] > 0:
         byts = 2 * 2 * N * N * 4  # read + write of both spins' G (FP32); X and Y' panels are O(N m)
         ach = byts * fg["intervals"] / (fg["ms"] / 1e3) / 1e9
-        out.append({"kernel": "rankm_kernel: the rank-m flush product G -= X Y' (SIMT FP32, both spins)", "bound": "hbm",
+        out.append({"kernel": "rankm_kernel: the rank-m flush product G += X Y (SIMT FP32, both spins)", "bound": "hbm",
                     "achieved": ach, "peak": pk["hbm_gbs"], "unit": "GB/s", "frac": ach / pk["hbm_gbs"],
                     "traffic": NCU_TRAFFIC["flush_gemm"], "launches": fg["intervals"],
                     "ms_per_launch": fg["ms"] / fg["intervals"], "ms_per_step": fg["ms"] / steps,
@@ -1233,7 +1233,7 @@ def tform_leg(afqmc, torch, stream, args, seed):
         return {"value": N * M * 2 / (ms_sweep / 1e3), "unit": UNIT, "ms_per_step": ms_sweep,
                 "phases_ms_per_step": {k: v["ms"] for k, v in prof.items() if v["intervals"]},
                 "note": "T form: the window kernel of the G form on blocks 1 - U_R[J,:] T U_L[:,J]; each window's "
-                        "update T <- T - (T U_L[:,I]) W (U_R[I,:] T) and the rows I of U_R run on the main stream "
+                        "update T <- T + V Y (from T U_L[:,I] and U_R[I,:] T) and the rows I of U_R run on the main stream "
                         "(no pipelined flush yet); the recompute forms T only"}
     finally:
         c.close()
